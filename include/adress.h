@@ -214,10 +214,10 @@ adress_status adress_compute_forces(adress_handle h, double* energies);
  * step count, up to 100 steps per graph): one prologue kernel (half kick, drift,
  * mapping), one fused kernel per further step (forces, thermostat, both half kicks,
  * drift, next mapping), one last kernel (forces, thermostat, second half kick); after each
- * mapping a decide kernel sets the conditional node that runs the list rebuild.  Asynchronous; errors surface at adress_check.
- * With the environment variable ADRESS_EAGER=1 set before adress_init, kernels are
- * launched one by one and the rebuild is decided on the host (synchronising every step);
- * per-kernel profilers cannot see kernels inside graphs that hold conditional nodes. */
+ * mapping a cooperative list kernel decides on a rebuild and, if needed, does it.  Small
+ * systems run all middle steps (between density samples) in one cooperative kernel.
+ * Asynchronous; errors surface at adress_check.  With the environment variable ADRESS_EAGER=1
+ * set before adress_init, the same kernels are launched one by one, without a graph. */
 adress_status adress_step(adress_handle h, int32_t nsteps);
 
 /* One thermodynamic-force iteration block (Sec. "Free energy corrections and the

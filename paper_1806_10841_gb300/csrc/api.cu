@@ -128,6 +128,26 @@ static cudaError_t alloc_pair_buffers(adress_ctx* h) {
   return e;
 }
 
+// Zero the arrival counters of the grid barriers (nothing of the handle may be running): when
+// the grids change, and after a barrier gave up.
+static cudaError_t reset_barriers(adress_ctx* h) {
+  cudaError_t e = cudaMemsetAsync(h->buf.ctrl->bar, 0, sizeof(Ctrl::bar), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(&h->buf.ctrl->arrive, 0, sizeof(Ctrl::arrive), h->stream);
+  return e;
+}
+
+// After a barrier gave up: the barriers, the maxima and the cell counters (a build may have
+// stopped anywhere) as a fresh handle has them; the lists must be built again.
+static cudaError_t revive(adress_ctx* h) {
+  cudaError_t e = reset_barriers(h);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->buf.ctrl->ext_slot, 0, sizeof(Ctrl::ext_slot), h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(h->buf.cell_count, 0, sizeof(unsigned long long) * (size_t)h->sys.ncell, h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(&h->buf.ctrl->dead, 0, sizeof(Ctrl::dead), h->stream);
+  h->lists_built = false;
+  return e;
+}
+
 static void free_graphs(adress_ctx* h) {
   for (auto& kv : h->graphs) {
     if (kv.second.second) cudaGraphExecDestroy(kv.second.second);
@@ -321,28 +341,28 @@ static adress_status setup_cells(adress_ctx* h, double skin) {
   s.ncell = (int)total;
   // energy interpolation: a molecule within r_list of the hybrid layer may pair with a
   // hybrid one (weight (l_a + l_b)/2 > 0), so it is a high-resolution item too
-  for (Box& B : h->boxes) B.d_hr = B.d_at + B.d_hy + (s.scheme == 1 ? r_list : 0.5 * skin);
+  for (Box& B : h->boxes) {
+    B.d_hr = B.d_at + B.d_hy + (s.scheme == 1 ? r_list : 0.5 * skin);
+    B.d_hr_f = (float)(B.d_hr + 1e-3);
+  }
   s.bx = h->boxes[0];
 
   cudaError_t e = cudaSuccess;
   if (s.ncell > h->ncell_cap) {
-    int *cc = b.cell_count, *cf = b.cell_fill, *cs = b.cell_start;
-    if (e == cudaSuccess) e = realloc_owned(h, &cc, s.ncell);
-    if (e == cudaSuccess) e = realloc_owned(h, &cf, s.ncell);
-    if (e == cudaSuccess) e = realloc_owned(h, &cs, s.ncell + 1);
+    if (e == cudaSuccess) e = realloc_owned(h, &b.cell_count, s.ncell);
+    if (e == cudaSuccess) e = realloc_owned(h, &b.cell_start, s.ncell + 1);
+    if (e == cudaSuccess) e = realloc_owned(h, &b.cell_hr, s.ncell + 1);
     if (e == cudaSuccess) e = realloc_owned(h, &h->cell_rank, s.ncell);
     if (e == cudaSuccess && s.nbox > 1) e = realloc_owned(h, &h->cell_box, s.ncell);
     if (e == cudaSuccess) e = realloc_owned(h, &h->buf.dense_cells, s.ncell);
     if (e == cudaSuccess) e = realloc_owned(h, &h->nbr_cells, (size_t)s.ncell * 27);
-    b.cell_count = cc;
-    b.cell_fill = cf;
-    b.cell_start = cs;
     if (e != cudaSuccess) return fail(h, ADRESS_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     h->ncell_cap = s.ncell;
   }
   // the list build expects zero cell counters (it leaves them zero after each build)
-  e = cudaMemsetAsync(b.cell_count, 0, sizeof(int) * (size_t)s.ncell, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b.cell_fill, 0, sizeof(int) * (size_t)s.ncell, h->stream);
+  e = cudaMemsetAsync(b.cell_count, 0, sizeof(unsigned long long) * (size_t)s.ncell, h->stream);
+  // and the grid barriers' arrival counters at a multiple of a grid that may change
+  if (e == cudaSuccess) e = reset_barriers(h);
   if (e != cudaSuccess) return fail(h, ADRESS_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   b.cell_rank = h->cell_rank;
   b.cell_box = h->cell_box;
@@ -464,6 +484,7 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   }
   cudaGetDevice(&h->device);
   Sys& s = h->sys;
+  if (cudaDeviceGetAttribute(&s.n_sm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || s.n_sm < 1) s.n_sm = 152;
   s.nbox = nbox;
   s.M = (int)mtot;
   s.NA = c->atoms_per_mol;
@@ -629,11 +650,9 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
     if (c->n_centers > 0) A(b.kcen[p], M);
   }
   A(b.mcell, M);
-  A(b.sorted, M);
+  A(b.mslot, M);
   A(b.fill_tmp, M);
   A(b.scom, M);
-  A(b.flag, M);
-  A(b.pos, M + 1);
   A(b.items, M);
   A(b.item_of, M);
   A(b.nn, M);
@@ -790,12 +809,13 @@ static adress_status read_ctrl(adress_handle h, Ctrl* c) {
 // Map positions, rebuild lists; grow the capacity and redo while a list overflows.
 static adress_status build_lists_sync(adress_handle h) {
   for (int attempt = 0; attempt < 4; ++attempt) {
-    CUDA_OR_FAIL(h, launch_com(h->sys, h->buf, h->precision, 0, h->stream, DecideArgs{1, 0, 0, 0}));
-    CUDA_OR_FAIL(h, launch_rebuild(h->sys, h->buf, h->stream));
+    CUDA_OR_FAIL(h, launch_map(h->sys, h->buf, h->precision, 0, h->stream));
+    CUDA_OR_FAIL(h, launch_lists(h->sys, h->buf, DecideArgs{1, 0, 1}, h->stream));
     CUDA_OR_FAIL(h, launch_max_nn(h->sys, h->buf, h->stream));
     Ctrl c;
     adress_status st = read_ctrl(h, &c);
     if (st != ADRESS_OK) return st;
+    if (c.dead) CUDA_OR_FAIL(h, revive(h));
     if (c.err == ADRESS_ERR_LIST_OVERFLOW || c.max_nn > h->sys.cap) {
       int cap = ((int)ceil(c.max_nn * 1.5) + 8 + 3) & ~3;
       cap = std::min(cap, h->sys.M - 1);
@@ -846,90 +866,53 @@ adress_status adress_compute_forces(adress_handle h, double* energies) {
   return ADRESS_OK;
 }
 
-// Capture `nsteps` steps into one graph:
-//   prologue (half kick + drift + mapping) -> decide -> IF(rebuild){lists}
-//   { fused step -> decide -> IF(rebuild){lists} } x (nsteps - 1)
+// Launch `nsteps` steps:
+//   prologue (half kick + drift + mapping) -> decision and lists
+//   { fused step -> decision and lists } x (nsteps - 1)
 //   last step (thermostat + second half kick, v and f stored)
-// `decide` sets the conditional of the IF node that follows it.
+// with a density sample after every sample_every-th mapping and the thermodynamic-force
+// update at the end.  The middle runs as one kernel per stretch between samples where that is
+// faster (run_kernel_pays), else as a step and a list kernel per step.
+static cudaError_t launch_steps(adress_handle h, int nsteps, int sample_every, int tf_update, double alpha,
+                                cudaStream_t st) {
+  const Sys& s = h->sys;
+  const Bufs& b = h->buf;
+  const DecideArgs da{0, 1, 1};
+  const bool run = run_kernel_pays(s);
+  cudaError_t e = launch_map(s, b, h->precision, 1, st);
+  if (e == cudaSuccess) e = launch_lists(s, b, da, st);
+  int done = 1;  // mappings so far: positions of time level `done` are current
+  while (e == cudaSuccess) {
+    if (sample_every > 0 && done % sample_every == 0) e = launch_density(s, b, h->precision, st);
+    if (e != cudaSuccess || done >= nsteps) break;
+    if (run) {
+      int m = nsteps - done;
+      if (sample_every > 0) m = std::min(m, sample_every - done % sample_every);
+      e = launch_run(s, b, h->precision, m, st);
+      done += m;
+    } else {
+      if (s.cg_mode) e = mlp_pairs(s, b, h->mlp_args(), b.fpair, st);
+      if (e == cudaSuccess) e = launch_step(s, b, h->precision, 2, 0, st);
+      if (e == cudaSuccess) e = launch_lists(s, b, da, st);
+      ++done;
+    }
+  }
+  if (e == cudaSuccess && s.cg_mode) e = mlp_pairs(s, b, h->mlp_args(), b.fpair, st);
+  if (e == cudaSuccess) e = launch_step(s, b, h->precision, 1, 0, st);
+  if (e == cudaSuccess && tf_update) e = launch_tf_update(s, b, alpha, st);
+  return e;
+}
+
+// The same as one graph.
 static adress_status capture_steps(adress_handle h, int nsteps, int sample_every, int tf_update, double alpha,
                                    cudaGraph_t* gout, cudaGraphExec_t* xout) {
   cudaGraph_t g = nullptr;
-  CUDA_OR_FAIL(h, cudaGraphCreate(&g, 0));
-  std::vector<cudaGraphNode_t> deps;
-  cudaStream_t cs = h->cap_stream;
-  auto grab = [&](std::vector<cudaGraphNode_t>& into) -> cudaError_t {
-    cudaStreamCaptureStatus cst;
-    const cudaGraphNode_t* d = nullptr;
-    size_t nd = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, nullptr, &d, nullptr, &nd);
-    if (e != cudaSuccess) return e;
-    into.assign(d, d + nd);
-    return cudaSuccess;
-  };
-  cudaError_t e = cudaSuccess;
-  for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-    cudaGraphConditionalHandle cond;
-    e = cudaGraphConditionalHandleCreate(&cond, g, 0, 0);
-    if (e != cudaSuccess) break;
-    e = cudaStreamBeginCaptureToGraph(cs, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(),
-                                      cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) break;
-    const DecideArgs da{0, 1, 1, cond};  // the mapping kernel's last block sets the conditional
-    cudaError_t le = cudaSuccess;
-    if (k > 0 && h->sys.cg_mode) le = mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, cs);
-    if (le == cudaSuccess)
-      le = k == 0 ? launch_com(h->sys, h->buf, h->precision, 1, cs, da)
-                  : launch_step(h->sys, h->buf, h->precision, 2, 0, cs, da);
-    std::vector<cudaGraphNode_t> tail;
-    cudaError_t ge = grab(tail);
-    cudaGraph_t gg = g;
-    e = cudaStreamEndCapture(cs, &gg);
-    if (e == cudaSuccess) e = le;
-    if (e == cudaSuccess) e = ge;
-    if (e != cudaSuccess) break;
-
-    cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-    cp.conditional.handle = cond;
-    cp.conditional.type = cudaGraphCondTypeIf;
-    cp.conditional.size = 1;
-    cudaGraphNode_t cnode;
-    e = cudaGraphAddNode(&cnode, g, tail.data(), nullptr, tail.size(), &cp);
-    if (e != cudaSuccess) break;
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) break;
-    le = launch_rebuild(h->sys, h->buf, cs);
-    cudaGraph_t bb = body;
-    e = cudaStreamEndCapture(cs, &bb);
-    if (e == cudaSuccess) e = le;
-    if (e != cudaSuccess) break;
-    deps.assign(1, cnode);
-    // positions of time level k+1 are mapped and current here: sample the profile
-    if (sample_every > 0 && (k + 1) % sample_every == 0) {
-      e = cudaStreamBeginCaptureToGraph(cs, g, deps.data(), nullptr, deps.size(), cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) break;
-      le = launch_density(h->sys, h->buf, h->precision, cs);
-      ge = grab(deps);
-      gg = g;
-      e = cudaStreamEndCapture(cs, &gg);
-      if (e == cudaSuccess) e = le;
-      if (e == cudaSuccess) e = ge;
-    }
-  }
-  if (e == cudaSuccess) {
-    e = cudaStreamBeginCaptureToGraph(cs, g, deps.data(), nullptr, deps.size(), cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      cudaError_t le = cudaSuccess;
-      if (h->sys.cg_mode) le = mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, cs);
-      if (le == cudaSuccess) le = launch_step(h->sys, h->buf, h->precision, 1, 0, cs);
-      if (le == cudaSuccess && tf_update) le = launch_tf_update(h->sys, h->buf, alpha, cs);
-      cudaGraph_t gg = g;
-      e = cudaStreamEndCapture(cs, &gg);
-      if (e == cudaSuccess) e = le;
-    }
-  }
+  CUDA_OR_FAIL(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  const cudaError_t le = launch_steps(h, nsteps, sample_every, tf_update, alpha, h->cap_stream);
+  cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
+  if (le != cudaSuccess) e = le;
   if (e != cudaSuccess) {
-    cudaGraphDestroy(g);
+    if (g) cudaGraphDestroy(g);
     return fail(h, ADRESS_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
   }
   cudaGraphExec_t x = nullptr;
@@ -964,21 +947,7 @@ adress_status adress_run(adress_handle h, int32_t nsteps, int32_t sample_every, 
   if (nsteps < 1 || nsteps > 1000 || sample_every < 0) return fail(h, ADRESS_ERR_ARG, "need 1 <= nsteps <= 1000, sample_every >= 0");
   if (!h->bound || !h->lists_built) return fail(h, ADRESS_ERR_STATE, "bind state and build lists first");
   if (h->eager) {
-    for (int k = 0; k < nsteps; ++k) {
-      const DecideArgs da{0, 1, 0, 0};
-      if (k > 0 && h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
-      if (k == 0) CUDA_OR_FAIL(h, launch_com(h->sys, h->buf, h->precision, 1, h->stream, da));
-      else CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 2, 0, h->stream, da));
-      Ctrl c;
-      adress_status st = read_ctrl(h, &c);
-      if (st != ADRESS_OK) return st;
-      if (c.rebuild) CUDA_OR_FAIL(h, launch_rebuild(h->sys, h->buf, h->stream));
-      if (sample_every > 0 && (k + 1) % sample_every == 0)
-        CUDA_OR_FAIL(h, launch_density(h->sys, h->buf, h->precision, h->stream));
-    }
-    if (h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
-    CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 1, 0, h->stream));
-    if (tf_update) CUDA_OR_FAIL(h, launch_tf_update(h->sys, h->buf, alpha, h->stream));
+    CUDA_OR_FAIL(h, launch_steps(h, nsteps, sample_every, tf_update, alpha, h->stream));
     return ADRESS_OK;
   }
   return launch_graph(h, nsteps, sample_every, tf_update, alpha);
@@ -990,18 +959,7 @@ adress_status adress_step(adress_handle h, int32_t nsteps) {
   if (!h->bound || !h->lists_built) return fail(h, ADRESS_ERR_STATE, "bind state and build lists first");
   if (nsteps == 0) return ADRESS_OK;
   if (h->eager) {
-    for (int k = 0; k < nsteps; ++k) {
-      const DecideArgs da{0, 1, 0, 0};
-      if (k > 0 && h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
-      if (k == 0) CUDA_OR_FAIL(h, launch_com(h->sys, h->buf, h->precision, 1, h->stream, da));
-      else CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 2, 0, h->stream, da));
-      Ctrl c;
-      adress_status st = read_ctrl(h, &c);
-      if (st != ADRESS_OK) return st;
-      if (c.rebuild) CUDA_OR_FAIL(h, launch_rebuild(h->sys, h->buf, h->stream));
-    }
-    if (h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
-    CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 1, 0, h->stream));
+    CUDA_OR_FAIL(h, launch_steps(h, nsteps, 0, 0, 0.0, h->stream));
     return ADRESS_OK;
   }
   int left = nsteps;
@@ -1033,7 +991,8 @@ adress_status adress_get_step(adress_handle h, int64_t* step) {
 adress_status adress_com_lambda(adress_handle h, double* com, double* w) {
   if (!h || !com || !w) return ADRESS_ERR_ARG;
   if (!h->bound) return fail(h, ADRESS_ERR_STATE, "no state bound");
-  CUDA_OR_FAIL(h, launch_com(h->sys, h->buf, h->precision, 0, h->stream, DecideArgs{0, 0, 0, 0}));
+  CUDA_OR_FAIL(h, launch_map(h->sys, h->buf, h->precision, 0, h->stream));
+  CUDA_OR_FAIL(h, launch_lists(h->sys, h->buf, DecideArgs{0, 0, 0}, h->stream));
   CUDA_OR_FAIL(h, launch_export_com(h->sys, h->buf, h->precision, com, w, h->stream));
   return ADRESS_OK;
 }
@@ -1131,7 +1090,8 @@ adress_status adress_kinetic(adress_handle h, double* out) {
 adress_status adress_density_accumulate(adress_handle h) {
   if (!h) return ADRESS_ERR_ARG;
   if (!h->bound) return fail(h, ADRESS_ERR_STATE, "no state bound");
-  CUDA_OR_FAIL(h, launch_com(h->sys, h->buf, h->precision, 0, h->stream, DecideArgs{0, 0, 0, 0}));
+  CUDA_OR_FAIL(h, launch_map(h->sys, h->buf, h->precision, 0, h->stream));
+  CUDA_OR_FAIL(h, launch_lists(h->sys, h->buf, DecideArgs{0, 0, 0}, h->stream));
   CUDA_OR_FAIL(h, launch_density(h->sys, h->buf, h->precision, h->stream));
   return ADRESS_OK;
 }
@@ -1214,12 +1174,12 @@ adress_status adress_time_kernels(adress_handle h, int32_t reps, float* ms_out) 
     if (e == cudaSuccess) e = cudaEventElapsedTime(&t, ev[0], ev[1]);
     acc[which] += t;
   };
-  timed(0, [&] { return launch_com(h->sys, h->buf, h->precision, 1, st, DecideArgs{1, 1, 0, 0}); });
-  timed(1, [&] { return launch_rebuild(h->sys, h->buf, st); });
+  timed(0, [&] { return launch_map(h->sys, h->buf, h->precision, 1, st); });
+  timed(1, [&] { return launch_lists(h->sys, h->buf, DecideArgs{1, 1, 1}, st); });
   for (int r = 0; r < reps && e == cudaSuccess; ++r) {
     if (h->sys.cg_mode && e == cudaSuccess) e = mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, st);
-    timed(2, [&] { return launch_step(h->sys, h->buf, h->precision, 2, 0, st, DecideArgs{1, 1, 0, 0}); });
-    timed(1, [&] { return launch_rebuild(h->sys, h->buf, st); });
+    timed(2, [&] { return launch_step(h->sys, h->buf, h->precision, 2, 0, st); });
+    timed(1, [&] { return launch_lists(h->sys, h->buf, DecideArgs{1, 1, 1}, st); });
   }
   if (h->sys.cg_mode && e == cudaSuccess) e = mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, st);
   timed(3, [&] { return launch_step(h->sys, h->buf, h->precision, 1, 0, st); });
@@ -1244,6 +1204,7 @@ adress_status adress_set_tuning(adress_handle h, int32_t force_block, double ski
     return fail(h, st, "set_tuning: " + h->err);
   }
   h->sys.force_block = force_block;
+  CUDA_OR_FAIL(h, reset_barriers(h));
   free_graphs(h);
   h->lists_built = false;
   return ADRESS_OK;
@@ -1296,6 +1257,8 @@ adress_status adress_autotune(adress_handle h, int32_t nsteps, double* results, 
     return fail(h, ADRESS_ERR_CUDA, std::string("autotune save: ") + cudaGetErrorString(e));
   }
   c0.err = 0;
+  c0.bar[0] = c0.bar[1] = 0;  // the trials change the grids
+  c0.arrive = 0;
   auto restore = [&]() -> cudaError_t {
     cudaError_t r = cudaMemcpyAsync(h->buf.x, x0, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st);
     if (r == cudaSuccess) r = cudaMemcpyAsync(h->buf.v, v0, n3 * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -1493,7 +1456,7 @@ adress_status adress_mlp_collect(adress_handle h, int64_t cap, int64_t* n_total)
     CUDA_OR_FAIL(h, dalloc(h, &h->mlp_offs, M + 1));
   }
   CUDA_OR_FAIL(h, mlp_collect(h->sys, h->buf, 0, nullptr, 0, 0, nullptr, nullptr, nullptr, h->mlp_counts, h->stream));
-  CUDA_OR_FAIL(h, device_exclusive_scan(h->mlp_counts, h->mlp_offs, M, h->buf.scan_tmp, h->mlp_offs + M, h->stream));
+  CUDA_OR_FAIL(h, device_exclusive_scan(h->mlp_counts, h->mlp_offs, M, (int*)h->buf.scan_tmp, h->mlp_offs + M, h->stream));
   int found = 0;
   CUDA_OR_FAIL(h, cudaMemcpyAsync(&found, h->mlp_offs + M, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
@@ -1674,6 +1637,7 @@ adress_status adress_check(adress_handle h) {
   if (st != ADRESS_OK) return st;
   if (c.err != 0) {
     int zero = 0;
+    if (c.dead) CUDA_OR_FAIL(h, revive(h));
     CUDA_OR_FAIL(h, cudaMemcpyAsync(&h->buf.ctrl->err, &zero, sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
     char msg[160];

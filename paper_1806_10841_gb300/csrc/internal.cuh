@@ -22,32 +22,43 @@ constexpr unsigned kMmaWaitPolls = 1u << 22;
 // Slots the mapping kernels' block maxima are spread over (see publish_extent).
 constexpr int kExtSlots = 32;
 
+// Candidates a warp of the list build stages at once.
+constexpr int kMaxCand = 160;
+
+// Poll limit of a grid-wide barrier (each poll is one L2 read): seconds, far beyond the
+// longest phase between two barriers.
+constexpr unsigned kBarrierPolls = 1u << 23;
+
 // Device control block: list-validity trackers, error word, counters.
 struct Ctrl {
-  int rebuild;            // decision for the current step
   int err;                // first device error (adress_status), 0 = none
+  int err_info;
   int n_hr;               // high-resolution work items (first in `items`)
   int n_cg;
   long long step;         // time level of the state's forces
   int rebuilds;
   float ext_now;
   int max_nn;
-  int err_info;
   int parity;          // which half of the double-buffered molecule arrays is current
   int n_dense;         // cells passed to the dense-cell list builder in this build
   int force_rebuild;   // set by the host (moved resolution centres), cleared by a list build
+  int n_netc;  // candidate pairs of the network CG force from the last list build (Bufs::netc)
+  int dead;            // a grid barrier gave up: no list may be built before the host resets
+  unsigned arrive;     // blocks of k_lists or k_run that are done with the control block
+  // arrival counters of the grid barriers of k_lists [0] and k_run [1]: multiples of the
+  // kernel's grid between launches
+  unsigned long long bar[2];
   // float bits of the last mapping's largest squared atom-to-COM distance [0] and largest
   // squared COM displacement since the last build [1], as block maxima spread over
-  // kExtSlots slots (block b uses slot b mod kExtSlots); the decide kernel folds and clears them
-  unsigned ext_slot[2][kExtSlots];
-  int n_netc;  // candidate pairs of the network CG force from the last list build (Bufs::netc)
+  // kExtSlots slots (block b uses slot b mod kExtSlots); the decision folds them.  Set 0,
+  // except inside k_run, which goes round all three so that it can clear one while its blocks
+  // publish to and read from the others; all are zero between launches.
+  unsigned ext_slot[3][2][kExtSlots];
 };
 
-// Arguments of the rebuild decision taken after a mapping (k_decide in observe.cu): force a
-// rebuild, advance the time level, set the graph conditional handle h.
+// What follows a mapping: force a rebuild, advance the time level, whether lists may be built.
 struct DecideArgs {
-  int force, advance, use_h;
-  cudaGraphConditionalHandle h;
+  int force, advance, build;
 };
 
 // Geometry of one periodic box (one replica): edges, fixed-point maps, slab and cells.
@@ -60,6 +71,7 @@ struct Box {
   int fxq[3];
   unsigned xc32;                // slab centre in 32-bit fixed point
   double xc, d_at, d_hy, d_hr;  // d_hr: high-resolution candidate bound at list build
+  float d_hr_f;                 // the FP32 path's: d_hr plus its distances' margin
   double pi_half_over_dhy;
   float d_at_f, d_hyend_f, pi_half_over_dhy_f, near_at, near_hyend;
   int nc[3];
@@ -107,6 +119,7 @@ struct Sys {
   int ncell;  // cells of all boxes
   int cap;  // neighbour-list capacity per molecule
   int force_block;  // threads per block of the mapping and force kernels
+  int n_sm;         // multiprocessors of the handle's device
   int cg_mode;  // 0: tabulated F^CG, 1: learned network (pair forces in Bufs::fpair)
   double dt_m[kMaxNA];  // dt / m (both half kicks of a fused step)
   // water-like model (nb_model 1): site-pair Lennard-Jones c12 = 4 eps sigma^12,
@@ -170,19 +183,17 @@ struct Bufs {
   float4* off32[2];        // (FP32 path)
   // lists
   int* mcell;       // Morton rank of each molecule's cell
-  int* cell_count;  // [ncell]
-  int* cell_fill;   // [ncell]
-  int* cell_start;  // [ncell+1]
-  int* sorted;      // molecules grouped by cell, cells in Morton order, each cell in id order
-  int* fill_tmp;    // [M] cell-grouped molecules in fill (arbitrary) order
-  int4* scom;       // [M] fixed-point centres in `sorted` order (staged by the list build)
-  int* flag;        // [M] high-resolution candidate flag at sorted positions
-  int* pos;         // [M] exclusive scan of flag
+  int* mslot;       // place in its cell's unsorted slice | high-resolution flag in bit 31
+  unsigned long long* cell_count;  // [ncell] molecules (low word), high-resolution ones (high)
+  int* cell_start;  // [ncell+1] first sorted position of a cell (cells in Morton order)
+  int* cell_hr;     // [ncell+1] high-resolution molecules in the cells before
+  int* fill_tmp;    // [M] cell-grouped molecules in fill (arbitrary) order, tagged like mslot
+  int4* scom;       // [M] fixed-point centre + tagged id, cell by cell in id order
   int* items;       // [M] work items: high-resolution candidates first, then CG
   int* item_of;     // [M] work item of each molecule
   int* nn;          // [M] neighbour count per item
   int* nbr;         // [M*cap] neighbour molecule of item t in slot q at nbr[t*cap + q]
-  int* scan_tmp;    // block sums for device-wide scans
+  unsigned long long* scan_tmp;  // block sums for device-wide scans
   const int* cell_rank;  // linear cell -> Morton rank
   // tables
   const double* cgF64;
@@ -275,23 +286,24 @@ struct P32 {
 };
 
 // launchers (one per translation unit)
-cudaError_t launch_com(const Sys& s, const Bufs& b, int precision, int integrate, cudaStream_t st,
-                       DecideArgs da = DecideArgs{0, 0, 0, 0});
-cudaError_t launch_rebuild(const Sys& s, const Bufs& b, cudaStream_t st);
-// Rebuild decision after a mapping kernel (one thread); also flips the current half of the
-// molecule arrays and, in a graph, sets the conditional of the rebuild node.
-cudaError_t launch_decide(const Sys& s, const Bufs& b, DecideArgs da, cudaStream_t st);
+cudaError_t launch_map(const Sys& s, const Bufs& b, int precision, int integrate, cudaStream_t st);
+// After a mapping kernel: fold its maxima, decide on a rebuild and (da.build) build the lists
+// if needed, make the mapping current (and clear the network's pair count).
+cudaError_t launch_lists(const Sys& s, const Bufs& b, DecideArgs da, cudaStream_t st);
 cudaError_t launch_max_nn(const Sys& s, const Bufs& b, cudaStream_t st);
 // The network force's candidate pairs of the current lists with their mirror slots
-// (Bufs::netc, counted in Ctrl::n_netc, which the caller zeroes); launch_rebuild runs it in
-// CG mode 1.
+// (Bufs::netc, counted in Ctrl::n_netc, which the caller zeroes); a list build adds them
+// itself in CG mode 1.
 cudaError_t launch_net_candidates(const Sys& s, const Bufs& b, cudaStream_t st);
 // out[i] = sum_{j<i} in[j] for i < n, *total = sum of all (n <= 8M)
 cudaError_t device_exclusive_scan(const int* in, int* out, int n, int* tmp, int* total, cudaStream_t st);
 // mode: 0 conservative forces, 1 last step of a run (thermostat + second half kick),
 // 2 fused step (thermostat + both half kicks + drift + next mapping)
-cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st,
-                        DecideArgs da = DecideArgs{0, 0, 0, 0});
+cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
+// nsteps fused steps, each with its rebuild decision and lists, in one cooperative launch.
+cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
+// Whether launch_run is the faster way to advance this system (tabulated CG force only).
+bool run_kernel_pays(const Sys& s);
 
 cudaError_t launch_energy_reduce(const Sys& s, const Bufs& b, int nparts, int nvals, cudaStream_t st);
 cudaError_t launch_kinetic(const Sys& s, const Bufs& b, cudaStream_t st);

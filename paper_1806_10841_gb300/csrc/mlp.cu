@@ -792,109 +792,6 @@ __device__ __forceinline__ void pack_pair_inputs(const float f[9], const float (
     }
 }
 
-// A molecule deep in the atomistic region at the list build: it keeps lambda = 1 until the
-// next build (its centre moves by less than skin/2 before then).  thr = d_at - skin/2 - 1e-3
-// of the molecule's box (as float for the FP32 path, whose distances are floats).
-template <bool F64>
-__device__ __forceinline__ bool deep_atomistic(const Sys& s, const Bufs& b, int cur, int a, double thr, float thr_f) {
-  if (s.lam_uniform_on) return s.lam_uniform >= 1.0;
-  if constexpr (F64)
-    return fabs(b.dxc64[cur][a]) < thr;
-  else
-    return fabsf(b.molf[cur][a].x) < thr_f;
-}
-
-// Candidate pairs of the network force, built with the lists: every
-// listed slot (t, q) whose molecule pair a = items[t] < m is within rc_cg + skin and is not
-// made of two deep-atomistic molecules.  Until the next build every pair that needs the
-// network (weight below 1, centres within rc_cg) is among them: the centres move by less
-// than skin/2 each, and a pair of deep-atomistic molecules keeps weight 1.  Records (slot,
-// mirror slot, a, m); four lanes per work item, one atomic per warp (the order varies between
-// runs, the set does not).
-template <bool F64>
-__global__ void __launch_bounds__(128) k_net_candidates(const __grid_constant__ Sys s, Bufs b) {
-  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, g = threadIdx.x & 3;
-  const int lane = threadIdx.x & 31;
-  const bool live = t < s.M;
-  const int cur = b.ctrl->parity;
-  const int a = live ? b.items[t] : 0;
-  const int n = live ? b.nn[t] : 0;
-  const Box& X = box_of(s, b, a);
-  // the threshold once per thread (neighbours share the box of the work item); the FP32
-  // path forms it from float parameters (skin = sqrt(r_cg_list2) - rc_cg), off the FP64 pipe
-  const double thr = F64 ? X.d_at - 0.5 * s.skin - 1e-3 : 0.0;
-  const float thr_f = X.d_at_f - 0.5f * (sqrtf(s.f.r_cg_list2) - sqrtf(s.f.rc_cg2)) - 1e-3f;
-  const bool deep_a = live && deep_atomistic<F64>(s, b, cur, a, thr, thr_f);
-  const int* row = b.nbr + (size_t)t * s.cap;
-  auto candidate = [&](int m) -> bool {
-    if (m <= a || (deep_a && deep_atomistic<F64>(s, b, cur, m, thr, thr_f))) return false;
-    if constexpr (F64) {
-      const double4_32a A = b.com64[cur][a], B = b.com64[cur][m];
-      return pair_r2(minimg_cmp(A.x - B.x, X.L[0], X.halfL[0]), minimg_cmp(A.y - B.y, X.L[1], X.halfL[1]),
-                     minimg_cmp(A.z - B.z, X.L[2], X.halfL[2])) < s.r_cg_list2;
-    } else {
-      const int4 A = b.com_fx[cur][a], B = b.com_fx[cur][m];
-      return pair_r2((float)(int)((unsigned)A.x - (unsigned)B.x) * X.fx_scale[0],
-                     (float)(int)((unsigned)A.y - (unsigned)B.y) * X.fx_scale[1],
-                     (float)(int)((unsigned)A.z - (unsigned)B.z) * X.fx_scale[2]) < s.f.r_cg_list2;
-    }
-  };
-  unsigned long long sel = 0ull;
-  int cnt = 0;
-  for (int q = g, j = 0; q < n; q += 4, ++j)
-    if (candidate(row[q])) {
-      ++cnt;
-      if (j < 64) sel |= 1ull << j;
-    }
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  int base = 0;
-  if (lane == 31 && incl > 0) base = atomicAdd(&b.ctrl->n_netc, incl);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  long long p = (long long)base + (incl - cnt);
-  if (cnt == 0) return;
-  int qx = g + 256;  // where the search for candidates beyond the mask resumes
-  for (int left = cnt; left > 0; --left) {
-    int q;
-    if (sel) {
-      q = g + 4 * (__ffsll((long long)sel) - 1);
-      sel &= sel - 1;
-    } else {
-      for (q = qx; q < n; q += 4)
-        if (candidate(row[q])) break;
-      if (q >= n) return;  // not reached: the first walk counted this slot
-      qx = q + 4;
-    }
-    if (p >= b.ncap) {  // not reached: at most one record per unordered listed pair
-      set_error(b.ctrl, ADRESS_ERR_LIST_OVERFLOW, (int)p);
-      return;
-    }
-    // the mirror slot: where a sits in m's list (the lists are symmetric)
-    const int m = row[q], tb = b.item_of[m], nb = b.nn[tb];
-    const int* rb = b.nbr + (size_t)tb * s.cap;
-    int found = -1;
-    for (int qq = 0; qq < nb; ++qq)
-      if (rb[qq] == a) {
-        found = qq;
-        break;
-      }
-    if (found < 0) set_error(b.ctrl, ADRESS_ERR_STATE, a);
-    b.netc[p] = make_int4(t * s.cap + q, found < 0 ? -1 : tb * s.cap + found, a, m);
-    ++p;
-  }
-}
-
-cudaError_t launch_net_candidates(const Sys& s, const Bufs& b, cudaStream_t st) {
-  const int blocks = ceil_div((long long)s.M * 4, 128);
-  if (s.fp64) k_net_candidates<true><<<blocks, 128, 0, st>>>(s, b);
-  else k_net_candidates<false><<<blocks, 128, 0, st>>>(s, b);
-  return cudaGetLastError();
-}
-
 // Pairs that need the network this step, from the candidates of the last build: the force
 // kernel's test (centres within rc_cg, weight below 1) in its own precision and arithmetic,
 // then the pair's features, normalised bf16 inputs of both orderings and its two list slots
@@ -1199,8 +1096,8 @@ cudaError_t mlp_collect(const Sys& s, const Bufs& b, int pass, const int* offs, 
 
 cudaError_t mlp_pairs(const Sys& s, const Bufs& b, const MlpDevArgs& a, float* fpair, cudaStream_t st) {
   const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
-  cudaError_t e = cudaMemsetAsync(b.npair, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
+  // the pair count is zero here: cleared with the mapping (k_lists)
+  cudaError_t e;
   // persistent grid for the candidates (their count is on the device): 22 blocks per SM,
   // about two waves of the 10 that the kernel's 48 registers let reside (11, 16, 20, 33 and
   // 44 blocks per SM measured slower at 800k atoms)

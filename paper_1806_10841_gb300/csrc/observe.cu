@@ -1,5 +1,4 @@
-// Control and observables: the list-rebuild decision (which also flips the current half of
-// the double-buffered molecule arrays), deterministic FP64 reductions, the COM density
+// Observables: deterministic FP64 reductions, the COM density
 // profile and the thermodynamic-force iteration, and the FP64 export of centres of mass.
 #include <math.h>
 
@@ -8,50 +7,6 @@
 #include "internal.cuh"
 
 namespace adress {
-
-// Rebuild decision after a mapping: rebuild when a centre moved more than skin/2 since the
-// last build (it could have changed class or found a new partner), when the widest
-// molecule makes max(rc_cg, rc_at + 2 ext) + 2 disp exceed the list cutoff, or when the
-// host asked for it (the resolution region moved).  The mapping
-// just written becomes current; the maxima are reset for the next mapping.
-__global__ void k_decide(const __grid_constant__ Sys s, Bufs b, DecideArgs da) {
-  static_assert(kExtSlots == 32, "one slot per lane");
-  // launched as a programmatic dependent of the mapping kernel: its launch overlaps the
-  // mapping's last blocks, and this wait returns once that grid has completed and its
-  // writes are visible
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  Ctrl* c = b.ctrl;
-  const int l = threadIdx.x;
-  const unsigned me = __reduce_max_sync(0xffffffffu, c->ext_slot[0][l]);
-  const unsigned mdd = __reduce_max_sync(0xffffffffu, c->ext_slot[1][l]);
-  c->ext_slot[0][l] = 0u;
-  c->ext_slot[1][l] = 0u;
-  if (l != 0) return;
-  const float e = sqrtf(__uint_as_float(me));
-  const float md = sqrtf(__uint_as_float(mdd));
-  const double cut = fmax(s.rc_cg, s.rc_at + 2.0 * (double)e);
-  const int rb = da.force || c->force_rebuild || (md > 0.5 * s.skin) || (cut + 2.0 * md > s.r_list);
-  if (cut > s.r_list) set_error(c, ADRESS_ERR_EXTENT, (int)(e * 1000));
-  c->rebuild = rb;
-  c->ext_now = e;
-  if (rb) c->rebuilds += 1;
-  if (da.advance) c->step += 1;
-  c->parity ^= 1;
-  if (da.use_h) cudaGraphSetConditional(da.h, (unsigned int)rb);
-}
-
-cudaError_t launch_decide(const Sys& s, const Bufs& b, DecideArgs da, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(1);
-  cfg.blockDim = dim3(32);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_decide, s, b, da);
-}
 
 // ---- deterministic FP64 reductions: per-block partials, then one fixed-order block ----
 

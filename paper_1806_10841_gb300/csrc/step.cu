@@ -7,6 +7,8 @@ namespace adress {
 
 cudaError_t launch_step_ljrf(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
 cudaError_t launch_step_hadress(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
+cudaError_t launch_run_ljrf(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
+cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
 
 template <class P, int NA>
 static void launch_prologue_na(const Sys& s, const Bufs& b, int integrate, cudaStream_t st) {
@@ -30,11 +32,10 @@ static void launch_prologue_p(const Sys& s, const Bufs& b, int integrate, cudaSt
   }
 }
 
-cudaError_t launch_com(const Sys& s, const Bufs& b, int precision, int integrate, cudaStream_t st, DecideArgs da) {
+cudaError_t launch_map(const Sys& s, const Bufs& b, int precision, int integrate, cudaStream_t st) {
   if (precision == ADRESS_FP64) launch_prologue_p<P64>(s, b, integrate, st);
   else launch_prologue_p<P32>(s, b, integrate, st);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? launch_decide(s, b, da, st) : e;
+  return cudaGetLastError();
 }
 
 template <class P>
@@ -47,19 +48,35 @@ static void launch_step_p(const Sys& s, const Bufs& b, int mode, int energy, cud
   }
 }
 
-cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st,
-                        DecideArgs da) {
-  cudaError_t e;
-  if (s.scheme == 1) {
-    e = launch_step_hadress(s, b, precision, mode, energy, st);
-  } else if (s.nb_model == 1) {
-    e = launch_step_ljrf(s, b, precision, mode, energy, st);
-  } else {
-    if (precision == ADRESS_FP64) launch_step_p<P64>(s, b, mode, energy, st);
-    else launch_step_p<P32>(s, b, mode, energy, st);
-    e = cudaGetLastError();
+cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st) {
+  if (s.scheme == 1) return launch_step_hadress(s, b, precision, mode, energy, st);
+  if (s.nb_model == 1) return launch_step_ljrf(s, b, precision, mode, energy, st);
+  if (precision == ADRESS_FP64) launch_step_p<P64>(s, b, mode, energy, st);
+  else launch_step_p<P32>(s, b, mode, energy, st);
+  return cudaGetLastError();
+}
+
+template <class P>
+static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
+  switch (s.NA) {
+    case 1: return launch_run_na<P, 1, 0, false>(s, b, nsteps, st);
+    case 2: return launch_run_na<P, 2, 0, false>(s, b, nsteps, st);
+    case 3: return launch_run_na<P, 3, 0, false>(s, b, nsteps, st);
+    default: return launch_run_na<P, 4, 0, false>(s, b, nsteps, st);
   }
-  return (e == cudaSuccess && mode == MODE_FUSED) ? launch_decide(s, b, da, st) : e;
+}
+
+// The run kernel where one tile per SM covers the system: there a step is latency, and a grid
+// barrier costs less than two launches (1000 molecules: 16.9 us a step in it, 18.7 as
+// launches); at 33,333 molecules launches are the faster way (22.9 against 25.2 us).
+bool run_kernel_pays(const Sys& s) {
+  return !s.cg_mode && ceil_div((long long)s.M * step_lanes(s), s.force_block) <= s.n_sm;
+}
+
+cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
+  if (s.scheme == 1) return launch_run_hadress(s, b, precision, nsteps, st);
+  if (s.nb_model == 1) return launch_run_ljrf(s, b, precision, nsteps, st);
+  return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, nsteps, st) : launch_run_p<P32>(s, b, nsteps, st);
 }
 
 }  // namespace adress

@@ -24,7 +24,10 @@
 #pragma once
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.cuh"
+#include "lists_impl.cuh"
 
 namespace adress {
 
@@ -413,7 +416,7 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
 // fence, no returned value, so blocks retire at once) into slot blockIdx mod kExtSlots:
 // spread over 32 slots the blocks' atomics rarely meet at one address (one address for
 // all blocks cost ~2 us of the fused step at 800k atoms); the decide kernel folds them.
-__device__ __forceinline__ void publish_extent(const Bufs& b, float ext2, float disp2) {
+__device__ __forceinline__ void publish_extent(const Bufs& b, int set, float ext2, float disp2) {
   __shared__ unsigned red[2][kMaxForceBlock / 32];
   const unsigned e = __reduce_max_sync(0xffffffffu, __float_as_uint(ext2));
   const unsigned dm = __reduce_max_sync(0xffffffffu, __float_as_uint(disp2));
@@ -430,20 +433,15 @@ __device__ __forceinline__ void publish_extent(const Bufs& b, float ext2, float 
       me = max(me, red[0][k]);
       md = max(md, red[1][k]);
     }
-    atomicMax(&b.ctrl->ext_slot[0][blockIdx.x & (kExtSlots - 1)], me);
-    atomicMax(&b.ctrl->ext_slot[1][blockIdx.x & (kExtSlots - 1)], md);
+    atomicMax(&b.ctrl->ext_slot[set][0][blockIdx.x & (kExtSlots - 1)], me);
+    atomicMax(&b.ctrl->ext_slot[set][1][blockIdx.x & (kExtSlots - 1)], md);
   }
 }
 
 // ---------------- k_map / k_prologue ---------------------------------------------------
 
-// The decide kernel that follows a mapping kernel may be scheduled once every block of the
-// mapping has started (it waits for the mapping grid's completion itself).
-__device__ __forceinline__ void allow_dependent_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
-
 template <class P, int NA, bool INTEGRATE, bool MULTI>
 __global__ void __launch_bounds__(kMaxForceBlock) k_prologue(const __grid_constant__ Sys s, Bufs b) {
-  allow_dependent_launch();
   const int lane = threadIdx.x & 31, g = threadIdx.x & 3, base = lane & ~3;
   const unsigned gmask = 0xFu << base;
   const int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 2;
@@ -474,7 +472,7 @@ __global__ void __launch_bounds__(kMaxForceBlock) k_prologue(const __grid_consta
   float ext2 = 0.f, disp2 = 0.f;
   if (P::fp64) map_group64<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
   else map_group32<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
-  publish_extent(b, ext2, disp2);
+  publish_extent(b, 0, ext2, disp2);
 }
 
 // ---------------- k_step ----------------------------------------------------------------
@@ -489,18 +487,21 @@ constexpr int step_min_blocks() {
   return P::fp64 ? 1 : (MODEL == 0 && !MULTI ? 10 : 8);
 }
 
+// The step of the molecules of one tile of the grid (a block's worth of threads): thread gtid
+// of the whole grid.  cur: current half of the molecule arrays; step: the time level of the
+// forces; ext_now: the largest atom-to-COM distance; the next mapping's maxima are merged into
+// ext2 and disp2 (MODE_FUSED).  Every thread of a block calls.
 template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS>
-__global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULTI>()) k_step(const __grid_constant__ Sys s, Bufs b) {
+__device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int gtid, const int cur,
+                                          const long long step, const float ext_now, float& ext2, float& disp2) {
   using Q = Prec<P>;
   using real = typename Q::real;
-  if (MODE == MODE_FUSED) allow_dependent_launch();
   const int lane = threadIdx.x & 31, g = threadIdx.x & 3, base = lane & ~3;
   const unsigned gmask = 0xFu << base;
   // SPLIT > 1 (water): a high-resolution item takes SPLIT groups of four lanes in the same
   // warp, group `sub` every SPLIT-th neighbour from slot `sub`; CG items keep one group.
   constexpr int SPLIT = MODEL == 1 ? kSplitWater : 1;
   static_assert(SPLIT == 1 || SPLIT == 2 || SPLIT == 4, "lane groups per item");
-  const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
   int t = gtid >> 2, sub = 0;
   if (SPLIT > 1) {
     const int n_hr0 = b.ctrl->n_hr;
@@ -515,7 +516,6 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
   const bool live = live_item && sub == 0;  // the group that integrates and maps the molecule
   const bool own = live && g < NA;
   const bool own_pair = live_item && g < NA;  // lanes that evaluate pair forces
-  const int cur = b.ctrl->parity;
   // the first list slot this lane reads is fetched together with the item, before the count
   // is known (slots below the capacity lie inside the list array; the value is used only
   // when the count covers the slot)
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
   const real eps = par<real>(s.eps, s.f.eps), sig2 = par<real>(s.sig2, s.f.sig2);
   const real rc_at2 = par<real>(s.rc_at2, s.f.rc_at2), rc_cg2 = par<real>(s.rc_cg2, s.f.rc_cg2);
   const real inv_dr = par<real>(s.cg_inv_dr, s.f.cg_inv_dr);
-  const real reach = par<real>(s.rc_at, s.f.rc_at) + (real)2 * (real)b.ctrl->ext_now;
+  const real reach = par<real>(s.rc_at, s.f.rc_at) + (real)2 * (real)ext_now;
   const real reach_at2 = reach * reach;
   const int gg0 = g < NA ? g : 0;
   const real frac_g = par<real>(s.frac[gg0], s.f.frac[gg0]);
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
   real dv = 0;
   // slow-force weight at this time level (1 without multiple time stepping)
   real sw = 1;
-  if (s.respa_n > 1) sw = b.ctrl->step % s.respa_n == 0 ? (real)s.respa_n : (real)0;
+  if (s.respa_n > 1) sw = step % s.respa_n == 0 ? (real)s.respa_n : (real)0;
   const bool slow = sw != (real)0 || ENERGY;
 
   if (hr_item) {
@@ -900,7 +900,6 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
     double x[3] = {0.0, 0.0, 0.0};
     if (own) {
       // Langevin force with the half-step velocity, noise keyed by (seed, time level n)
-      const long long step = b.ctrl->step;
       const unsigned ia = (unsigned)(i - B.mol0 * NA);  // atom index within its replica
       unsigned c[4] = {ia, (unsigned)step, (unsigned)((unsigned long long)step >> 32), (unsigned)(2 * B.replica)};
       philox4x32_10(c, s.seed_lo, s.seed_hi);
@@ -971,11 +970,11 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
         const double x0 = P::fp64 ? shfl_d(gmask, x[d], base) : shfl_d(gmask, x[d], base);
         if (!own) x[d] = x0;
       }
-      float ext2 = 0.f, disp2 = 0.f;
       const int nxt = cur ^ 1;
-      if (P::fp64) map_group64<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
-      else map_group32<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
-      publish_extent(b, ext2, disp2);
+      float d2 = 0.f;
+      if (P::fp64) map_group64<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, d2);
+      else map_group32<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, d2);
+      disp2 = fmaxf(disp2, d2);
     }
   }
 
@@ -988,11 +987,78 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
       vir += __shfl_xor_sync(0xffffffffu, vir, o);
     }
     if (lane == 0) {
-      const size_t wid = (size_t)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+      const size_t wid = (size_t)gtid >> 5;
       b.part[wid * 4 + 0] = e_at;
       b.part[wid * 4 + 1] = e_cg;
       b.part[wid * 4 + 2] = e_b;
       b.part[wid * 4 + 3] = vir;
+    }
+  }
+}
+
+template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS>
+__global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULTI>()) k_step(const __grid_constant__ Sys s, Bufs b) {
+  const Ctrl* c = b.ctrl;
+  float ext2 = 0.f, disp2 = 0.f;
+  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS>(s, b, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
+                                                   c->ext_now, ext2, disp2);
+  if (MODE == MODE_FUSED) publish_extent(b, 0, ext2, disp2);
+}
+
+// ---------------- k_run ------------------------------------------------------------------
+
+// Resident blocks per SM of the run kernel (its registers: 64 a thread).
+template <class P>
+constexpr int run_min_blocks() {
+  return P::fp64 ? 3 : 8;
+}
+
+// nsteps fused steps in one cooperative launch: every block takes its tiles of the step, a
+// grid barrier ends the mapping, every block takes the rebuild decision itself and the grid
+// rebuilds the lists when needed.  For small systems (run_kernel_pays).
+template <class P, int NA, bool MULTI, int MODEL, bool HS>
+__global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, int nsteps) {
+  Ctrl* c = b.ctrl;
+  if (grid_is_dead(c)) return;
+  int cur = c->parity, set = 0, dirty = 0, rebuilt = 0;
+  long long step = c->step;
+  float ext_now = c->ext_now;
+  const int ntiles = (int)(((long long)s.M * (MODEL == 1 ? kSplitWater * kGroup : kGroup) + blockDim.x - 1) / blockDim.x);
+  GridBarrier bar(c, &c->bar[1]);
+  for (int k = 0; k < nsteps; ++k) {
+    float ext2 = 0.f, disp2 = 0.f;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS>(s, b, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
+                                                            ext2, disp2);
+    publish_extent(b, set, ext2, disp2);
+    if (!bar.sync()) return;
+    const Decision d = decide_rebuild(s, c, set, 0);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+      // the set of the previous step: every block has read it, and the step after the next
+      // publishes to it
+      c->ext_slot[(set + 2) % 3][0][threadIdx.x] = 0u;
+      c->ext_slot[(set + 2) % 3][1][threadIdx.x] = 0u;
+      if (threadIdx.x == 0 && d.too_wide) set_error(c, ADRESS_ERR_EXTENT, (int)(d.ext * 1000));
+    }
+    cur ^= 1;
+    ++step;
+    dirty = set;
+    set = (set + 1) % 3;
+    ext_now = d.ext;
+    if (d.rebuild) {
+      ++rebuilt;
+      if (!rebuild_lists<kMaxForceBlock / 32>(s, b, cur, bar)) return;
+      if (!bar.sync()) return;
+    }
+  }
+  if (threadIdx.x < 32 && last_to_arrive(c)) {
+    c->ext_slot[dirty][0][threadIdx.x] = 0u;
+    c->ext_slot[dirty][1][threadIdx.x] = 0u;
+    if (threadIdx.x == 0) {
+      c->parity = cur;
+      c->step = step;
+      c->ext_now = ext_now;
+      c->rebuilds += rebuilt;
     }
   }
 }
@@ -1022,6 +1088,23 @@ static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cu
       else k_step<P, NA, MODE_FUSED, false, false, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
       break;
   }
+}
+
+// As many blocks as fit on the device at once, at most one per tile.
+template <class P, int NA, int MODEL, bool HS>
+static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
+  const int tiles = ceil_div((long long)s.M * step_lanes(s), s.force_block);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(std::min(tiles, s.n_sm * run_min_blocks<P>()));
+  cfg.blockDim = dim3(s.force_block);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (s.nbox > 1) return cudaLaunchKernelEx(&cfg, k_run<P, NA, true, MODEL, HS>, s, b, nsteps);
+  return cudaLaunchKernelEx(&cfg, k_run<P, NA, false, MODEL, HS>, s, b, nsteps);
 }
 
 }  // namespace adress
