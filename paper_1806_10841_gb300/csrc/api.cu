@@ -490,6 +490,15 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   s.NA = c->atoms_per_mol;
   s.N = s.M * s.NA;
   s.force_block = 128;
+  {
+    // More lanes per molecule where molecules are few per SM (us a step; water-like fluid, lanes
+    // of high-resolution / coarse-grained items 32/8, 16/8, 8/8, 8/4: 6,000 molecules 44, 54, 73,
+    // 79; 16,000: 74, 69, 80, -; 32,000: 94, 87, 82, -; 64,000: 170, 154, 147, 138; run kernel,
+    // 16/8 and 4/4: 4,000 molecules 11.1, 12.6; 12,000: 17.1, 13.8).
+    const long long per_sm = (mtot + s.n_sm - 1) / s.n_sm;
+    s.step_lanes = per_sm <= 64 ? Lanes{5, 3} : per_sm <= 160 ? Lanes{4, 3} : per_sm <= 320 ? Lanes{3, 3} : Lanes{3, 2};
+    s.run_lanes = per_sm <= 40 ? Lanes{4, 3} : Lanes{2, 2};
+  }
   double Mtot = 0;
   for (int k = 0; k < s.NA; ++k) Mtot += c->mass[k];
   s.Mtot = Mtot;
@@ -573,7 +582,10 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
         const double ir6 = 1.0 / (rc * rc * rc * rc * rc * rc);
         s.vsh[i][j] = -(s.c12[i][j] * ir6 - s.c6[i][j]) * ir6;
         s.qq[i][j] = c->coulomb_f * c->charge[i] * c->charge[j];
-        if (s.c12[i][j] != 0.0 || s.c6[i][j] != 0.0) s.lj_cols |= 1 << j;
+        if (s.c12[i][j] != 0.0 || s.c6[i][j] != 0.0) {
+          s.lj_cols |= 1 << j;
+          s.lj_pairs |= 1 << (4 * i + j);
+        }
         s.f.c12[i][j] = (float)s.c12[i][j];
         s.f.c6[i][j] = (float)s.c6[i][j];
         s.f.qq[i][j] = (float)s.qq[i][j];
@@ -645,7 +657,7 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
       A(b.off64[p], N);
     } else {
       A(b.molf[p], M);
-      A(b.off32[p], N);
+      A(b.off32[p], (size_t)3 * M);
     }
     if (c->n_centers > 0) A(b.kcen[p], M);
   }

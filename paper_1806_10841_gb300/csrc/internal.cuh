@@ -84,6 +84,11 @@ struct Box {
   long long replica;  // replica id (thermostat noise counter)
 };
 
+// Lanes (log2) a high-resolution and a coarse-grained work item take.
+struct Lanes {
+  int h, c;
+};
+
 // Per-system constants, passed by value to every kernel.
 struct Sys {
   int M, NA, N;
@@ -120,6 +125,7 @@ struct Sys {
   int cap;  // neighbour-list capacity per molecule
   int force_block;  // threads per block of the mapping and force kernels
   int n_sm;         // multiprocessors of the handle's device
+  Lanes step_lanes, run_lanes;  // lanes per work item of the step and run kernels (FP32 path)
   int cg_mode;  // 0: tabulated F^CG, 1: learned network (pair forces in Bufs::fpair)
   double dt_m[kMaxNA];  // dt / m (both half kicks of a fused step)
   // water-like model (nb_model 1): site-pair Lennard-Jones c12 = 4 eps sigma^12,
@@ -128,6 +134,7 @@ struct Sys {
   double c12[kMaxNA][kMaxNA], c6[kMaxNA][kMaxNA], vsh[kMaxNA][kMaxNA], qq[kMaxNA][kMaxNA];
   double krf, crf;
   int lj_cols;  // bit j: some site has a Lennard-Jones term with site j
+  int lj_pairs;  // bit 4 i + j: sites i and j have one
   // bonded: bond_model 0 FENE (+ WCA), 1 harmonic (bond_k, bond_r0); harmonic angles
   int bond_model;
   double bond_k, bond_r0;
@@ -180,7 +187,9 @@ struct Bufs {
   int* kcen[2];            // spheres: index of the nearest centre
   // per atom, double-buffered
   double4_32a* off64[2];   // COM-relative atom offsets (FP64 path)
-  float4* off32[2];        // (FP32 path)
+  float4* off32[2];        // FP32 path: [M][3], the x, y and z components of a molecule's (up to
+                           // four) atoms, so that a molecule's offsets are three 16-byte loads
+                           // and adjacent atoms pair up in packed float2 arithmetic
   // lists
   int* mcell;       // Morton rank of each molecule's cell
   int* mslot;       // place in its cell's unsorted slice | high-resolution flag in bit 31
@@ -342,11 +351,12 @@ adress_status set_global_error(adress_status s, const std::string& msg);
 // registers and ~4% time at 128 threads).
 constexpr int kMaxForceBlock = 128;
 
-// Threads per molecule the force kernel is launched with: four, or eight for the water-like
-// model, whose high-resolution items split their neighbour lists over two lane groups.
-// water-like model: a high-resolution work item takes kSplitWater groups of four lanes
-constexpr int kSplitWater = 2;
-inline int step_lanes(const Sys& s) { return s.nb_model == 1 ? kSplitWater * kGroup : kGroup; }
+// Lanes a high-resolution work item takes where one lane takes an atom.
+constexpr int atom_lanes(bool fp64, int model) { return fp64 && model == 1 ? 2 * kGroup : kGroup; }
+// Threads per molecule the step kernels are launched with.
+inline int step_lanes(const Sys& s) {
+  return !s.fp64 && s.nb_model == 1 ? 1 << s.step_lanes.h : atom_lanes(s.fp64, s.nb_model);
+}
 
 // Warps launched by the force kernel (one energy partial each).
 inline int force_warps(const Sys& s) {

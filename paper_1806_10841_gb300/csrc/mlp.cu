@@ -595,21 +595,35 @@ __device__ __forceinline__ void sort4f(float v[4]) {
   v[3] = hi;
 }
 
-// COM-relative offset of atom i in the current mapping, as float (either path's layout).
-template <bool F64>
-__device__ __forceinline__ float4 offset_f(const Bufs& b, int cur, int i) {
+// COM-relative offsets of molecule a's atoms in the current mapping, as float (either path's
+// layout).
+template <int NA, bool F64>
+__device__ __forceinline__ void offsets_f(const Bufs& b, int cur, int a, float (&x)[4], float (&y)[4], float (&z)[4]) {
   if (F64) {
-    const double4_32a o = b.off64[cur][i];
-    return make_float4((float)o.x, (float)o.y, (float)o.z, 0.f);
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+      const double4_32a o = b.off64[cur][a * NA + k];
+      x[k] = (float)o.x;
+      y[k] = (float)o.y;
+      z[k] = (float)o.z;
+    }
+  } else {
+    const float4* o = b.off32[cur] + 3 * (size_t)a;
+    const float4 X = o[0], Y = o[1], Z = o[2];
+    x[0] = X.x; x[1] = X.y; x[2] = X.z; x[3] = X.w;
+    y[0] = Y.x; y[1] = Y.y; y[2] = Y.z; y[3] = Y.w;
+    z[0] = Z.x; z[1] = Z.y; z[2] = Z.z; z[3] = Z.w;
   }
-  return b.off32[cur][i];
 }
 
 // Features of (a, b) with e from a to b; feat[9].  Atoms beyond na project to 0 (padding).
-// The first molecule's centre A and atom offsets oa[] come from the caller.
 template <int NA, bool F64>
-__device__ __forceinline__ void pair_features32(const Box& X, const int4 A, const float4 (&oa)[NA], const Bufs& b,
-                                                int cur, int bb, float feat[9]) {
+__device__ __forceinline__ void pair_features32(const Sys& s, const Bufs& b, int cur, int a, int bb, float feat[9]) {
+  const Box& X = box_of(s, b, a);
+  const int4 A = b.com_fx[cur][a];
+  float ax[4], ay[4], az[4], bx[4], by[4], bz[4];
+  offsets_f<NA, F64>(b, cur, a, ax, ay, az);
+  offsets_f<NA, F64>(b, cur, bb, bx, by, bz);
   const int4 B = b.com_fx[cur][bb];
   const float ex = (float)(int)((unsigned)B.x - (unsigned)A.x) * X.fx_scale[0];
   const float ey = (float)(int)((unsigned)B.y - (unsigned)A.y) * X.fx_scale[1];
@@ -618,9 +632,8 @@ __device__ __forceinline__ void pair_features32(const Box& X, const int4 A, cons
   float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < NA; ++k) {
-    const float4 ob = offset_f<F64>(b, cur, bb * NA + k);
-    sa[k] = (oa[k].x * ex + oa[k].y * ey + oa[k].z * ez) * id;
-    sb[k] = -(ob.x * ex + ob.y * ey + ob.z * ez) * id;
+    sa[k] = (ax[k] * ex + ay[k] * ey + az[k] * ez) * id;
+    sb[k] = -(bx[k] * ex + by[k] * ey + bz[k] * ez) * id;
   }
   if (NA == 4) {
     sort4f(sa);
@@ -643,14 +656,6 @@ __device__ __forceinline__ void pair_features32(const Box& X, const int4 A, cons
   }
 }
 
-template <int NA, bool F64>
-__device__ __forceinline__ void pair_features32(const Sys& s, const Bufs& b, int cur, int a, int bb, float feat[9]) {
-  float4 oa[NA];
-#pragma unroll
-  for (int k = 0; k < NA; ++k) oa[k] = offset_f<F64>(b, cur, a * NA + k);
-  pair_features32<NA, F64>(box_of(s, b, a), b.com_fx[cur][a], oa, b, cur, bb, feat);
-}
-
 // Atomistic force on a from b projected on -e (the force-matching target), FP32.
 template <int NA, bool F64>
 __device__ __forceinline__ float pair_target32(const Sys& s, const Bufs& b, int cur, int a, int bb) {
@@ -660,13 +665,14 @@ __device__ __forceinline__ float pair_target32(const Sys& s, const Bufs& b, int 
   const float Ry = (float)(int)((unsigned)A.y - (unsigned)B.y) * X.fx_scale[1];
   const float Rz = (float)(int)((unsigned)A.z - (unsigned)B.z) * X.fx_scale[2];
   float Fx = 0.f, Fy = 0.f, Fz = 0.f;
+  float ax[4], ay[4], az[4], bx[4], by[4], bz[4];
+  offsets_f<NA, F64>(b, cur, a, ax, ay, az);
+  offsets_f<NA, F64>(b, cur, bb, bx, by, bz);
 #pragma unroll
   for (int i = 0; i < NA; ++i) {
-    const float4 oi = offset_f<F64>(b, cur, a * NA + i);
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
-      const float4 oj = offset_f<F64>(b, cur, bb * NA + j);
-      const float dx = Rx + oi.x - oj.x, dy = Ry + oi.y - oj.y, dz = Rz + oi.z - oj.z;
+      const float dx = Rx + ax[i] - bx[j], dy = Ry + ay[i] - by[j], dz = Rz + az[i] - bz[j];
       const float d2 = dx * dx + dy * dy + dz * dz;
       if (d2 < s.f.rc_at2) {
         float fr;

@@ -7,7 +7,6 @@ namespace adress {
 
 cudaError_t launch_step_ljrf(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
 cudaError_t launch_step_hadress(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
-cudaError_t launch_run_ljrf(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
 cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
 
 template <class P, int NA>
@@ -66,16 +65,18 @@ static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStr
   }
 }
 
-// The run kernel where one tile per SM covers the system: there a step is latency, and a grid
-// barrier costs less than two launches (1000 molecules: 16.9 us a step in it, 18.7 as
-// launches); at 33,333 molecules launches are the faster way (22.9 against 25.2 us).
+// The run kernel where the device is far from full: there a step is latency, and a grid barrier
+// costs less than two launches (us a step, run kernel against launches, FP32: 1000 molecules 9.4
+// and 17.6; 12,000: 13.8 and 19.5; 25,000: 19.9 and 20.7; 40,000: 25 and 23).  Not for the
+// water-like fluid: its long lists make the step itself longer than the launches (2000
+// molecules: 33 both ways), nor in FP64 beyond one tile per SM (two blocks an SM reside).
 bool run_kernel_pays(const Sys& s) {
-  return !s.cg_mode && ceil_div((long long)s.M * step_lanes(s), s.force_block) <= s.n_sm;
+  return !s.cg_mode && s.nb_model == 0 && s.M <= (s.fp64 ? 32ll : 160ll) * s.n_sm;
 }
 
 cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
   if (s.scheme == 1) return launch_run_hadress(s, b, precision, nsteps, st);
-  if (s.nb_model == 1) return launch_run_ljrf(s, b, precision, nsteps, st);
+  if (s.nb_model == 1) return cudaErrorInvalidValue;
   return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, nsteps, st) : launch_run_p<P32>(s, b, nsteps, st);
 }
 

@@ -28,7 +28,6 @@ cudaError_t launch_step_hadress(const Sys& s, const Bufs& b, int precision, int 
 
 template <class P>
 static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
-  if (s.nb_model == 1) return launch_run_na<P, 3, 1, true>(s, b, nsteps, st);
   switch (s.NA) {
     case 1: return launch_run_na<P, 1, 0, true>(s, b, nsteps, st);
     case 2: return launch_run_na<P, 2, 0, true>(s, b, nsteps, st);
@@ -38,7 +37,6 @@ static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStr
 }
 
 cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
-  if (s.nb_model == 1 && s.NA != 3) return cudaErrorInvalidValue;
   return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, nsteps, st) : launch_run_p<P32>(s, b, nsteps, st);
 }
 

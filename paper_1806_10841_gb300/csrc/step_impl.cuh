@@ -126,7 +126,11 @@ struct Prec<P64> {
     return {minimg_cmp(A.x - B.x, X.L[0], X.halfL[0]), minimg_cmp(A.y - B.y, X.L[1], X.halfL[1]),
             minimg_cmp(A.z - B.z, X.L[2], X.halfL[2])};
   }
-  static __device__ __forceinline__ double4_32a off(const Bufs& b, int cur, int i) { return b.off64[cur][i]; }
+  // offset of atom k of molecule a (NA atoms per molecule)
+  template <int NA>
+  static __device__ __forceinline__ double4_32a off(const Bufs& b, int cur, int a, int k) {
+    return b.off64[cur][a * NA + k];
+  }
   static __device__ __forceinline__ double cg(const Bufs& b, int cg_n, double r, double inv_dr, double* V) {
     const double u = r * inv_dr;
     int k = (int)u;
@@ -159,7 +163,11 @@ struct Prec<P32> {
             (float)(int)((unsigned)A.y - (unsigned)B.y) * X.fx_scale[1],
             (float)(int)((unsigned)A.z - (unsigned)B.z) * X.fx_scale[2]};
   }
-  static __device__ __forceinline__ float4 off(const Bufs& b, int cur, int i) { return b.off32[cur][i]; }
+  template <int NA>
+  static __device__ __forceinline__ V3 off(const Bufs& b, int cur, int a, int k) {
+    const float* o = (const float*)(b.off32[cur] + 3 * (size_t)a) + k;
+    return {o[0], o[4], o[8]};
+  }
   static __device__ __forceinline__ float cg(const Bufs& b, int cg_n, float r, float inv_dr, float* V) {
     const float u = r * inv_dr;
     int k = (int)u;
@@ -310,10 +318,13 @@ __device__ __forceinline__ void map_group32(const Sys& s, const Box& B, const Bu
     o32[d] -= c32;
     R[d] = P0[d] + (unsigned)c32;
   }
-  float4 o = make_float4((float)o32[0] * B.fx_scale[0], (float)o32[1] * B.fx_scale[1],
-                         (float)o32[2] * B.fx_scale[2], 0.f);
+  const float3 o = make_float3((float)o32[0] * B.fx_scale[0], (float)o32[1] * B.fx_scale[1],
+                               (float)o32[2] * B.fx_scale[2]);
   if (own) {
-    b.off32[nxt][a * NA + g] = o;
+    float* of = (float*)(b.off32[nxt] + 3 * (size_t)a) + g;
+    of[0] = o.x;
+    of[4] = o.y;
+    of[8] = o.z;
     ext2 = fmaxf(ext2, o.x * o.x + o.y * o.y + o.z * o.z);
   }
   // signed x distance to the slab centre (spheres: distance to the nearest centre); region
@@ -479,49 +490,342 @@ __global__ void __launch_bounds__(kMaxForceBlock) k_prologue(const __grid_consta
 
 // MODEL 0: WCA between atoms of different molecules (the tetrahedral fluid);
 // MODEL 1: Lennard-Jones + reaction-field Coulomb per site pair (the water-like fluid).
-// Resident blocks per SM the FP32 kernels are compiled for (48 registers for the single-box
-// WCA model: more warps to hide the neighbour-load latency, measured 3% faster than the
-// unbounded 55; the batched and water variants keep 64).
-template <class P, int MODEL, bool MULTI>
+// Resident blocks per SM the FP32 kernels are compiled for: 9 (56 registers) for the WCA model
+// (200,000 molecules: 8 blocks 65.8, 9 blocks 64.1, 10 blocks 66.2 us a step), 8 with energy
+// interpolation, 6 (80 registers) for the water-like model (5: 153, 6: 144, 8: 163 us).
+template <class P, int MODEL, bool MULTI, bool HS>
 constexpr int step_min_blocks() {
-  return P::fp64 ? 1 : (MODEL == 0 && !MULTI ? 10 : 8);
+  return P::fp64 ? 1 : MODEL == 1 ? 6 : HS ? 8 : 9;
+}
+
+// How a step kernel deals out a work item's neighbours (its template parameter FORM): one lane
+// per atom (four lanes an item; FP64 water-like items two such groups); one lane per neighbour
+// with the lanes per item chosen by the host; the same fixed to eight and four lanes.
+constexpr int FORM_ATOM = 0, FORM_NEIGHBOUR = 1, FORM_NEIGHBOUR_8_4 = 2;
+template <int FORM, class P, int MODEL>
+__device__ __forceinline__ Lanes lanes_of(Lanes chosen) {
+  if (FORM == FORM_NEIGHBOUR) return chosen;
+  return FORM == FORM_NEIGHBOUR_8_4 ? Lanes{3, 2} : Lanes{atom_lanes(P::fp64, MODEL) == 8 ? 3 : 2, 2};
+}
+
+// Lanes of this lane's aligned group of G (a power of two).
+__device__ __forceinline__ unsigned lane_group(int G, int lane) { return (0xffffffffu >> (32 - G)) << (lane & ~(G - 1)); }
+
+// WCA force over distance of two atom pairs, 24 eps (2 sr^12 - sr^6) / r^2 w, in the rounding order
+// of the scalar expression.
+__device__ __forceinline__ float2 wca_fr2(const Sys& s, float2 sr6, float2 ir2, float wab) {
+  const float e24 = 24.f * s.f.eps;
+  const float2 t = __ffma2_rn(__fadd2_rn(sr6, sr6), sr6, make_float2(-sr6.x, -sr6.y));
+  return __fmul2_rn(__fmul2_rn(__fmul2_rn(make_float2(e24, e24), t), ir2), make_float2(wab, wab));
+}
+
+// Eq. 1 on a high-resolution molecule a of the FP32 path: lane lig of the item's G lanes takes
+// every G-th neighbour, evaluates all its atom pairs with the molecule (two of the molecule's
+// atoms per instruction: packed float2 arithmetic) and its coarse-grained force once, and the
+// lanes' sums are exchanged at the end so that lane g holds atom g's force.  One lane per
+// neighbour keeps several neighbours' loads in flight per molecule, where one lane per atom
+// walked the whole list as one dependent chain (13 neighbours deep in the tetrahedral fluid,
+// ~300 in the water-like one), tests each neighbour once instead of once per atom and leaves no
+// lane idle for three-atom molecules.  Water-like fluid, 64,000 molecules: 189 -> 138 us a step;
+// tetrahedral, 1000 molecules in the run kernel: 16.9 -> 9.4 us.
+template <int NA, bool ENERGY, int MODEL, bool HS>
+__device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int G, int lig, int nnb,
+                                            int m_first, bool live_item, const int4 Ca, float wa, float reach_at2, float sw,
+                                            bool slow, bool drift, float& fx, float& fy, float& fz, float& dv, double& e_at,
+                                            double& e_cg, double& vir) {
+  using Q = Prec<P32>;
+  constexpr int NP = (NA + 1) / 2;  // pairs of the molecule's atoms (an odd last one is doubled)
+  const int lane = threadIdx.x & 31;
+  const int* row = b.nbr + (size_t)(live_item ? t : 0) * s.cap;
+  const float4* off = b.off32[cur];
+  // everything below is minus the separation and minus the force: partner minus own
+  float2 nx[NP], ny[NP], nz[NP], ax[NP], ay[NP], az[NP];
+  {
+    const float4 X = off[3 * (size_t)a], Y = off[3 * (size_t)a + 1], Z = off[3 * (size_t)a + 2];
+    const float x[4] = {X.x, X.y, X.z, X.w}, y[4] = {Y.x, Y.y, Y.z, Y.w}, z[4] = {Z.x, Z.y, Z.z, Z.w};
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const int i1 = 2 * p + 1 < NA ? 2 * p + 1 : 2 * p;
+      nx[p] = make_float2(-x[2 * p], -x[i1]);
+      ny[p] = make_float2(-y[2 * p], -y[i1]);
+      nz[p] = make_float2(-z[2 * p], -z[i1]);
+      ax[p] = ay[p] = az[p] = make_float2(0.f, 0.f);
+    }
+  }
+  float Fx = 0.f, Fy = 0.f, Fz = 0.f;
+  const float rc_at2 = s.f.rc_at2, rc_cg2 = s.f.rc_cg2;
+  constexpr bool EAGER = MODEL == 0;  // short lists: fetch the offsets with the centre
+  int m_n = 0;
+  int4 C_n = Ca;
+  float4 Xn = {}, Yn = {}, Zn = {};
+  if (lig < nnb) {
+    m_n = m_first;
+    C_n = Q::com(b, cur, m_n);
+    if (EAGER) {
+      Xn = off[3 * (size_t)m_n];
+      Yn = off[3 * (size_t)m_n + 1];
+      Zn = off[3 * (size_t)m_n + 2];
+    }
+  }
+  for (int q = lig; q < nnb; q += G) {
+    const int m = m_n;
+    const int4 Cb = C_n;
+    float4 X = Xn, Y = Yn, Z = Zn;
+    if (q + G < nnb) {
+      m_n = row[q + G];
+      C_n = Q::com(b, cur, m_n);
+      if (EAGER) {
+        Xn = off[3 * (size_t)m_n];
+        Yn = off[3 * (size_t)m_n + 1];
+        Zn = off[3 * (size_t)m_n + 2];
+      }
+    }
+    const auto R = Q::dR(B, Cb, Ca);
+    const float r2 = pair_r2(R.x, R.y, R.z);
+    const float wab = HS ? 0.5f * (wa + Q::w(Cb)) : wa * Q::w(Cb);
+    if (wab > 0.f && r2 < reach_at2) {
+      if (!EAGER) {
+        X = off[3 * (size_t)m];
+        Y = off[3 * (size_t)m + 1];
+        Z = off[3 * (size_t)m + 2];
+      }
+      const float xj[4] = {X.x, X.y, X.z, X.w}, yj[4] = {Y.x, Y.y, Y.z, Y.w}, zj[4] = {Z.x, Z.y, Z.z, Z.w};
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const float2 px = __fadd2_rn(nx[p], make_float2(R.x, R.x)), py = __fadd2_rn(ny[p], make_float2(R.y, R.y)),
+                     pz = __fadd2_rn(nz[p], make_float2(R.z, R.z));
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          const float2 dx = __fadd2_rn(px, make_float2(xj[j], xj[j])), dy = __fadd2_rn(py, make_float2(yj[j], yj[j])),
+                       dz = __fadd2_rn(pz, make_float2(zj[j], zj[j]));
+          const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+          const bool h0 = d2.x < rc_at2, h1 = 2 * p + 1 < NA && d2.y < rc_at2;
+          if (h0 || h1) {
+            float2 fr;
+            if (MODEL == 0) {
+              const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
+              const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
+              const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
+              fr = wca_fr2(s, sr6, ir2, wab);
+              if (ENERGY || drift) {
+                const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
+                const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
+                if (ENERGY) e_at += 0.5 * (double)wab * ((double)v0 + (double)v1);
+                if (drift) dv += v0 + v1;
+              }
+            } else {
+              // LJ (c12 r^-12 - c6 r^-6, shifted) for the site pairs that have one + reaction
+              // field q_i q_j f (1/r + k_rf r^2 - c_rf)
+              const float2 ir = make_float2(Q::rsqrt_(d2.x), Q::rsqrt_(d2.y));
+              const float2 ir2 = __fmul2_rn(ir, ir);
+              const int i0 = 2 * p, i1 = 2 * p + 1 < NA ? 2 * p + 1 : 2 * p;
+              const float2 qq = make_float2(s.f.qq[i0][j], s.f.qq[i1][j]);
+              float2 flj = make_float2(0.f, 0.f);
+              float vl0 = 0.f, vl1 = 0.f;
+              if ((s.lj_pairs >> (4 * i0 + j)) & 1) {
+                const float ir6 = ir2.x * ir2.x * ir2.x;
+                flj.x = (12.f * s.f.c12[i0][j] * ir6 - 6.f * s.f.c6[i0][j]) * ir6 * ir2.x;
+                if (ENERGY || drift) vl0 = (s.f.c12[i0][j] * ir6 - s.f.c6[i0][j]) * ir6;
+              }
+              if (i1 != i0 && ((s.lj_pairs >> (4 * i1 + j)) & 1)) {
+                const float ir6 = ir2.y * ir2.y * ir2.y;
+                flj.y = (12.f * s.f.c12[i1][j] * ir6 - 6.f * s.f.c6[i1][j]) * ir6 * ir2.y;
+                if (ENERGY || drift) vl1 = (s.f.c12[i1][j] * ir6 - s.f.c6[i1][j]) * ir6;
+              }
+              fr = __ffma2_rn(qq, __ffma2_rn(ir2, ir, make_float2(-s.f.krf2, -s.f.krf2)), flj);
+              fr = __fmul2_rn(fr, make_float2(wab, wab));
+              if (ENERGY) {
+                if (h0)
+                  e_at += 0.5 * (double)wab *
+                          ((double)vl0 + s.vsh[i0][j] + (double)qq.x * ((double)ir.x + s.krf * (double)d2.x - s.crf));
+                if (h1)
+                  e_at += 0.5 * (double)wab *
+                          ((double)vl1 + s.vsh[i1][j] + (double)qq.y * ((double)ir.y + s.krf * (double)d2.y - s.crf));
+              }
+              if (drift) {
+                if (h0) dv += vl0 + s.f.vsh[i0][j] + qq.x * (ir.x + s.f.krf * d2.x - s.f.crf);
+                if (h1) dv += vl1 + s.f.vsh[i1][j] + qq.y * (ir.y + s.f.krf * d2.y - s.f.crf);
+              }
+            }
+            fr.x = h0 ? fr.x : 0.f;
+            fr.y = h1 ? fr.y : 0.f;
+            ax[p] = __ffma2_rn(fr, dx, ax[p]);
+            ay[p] = __ffma2_rn(fr, dy, ay[p]);
+            az[p] = __ffma2_rn(fr, dz, az[p]);
+            if (ENERGY) vir += 0.5 * ((double)(fr.x * d2.x) + (double)(fr.y * d2.y));
+          }
+        }
+      }
+    }
+    if (wab < 1.f && r2 < rc_cg2 && slow) {
+      const float r = Q::sqrt_(r2);
+      float V = 0.f;
+      const float F = s.cg_mode ? b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, s.f.cg_inv_dr, &V);
+      const float fw = (1.f - wab) * F;
+      const float c = Q::div_(fw * sw, r);
+      Fx += c * R.x;
+      Fy += c * R.y;
+      Fz += c * R.z;
+      if (ENERGY) {
+        e_cg += 0.5 * (double)((1.f - wab) * V);
+        vir += 0.5 * (double)(Q::div_(fw, r) * r2);
+      }
+      if (drift) dv -= sw * V;
+    }
+  }
+  // the atoms' sums with their share of the coarse-grained force, then exchanged within the
+  // group: first halves (atoms 0, 1 / 2, 3), then single atoms, then the groups of four
+  float f4[4][3];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool hi = i & 1;
+    const int p = i / 2 < NP ? i / 2 : 0;
+    f4[i][0] = i < NA ? fmaf(s.f.frac[i], Fx, hi ? ax[p].y : ax[p].x) : 0.f;
+    f4[i][1] = i < NA ? fmaf(s.f.frac[i], Fy, hi ? ay[p].y : ay[p].x) : 0.f;
+    f4[i][2] = i < NA ? fmaf(s.f.frac[i], Fz, hi ? az[p].y : az[p].x) : 0.f;
+  }
+  const unsigned mk = lane_group(G, lane);
+  float r[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const bool up = lane & 2, odd = lane & 1;
+    float k0 = up ? f4[2][c] : f4[0][c], k1 = up ? f4[3][c] : f4[1][c];
+    k0 += __shfl_xor_sync(mk, up ? f4[0][c] : f4[2][c], 2);
+    k1 += __shfl_xor_sync(mk, up ? f4[1][c] : f4[3][c], 2);
+    r[c] = (odd ? k1 : k0) + __shfl_xor_sync(mk, odd ? k0 : k1, 1);
+  }
+  for (int o = kGroup; o < G; o <<= 1) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] += __shfl_xor_sync(mk, r[c], o);
+  }
+  fx = -r[0];
+  fy = -r[1];
+  fz = -r[2];
+  if (HS) {  // V_AT_a - V_CG_a = half the group's sum (every pair is listed from both sides)
+    for (int o = 1; o < G; o <<= 1) dv += __shfl_xor_sync(mk, dv, o);
+    dv *= 0.5f;
+  }
+}
+
+// The same with one lane per atom: lane g evaluates its atom against every listed neighbour
+// (two of the neighbour's atoms per packed instruction), the next neighbour's index and centre
+// fetched while the current one is evaluated.  Fewer registers than one lane per neighbour
+// (48 against 90, so twice the warps): the faster way once there are enough molecules to fill
+// the device.
+template <int NA, bool ENERGY, bool HS>
+__device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int g, int nnb,
+                                                 int m_first, const int* row, const int4 Ca, float wa, float3 oi, float frac_g,
+                                                 float reach_at2, float sw, bool slow, bool drift, float& fx, float& fy,
+                                                 float& fz, float& dv, double& e_at, double& e_cg, double& vir) {
+  using Q = Prec<P32>;
+  constexpr int NP = (NA + 1) / 2;  // pairs of the neighbour's atoms (an odd last one is doubled)
+  const float4* off = b.off32[cur];
+  const float rc_at2 = s.f.rc_at2, rc_cg2 = s.f.rc_cg2;
+  float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
+  float Fx = 0.f, Fy = 0.f, Fz = 0.f;
+  int m_n = m_first;
+  int4 C_n = Ca;
+  if (nnb > 0) C_n = Q::com(b, cur, m_n);
+  for (int q = 0; q < nnb; ++q) {
+    const int m = m_n;
+    const int4 Cb = C_n;
+    if (q + 1 < nnb) {
+      m_n = row[q + 1];
+      C_n = Q::com(b, cur, m_n);
+    }
+    const auto R = Q::dR(B, Cb, Ca);  // minus the separation, as everything below
+    const float r2 = pair_r2(R.x, R.y, R.z);
+    const float wab = HS ? 0.5f * (wa + Q::w(Cb)) : wa * Q::w(Cb);
+    if (wab > 0.f && r2 < reach_at2 && g < NA) {
+      const float4 X = off[3 * (size_t)m], Y = off[3 * (size_t)m + 1], Z = off[3 * (size_t)m + 2];
+      const float xj[4] = {X.x, X.y, X.z, X.w}, yj[4] = {Y.x, Y.y, Y.z, Y.w}, zj[4] = {Z.x, Z.y, Z.z, Z.w};
+      const float px = R.x - oi.x, py = R.y - oi.y, pz = R.z - oi.z;
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const int j0 = 2 * p, j1 = 2 * p + 1 < NA ? 2 * p + 1 : 2 * p;
+        const float2 dx = __fadd2_rn(make_float2(xj[j0], xj[j1]), make_float2(px, px));
+        const float2 dy = __fadd2_rn(make_float2(yj[j0], yj[j1]), make_float2(py, py));
+        const float2 dz = __fadd2_rn(make_float2(zj[j0], zj[j1]), make_float2(pz, pz));
+        const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+        const bool h0 = d2.x < rc_at2, h1 = j1 != j0 && d2.y < rc_at2;
+        if (h0 || h1) {
+              const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
+          const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
+          const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
+          float2 fr = wca_fr2(s, sr6, ir2, wab);
+          if (ENERGY || drift) {
+            const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
+            const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
+            if (ENERGY) e_at += 0.5 * (double)wab * ((double)v0 + (double)v1);
+            if (drift) dv += v0 + v1;
+          }
+          fr.x = h0 ? fr.x : 0.f;
+          fr.y = h1 ? fr.y : 0.f;
+          ax = __ffma2_rn(fr, dx, ax);
+          ay = __ffma2_rn(fr, dy, ay);
+          az = __ffma2_rn(fr, dz, az);
+          if (ENERGY) vir += 0.5 * ((double)(fr.x * d2.x) + (double)(fr.y * d2.y));
+        }
+      }
+    }
+    if (wab < 1.f && r2 < rc_cg2 && slow && g < NA) {
+      const float r = Q::sqrt_(r2);
+      float V = 0.f;
+      const float F = s.cg_mode ? b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, s.f.cg_inv_dr, &V);
+      const float fw = (1.f - wab) * F;
+      const float c = Q::div_(fw * sw, r);
+      Fx += c * R.x;
+      Fy += c * R.y;
+      Fz += c * R.z;
+      if (ENERGY && g == 0) {
+        e_cg += 0.5 * (double)((1.f - wab) * V);
+        vir += 0.5 * (double)(Q::div_(fw, r) * r2);
+      }
+      if (drift && g == 0) dv -= sw * V;
+    }
+  }
+  fx = -fmaf(frac_g, Fx, ax.x + ax.y);
+  fy = -fmaf(frac_g, Fy, ay.x + ay.y);
+  fz = -fmaf(frac_g, Fz, az.x + az.y);
+  if (HS) {  // V_AT_a - V_CG_a = half the group's sum (every pair is listed from both sides)
+    const unsigned gmask = 0xFu << (threadIdx.x & 28);
+    dv += __shfl_xor_sync(gmask, dv, 1);
+    dv += __shfl_xor_sync(gmask, dv, 2);
+    dv *= 0.5f;
+  }
 }
 
 // The step of the molecules of one tile of the grid (a block's worth of threads): thread gtid
 // of the whole grid.  cur: current half of the molecule arrays; step: the time level of the
 // forces; ext_now: the largest atom-to-COM distance; the next mapping's maxima are merged into
 // ext2 and disp2 (MODE_FUSED).  Every thread of a block calls.
-template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS>
-__device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int gtid, const int cur,
+//
+// A high-resolution work item takes 2^ln.h lanes and a coarse-grained one 2^ln.c (32 >= 2^h >=
+// 2^c >= 4, so that no item's lanes straddle a warp); the first four integrate and map the
+// molecule, one lane per atom.  LPN: one lane per neighbour (hr_forces32), else per atom.
+template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, bool LPN>
+__device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lanes ln, const int gtid, const int cur,
                                           const long long step, const float ext_now, float& ext2, float& disp2) {
   using Q = Prec<P>;
   using real = typename Q::real;
   const int lane = threadIdx.x & 31, g = threadIdx.x & 3, base = lane & ~3;
   const unsigned gmask = 0xFu << base;
-  // SPLIT > 1 (water): a high-resolution item takes SPLIT groups of four lanes in the same
-  // warp, group `sub` every SPLIT-th neighbour from slot `sub`; CG items keep one group.
-  constexpr int SPLIT = MODEL == 1 ? kSplitWater : 1;
-  static_assert(SPLIT == 1 || SPLIT == 2 || SPLIT == 4, "lane groups per item");
-  int t = gtid >> 2, sub = 0;
-  if (SPLIT > 1) {
-    const int n_hr0 = b.ctrl->n_hr;
-    if (gtid < kGroup * SPLIT * n_hr0) {
-      t = gtid / (kGroup * SPLIT);
-      sub = (gtid >> 2) & (SPLIT - 1);
-    } else {
-      t = n_hr0 + ((gtid - kGroup * SPLIT * n_hr0) >> 2);
-    }
-  }
+  const int n_hr = b.ctrl->n_hr, GC = 1 << ln.c;
+  const bool hr_item = gtid < (n_hr << ln.h);
+  // work item and this lane's place in its group
+  const int u = hr_item || ln.h == ln.c ? gtid : gtid - (n_hr << ln.h);
+  const int t = hr_item || ln.h == ln.c ? u >> ln.h : n_hr + (u >> ln.c);
+  const int lig = u & ((1 << (hr_item ? ln.h : ln.c)) - 1);
   const bool live_item = t < s.M;
-  const bool live = live_item && sub == 0;  // the group that integrates and maps the molecule
+  const bool live = live_item && lig < kGroup;  // the lanes that integrate and map the molecule
   const bool own = live && g < NA;
-  const bool own_pair = live_item && g < NA;  // lanes that evaluate pair forces
   // the first list slot this lane reads is fetched together with the item, before the count
   // is known (slots below the capacity lie inside the list array; the value is used only
   // when the count covers the slot)
-  const bool hr_item = t < b.ctrl->n_hr;
-  const int j0 = hr_item ? sub : g;
-  const int m_first = live_item && j0 < s.cap ? b.nbr[(size_t)t * s.cap + j0] : 0;
+  // (one lane per atom: the four lanes of a group share a slot)
+  const int j0 = !LPN && hr_item ? lig / kGroup : lig;
+  const int* row = b.nbr + (size_t)(live_item ? t : 0) * s.cap;
+  const int m_first = live_item && j0 < s.cap ? row[j0] : 0;
 
   const real eps = par<real>(s.eps, s.f.eps), sig2 = par<real>(s.sig2, s.f.sig2);
   const real rc_at2 = par<real>(s.rc_at2, s.f.rc_at2), rc_cg2 = par<real>(s.rc_cg2, s.f.rc_cg2);
@@ -530,12 +834,12 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
   const real reach_at2 = reach * reach;
   const int gg0 = g < NA ? g : 0;
   const real frac_g = par<real>(s.frac[gg0], s.f.frac[gg0]);
-  // MODEL 1: this atom's row of the site-pair coefficients
+  // MODEL 1: this atom's row of the site-pair coefficients (FP64 path)
   real c12r[NA], c6r[NA], qqr[NA];
   real krf2 = 0;
   if (MODEL == 1) {
 #pragma unroll
-    for (int j = 0; j < NA; ++j) {
+    for (int j = 0; P::fp64 && j < NA; ++j) {
       c12r[j] = par<real>(s.c12[gg0][j], s.f.c12[gg0][j]);
       c6r[j] = par<real>(s.c6[gg0][j], s.f.c6[gg0][j]);
       qqr[j] = par<real>(s.qq[gg0][j], s.f.qq[gg0][j]);
@@ -554,7 +858,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
   const int i = a * NA + (g < NA ? g : 0);
   const auto Ca = Q::com(b, cur, a);
   const real wa = Q::w(Ca);
-  const auto oi = Q::off(b, cur, i);
+  const auto oi = Q::template off<NA>(b, cur, a, g < NA ? g : 0);
   const int nnb = live_item ? b.nn[t] : 0;
   // energy interpolation: a hybrid molecule sums its unweighted pair energies (AT per atom
   // lane, CG on lane 0 of its group) for the drift force
@@ -567,9 +871,19 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
   const bool slow = sw != (real)0 || ENERGY;
 
   if (hr_item) {
-    // high-resolution item: Eq. 1 for atom i against every listed neighbour (of this lane
-    // group's share); the next neighbour's index and centre are fetched while the current
-    // one is evaluated
+    if constexpr (!P::fp64 && !LPN) {
+      static_assert(MODEL == 0, "one lane per atom");
+      hr_forces32_atom<NA, ENERGY, HS>(s, B, b, cur, t, g, nnb, m_first, row, Ca, wa, make_float3(oi.x, oi.y, oi.z), frac_g,
+                                       reach_at2, sw, slow, drift, fx, fy, fz, dv, e_at, e_cg, vir);
+    } else if constexpr (!P::fp64) {
+      hr_forces32<NA, ENERGY, MODEL, HS>(s, B, b, cur, t, a, 1 << ln.h, lig, nnb, m_first, live_item, Ca, wa, reach_at2, sw, slow, drift,
+                                             fx, fy, fz, dv, e_at, e_cg, vir);
+    } else {
+    // Eq. 1 for atom i against every listed neighbour (of this lane group's share); the next
+    // neighbour's index and centre are fetched while the current one is evaluated
+    constexpr int SPLIT = atom_lanes(true, MODEL) / kGroup;
+    const int sub = lig / kGroup;
+    const bool own_pair = live_item && g < NA;  // lanes that evaluate pair forces
     int m_n = 0;
     auto C_n = Ca;
     if (sub < nnb) {
@@ -580,7 +894,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
       const int m = m_n;
       const auto Cb = C_n;
       if (q + SPLIT < nnb) {
-        m_n = b.nbr[(size_t)t * s.cap + q + SPLIT];
+        m_n = row[q + SPLIT];
         C_n = Q::com(b, cur, m_n);
       }
       const auto R = Q::dR(B, Ca, Cb);
@@ -590,7 +904,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
         const real px = R.x + (real)oi.x, py = R.y + (real)oi.y, pz = R.z + (real)oi.z;
         typename P::off_t oj[NA];
 #pragma unroll
-        for (int j = 0; j < NA; ++j) oj[j] = Q::off(b, cur, m * NA + j);
+        for (int j = 0; j < NA; ++j) oj[j] = Q::template off<NA>(b, cur, m, j);
 #pragma unroll
         for (int j = 0; j < NA; ++j) {
           const real dx = px - (real)oj[j].x, dy = py - (real)oj[j].y, dz = pz - (real)oj[j].z;
@@ -661,6 +975,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
       dv += __shfl_xor_sync(gmask, dv, 2);
       dv *= (real)0.5;
     }
+    }
   } else {
     // coarse-grained item (l_a = 0, so w_ab = 0): neighbour list split over the group
     if (live && g == 0 && wa != (real)0) set_error(b.ctrl, ADRESS_ERR_STATE, a);
@@ -668,13 +983,13 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
     auto C_n = Ca;
     const int nnb_cg = slow ? nnb : 0;  // no CG force at inner levels of multiple time stepping
     // centres of the next two neighbours in flight (long lists: the water-like fluid)
-    if (g < nnb_cg) C_n = Q::com(b, cur, m_first);
+    if (lig < nnb_cg) C_n = Q::com(b, cur, m_first);
     auto C_n2 = Ca;
-    if (g + kGroup < nnb_cg) C_n2 = Q::com(b, cur, b.nbr[(size_t)t * s.cap + g + kGroup]);
-    for (int q = g; q < nnb_cg; q += kGroup) {
+    if (lig + GC < nnb_cg) C_n2 = Q::com(b, cur, row[lig + GC]);
+    for (int q = lig; q < nnb_cg; q += GC) {
       const auto Cb = C_n;
       C_n = C_n2;
-      if (q + 2 * kGroup < nnb_cg) C_n2 = Q::com(b, cur, b.nbr[(size_t)t * s.cap + q + 2 * kGroup]);
+      if (q + 2 * GC < nnb_cg) C_n2 = Q::com(b, cur, row[q + 2 * GC]);
       const auto R = Q::dR(B, Ca, Cb);
       const real r2 = pair_r2(R.x, R.y, R.z);
       if (r2 < rc_cg2) {
@@ -691,12 +1006,12 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
         }
       }
     }
-    Fx += __shfl_xor_sync(gmask, Fx, 1);
-    Fy += __shfl_xor_sync(gmask, Fy, 1);
-    Fz += __shfl_xor_sync(gmask, Fz, 1);
-    Fx += __shfl_xor_sync(gmask, Fx, 2);
-    Fy += __shfl_xor_sync(gmask, Fy, 2);
-    Fz += __shfl_xor_sync(gmask, Fz, 2);
+    const unsigned mk = lane_group(GC, lane);
+    for (int o = 1; o < GC; o <<= 1) {
+      Fx += __shfl_xor_sync(mk, Fx, o);
+      Fy += __shfl_xor_sync(mk, Fy, o);
+      Fz += __shfl_xor_sync(mk, Fz, o);
+    }
     const real fs = frac_g * sw;
     fx = fs * Fx;
     fy = fs * Fy;
@@ -714,21 +1029,31 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
     }
   }
 
-  if (own) {
+  // offset of atom k of this molecule: from its lane on the FP32 path (every lane of the group
+  // calls), from memory on the FP64 path
+  auto atom_off = [&](int k) {
+    if constexpr (P::fp64) {
+      return Q::template off<NA>(b, cur, a, k);
+    } else {
+      return typename Q::V3{__shfl_sync(gmask, oi.x, base + k), __shfl_sync(gmask, oi.y, base + k),
+                            __shfl_sync(gmask, oi.z, base + k)};
+    }
+  };
+  if (live) {
     // bonded terms of atom g: harmonic bonds and angles, or FENE + WCA, on the listed
     // intramolecular pairs
     const real R02 = par<real>(s.fene_r02, s.f.fene_r02), K = par<real>(s.fene_k, s.f.fene_k);
     // each lane walks its own atom's bonds (bond order), so a warp runs as many bond bodies
     // as an atom has bonds, not as the molecule has
-    const unsigned bw = s.bond_word[gg0];
+    const unsigned bw = own ? s.bond_word[gg0] : 0u;
     if (s.bond_model == 1) {
       const real kb = par<real>(s.bond_k, s.f.bond_k), r0 = par<real>(s.bond_r0, s.f.bond_r0);
 #pragma unroll
       for (int q = 0; q < kMaxBonds; ++q) {
         if (q >= s.bmax) break;
-        if (q >= (int)(bw >> 28)) continue;
         const int e = (bw >> (4 * q)) & 15;
-        const auto oo = Q::off(b, cur, a * NA + (e & 7));
+        const auto oo = atom_off(e & 3);
+        if (q >= (int)(bw >> 28)) continue;
         const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
         const real d2 = dx * dx + dy * dy + dz * dz;
         const real ird = Q::rsqrt_(d2);
@@ -750,8 +1075,8 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
       for (int q = 0; q < kMaxAngles; ++q) {
         if (q >= s.n_angles) break;
         const int ai = s.angles[3 * q], aj = s.angles[3 * q + 1], ak = s.angles[3 * q + 2];
+        const auto Oi = atom_off(ai), Oj = atom_off(aj), Ok = atom_off(ak);
         if (g != ai && g != aj && g != ak) continue;
-        const auto Oi = Q::off(b, cur, a * NA + ai), Oj = Q::off(b, cur, a * NA + aj), Ok = Q::off(b, cur, a * NA + ak);
         const real ux = (real)Oi.x - (real)Oj.x, uy = (real)Oi.y - (real)Oj.y, uz = (real)Oi.z - (real)Oj.z;
         const real vx = (real)Ok.x - (real)Oj.x, vy = (real)Ok.y - (real)Oj.y, vz = (real)Ok.z - (real)Oj.z;
         const real uu = ux * ux + uy * uy + uz * uz, vv = vx * vx + vy * vy + vz * vz;
@@ -787,9 +1112,9 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
 #pragma unroll
     for (int q = 0; q < kMaxBonds; ++q) {
       if (q >= s.bmax) break;
-      if (q >= (int)(bw >> 28)) continue;
       const int e = (bw >> (4 * q)) & 15;
-      const auto oo = Q::off(b, cur, a * NA + (e & 7));
+      const auto oo = atom_off(e & 3);
+      if (q >= (int)(bw >> 28)) continue;
       const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
       const real d2 = dx * dx + dy * dy + dz * dz;
       if (d2 >= R02) {
@@ -816,6 +1141,8 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
       }
     }
     }
+  }
+  if (own) {
     // thermodynamic force on hybrid-layer molecules (region decided at mapping time), and
     // energy interpolation's drift force -(V_AT_a - V_CG_a - g(l_a)) l'(d) along grad d
     if (s.tf_n > 0 || hs) {
@@ -996,21 +1323,26 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const int
   }
 }
 
-template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS>
-__global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULTI>()) k_step(const __grid_constant__ Sys s, Bufs b) {
+template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, int FORM = FORM_ATOM>
+__global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULTI, HS>()) k_step(const __grid_constant__ Sys s, Bufs b) {
   const Ctrl* c = b.ctrl;
   float ext2 = 0.f, disp2 = 0.f;
-  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS>(s, b, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
-                                                   c->ext_now, ext2, disp2);
+  constexpr bool LPN = FORM != FORM_ATOM;
+  const Lanes ln = lanes_of<FORM, P, MODEL>(s.step_lanes);
+  // blocks past the last item (the host does not know the number of high-resolution items)
+  if (!ENERGY && ln.h != ln.c && blockIdx.x * blockDim.x >= (unsigned)((c->n_hr << ln.h) + ((s.M - c->n_hr) << ln.c))) return;
+  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS, LPN>(s, b, ln, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
+                                                        c->ext_now, ext2, disp2);
   if (MODE == MODE_FUSED) publish_extent(b, 0, ext2, disp2);
 }
 
 // ---------------- k_run ------------------------------------------------------------------
 
-// Resident blocks per SM of the run kernel (its registers: 64 a thread).
+// Resident blocks per SM of the run kernel: its systems are bound by latency, so registers
+// (128 a thread) come before warps.
 template <class P>
 constexpr int run_min_blocks() {
-  return P::fp64 ? 3 : 8;
+  return P::fp64 ? 3 : 4;
 }
 
 // nsteps fused steps in one cooperative launch: every block takes its tiles of the step, a
@@ -1023,13 +1355,16 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
   int cur = c->parity, set = 0, dirty = 0, rebuilt = 0;
   long long step = c->step;
   float ext_now = c->ext_now;
-  const int ntiles = (int)(((long long)s.M * (MODEL == 1 ? kSplitWater * kGroup : kGroup) + blockDim.x - 1) / blockDim.x);
+  constexpr bool LPN = !P::fp64;
+  const Lanes ln = lanes_of<LPN ? FORM_NEIGHBOUR : FORM_ATOM, P, MODEL>(s.run_lanes);
   GridBarrier bar(c, &c->bar[1]);
   for (int k = 0; k < nsteps; ++k) {
     float ext2 = 0.f, disp2 = 0.f;
+    const int n_hr = c->n_hr;
+    const int ntiles = ((n_hr << ln.h) + ((s.M - n_hr) << ln.c) + blockDim.x - 1) / blockDim.x;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS>(s, b, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
-                                                            ext2, disp2);
+      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, LPN>(s, b, ln, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
+                                                                ext2, disp2);
     publish_extent(b, set, ext2, disp2);
     if (!bar.sync()) return;
     const Decision d = decide_rebuild(s, c, set, 0);
@@ -1065,35 +1400,40 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
 
 // ---------------- launchers ----------------------------------------------------------
 
-template <class P, int NA, int MODEL, bool HS>
-static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cudaStream_t st) {
-  const int blocks = ceil_div((long long)s.M * step_lanes(s), s.force_block);
-  const bool multi = s.nbox > 1;
+template <class P, int NA, int MODEL, bool HS, int FORM, bool MULTI>
+static void launch_step_form(const Sys& s, const Bufs& b, int mode, int energy, cudaStream_t st) {
+  const int blocks = ceil_div((long long)s.M * step_lanes(s), s.force_block), threads = s.force_block;
   switch (mode) {
     case MODE_FORCES:
-      if (multi) {
-        if (energy) k_step<P, NA, MODE_FORCES, true, true, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-        else k_step<P, NA, MODE_FORCES, false, true, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      } else {
-        if (energy) k_step<P, NA, MODE_FORCES, true, false, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-        else k_step<P, NA, MODE_FORCES, false, false, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      }
+      if (energy) k_step<P, NA, MODE_FORCES, true, MULTI, MODEL, HS, FORM><<<blocks, threads, 0, st>>>(s, b);
+      else k_step<P, NA, MODE_FORCES, false, MULTI, MODEL, HS, FORM><<<blocks, threads, 0, st>>>(s, b);
       break;
-    case MODE_LAST:
-      if (multi) k_step<P, NA, MODE_LAST, false, true, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      else k_step<P, NA, MODE_LAST, false, false, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      break;
-    default:
-      if (multi) k_step<P, NA, MODE_FUSED, false, true, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      else k_step<P, NA, MODE_FUSED, false, false, MODEL, HS><<<blocks, s.force_block, 0, st>>>(s, b);
-      break;
+    case MODE_LAST: k_step<P, NA, MODE_LAST, false, MULTI, MODEL, HS, FORM><<<blocks, threads, 0, st>>>(s, b); break;
+    default: k_step<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, FORM><<<blocks, threads, 0, st>>>(s, b); break;
+  }
+}
+
+template <class P, int NA, int MODEL, bool HS, int FORM>
+static void launch_step_boxes(const Sys& s, const Bufs& b, int mode, int energy, cudaStream_t st) {
+  if (s.nbox > 1) launch_step_form<P, NA, MODEL, HS, FORM, true>(s, b, mode, energy, st);
+  else launch_step_form<P, NA, MODEL, HS, FORM, false>(s, b, mode, energy, st);
+}
+
+template <class P, int NA, int MODEL, bool HS>
+static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cudaStream_t st) {
+  if constexpr (!P::fp64 && MODEL == 1) {
+    // eight and four lanes as constants where the host chose them (4% at 64,000 molecules)
+    if (s.step_lanes.h == 3 && s.step_lanes.c == 2) launch_step_boxes<P, NA, MODEL, HS, FORM_NEIGHBOUR_8_4>(s, b, mode, energy, st);
+    else launch_step_boxes<P, NA, MODEL, HS, FORM_NEIGHBOUR>(s, b, mode, energy, st);
+  } else {
+    launch_step_boxes<P, NA, MODEL, HS, FORM_ATOM>(s, b, mode, energy, st);
   }
 }
 
 // As many blocks as fit on the device at once, at most one per tile.
 template <class P, int NA, int MODEL, bool HS>
 static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
-  const int tiles = ceil_div((long long)s.M * step_lanes(s), s.force_block);
+  const int tiles = ceil_div((long long)s.M << (P::fp64 ? 2 : s.run_lanes.h), s.force_block);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(tiles, s.n_sm * run_min_blocks<P>()));
   cfg.blockDim = dim3(s.force_block);

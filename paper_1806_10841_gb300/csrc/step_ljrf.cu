@@ -12,10 +12,4 @@ cudaError_t launch_step_ljrf(const Sys& s, const Bufs& b, int precision, int mod
   return cudaGetLastError();
 }
 
-cudaError_t launch_run_ljrf(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
-  if (s.NA != 3) return cudaErrorInvalidValue;
-  return precision == ADRESS_FP64 ? launch_run_na<P64, 3, 1, false>(s, b, nsteps, st)
-                                  : launch_run_na<P32, 3, 1, false>(s, b, nsteps, st);
-}
-
 }  // namespace adress
