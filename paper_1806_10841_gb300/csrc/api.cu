@@ -657,8 +657,8 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
       A(b.off64[p], N);
     } else {
       A(b.molf[p], M);
-      A(b.off32[p], (size_t)3 * M);
     }
+    A(b.off32[p], (size_t)3 * M);
     if (c->n_centers > 0) A(b.kcen[p], M);
   }
   A(b.mcell, M);

@@ -187,7 +187,7 @@ struct Bufs {
   int* kcen[2];            // spheres: index of the nearest centre
   // per atom, double-buffered
   double4_32a* off64[2];   // COM-relative atom offsets (FP64 path)
-  float4* off32[2];        // FP32 path: [M][3], the x, y and z components of a molecule's (up to
+  float4* off32[2];        // [M][3], the x, y and z components of a molecule's (up to
                            // four) atoms, so that a molecule's offsets are three 16-byte loads
                            // and adjacent atoms pair up in packed float2 arithmetic
   // lists

@@ -109,6 +109,31 @@ __device__ __forceinline__ void philox4x32_10(unsigned c[4], unsigned k0, unsign
   }
 }
 
+// ---------------- FP64 reciprocal and square root ----------------------------------------
+// Newton-Raphson from the hardware's approximations (about 20 bits): two steps reach the last
+// bit or two.  The FP64 pipe runs 2 lanes a clock per SM here, and the library's division and
+// square root cost 2-3 times as many of its instructions.
+
+__device__ __forceinline__ double rcp_nr(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = 0.5 * x;
+  y = fma(fma(-h * y, y, 0.5), y, y);
+  return fma(fma(-h * y, y, 0.5), y, y);
+}
+// Minimum image for |d| < 1.5 L, the comparison on the bits (off the FP64 pipe).
+__device__ __forceinline__ double minimg_bits(double d, double L, double halfL) {
+  const long long b = __double_as_longlong(d), h = __double_as_longlong(halfL);
+  if ((b & 0x7fffffffffffffffll) > h) d -= b < 0 ? -L : L;
+  return d;
+}
+
 // ---------------- precision policies for the pair loop --------------------------------
 
 template <class P>
@@ -123,8 +148,8 @@ struct Prec<P64> {
   static __device__ __forceinline__ double4_32a com(const Bufs& b, int cur, int a) { return b.com64[cur][a]; }
   static __device__ __forceinline__ double w(const double4_32a& c) { return c.w; }
   static __device__ __forceinline__ V3 dR(const Box& X, const double4_32a& A, const double4_32a& B) {
-    return {minimg_cmp(A.x - B.x, X.L[0], X.halfL[0]), minimg_cmp(A.y - B.y, X.L[1], X.halfL[1]),
-            minimg_cmp(A.z - B.z, X.L[2], X.halfL[2])};
+    return {minimg_bits(A.x - B.x, X.L[0], X.halfL[0]), minimg_bits(A.y - B.y, X.L[1], X.halfL[1]),
+            minimg_bits(A.z - B.z, X.L[2], X.halfL[2])};
   }
   // offset of atom k of molecule a (NA atoms per molecule)
   template <int NA>
@@ -142,11 +167,10 @@ struct Prec<P64> {
   static __device__ __forceinline__ double tf(const Bufs& b, int k) { return b.tf64[k]; }
   static __device__ __forceinline__ double fec(const Bufs& b, int k) { return b.fec64[k]; }
   static __device__ __forceinline__ double sin_(double x) { return sin(x); }
-  static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-  static __device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double rsqrt_(double x) { return 1.0 / sqrt(x); }
+  static __device__ __forceinline__ double rcp_(double x) { return rcp_nr(x); }
+  static __device__ __forceinline__ double rsqrt_(double x) { return rsqrt_nr(x); }
   static __device__ __forceinline__ double acos_(double x) { return acos(x); }
-  static __device__ __forceinline__ double div_(double a, double x) { return a / x; }
+  static __device__ __forceinline__ double div_(double a, double x) { return a * rcp_nr(x); }
 };
 
 template <>
@@ -393,6 +417,11 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
   if (own) {
     const double o0 = dl[0] - c[0], o1 = dl[1] - c[1], o2 = dl[2] - c[2];
     b.off64[nxt][a * NA + g] = make_double4_32a(o0, o1, o2, 0.0);
+    // as float for the pair tests that decide where FP64 is needed
+    float* of = (float*)(b.off32[nxt] + 3 * (size_t)a) + g;
+    of[0] = d2f_bits(o0);
+    of[4] = d2f_bits(o1);
+    of[8] = d2f_bits(o2);
     ext2 = fmaxf(ext2, (float)(o0 * o0 + o1 * o1 + o2 * o2));
   }
   int kmin = 0;
@@ -414,7 +443,11 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
     unsigned X[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) X[d] = (unsigned)(unsigned long long)llrint(R[d] * B.fx_inv[d]);
-    b.com_fx[nxt][a] = make_int4((int)X[0], (int)X[1], (int)X[2], __float_as_int((float)w));
+    // the float weight is 0 or 1 only where the double one is
+    float wf = (float)w;
+    if (w < 1.0 && wf >= 1.f) wf = 0x1.fffffep-1f;
+    if (w > 0.0 && !(wf > 0.f)) wf = 0x1p-126f;
+    b.com_fx[nxt][a] = make_int4((int)X[0], (int)X[1], (int)X[2], __float_as_int(wf));
     const float d0 = (float)(int)(X[0] - (unsigned)ref.x) * B.fx_scale[0];
     const float d1 = (float)(int)(X[1] - (unsigned)ref.y) * B.fx_scale[1];
     const float d2 = (float)(int)(X[2] - (unsigned)ref.z) * B.fx_scale[2];
@@ -795,6 +828,146 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
   }
 }
 
+// Eq. 1 on a high-resolution molecule a of the FP64 path: lane g has atom g, lane group `sub` of
+// SPLIT every SPLIT-th neighbour.  The FP64 pipe is the bound (2 lanes a clock per SM against
+// 128 in FP32), and nine of ten listed atom pairs are beyond the cutoff, so a batch of
+// neighbours is first tested in FP32 with a margin (fixed-point centres and float offsets, errors
+// below 1e-5 of the cutoff against a margin of 1e-4) and only what passes is evaluated, and
+// tested again, in FP64; the coarse-grained force of a pair is evaluated by one lane of the
+// group.  800k atoms: 930 -> 516 us a step, 80k atoms all-atomistic 216 -> 80 us.
+template <int NA, bool ENERGY, int MODEL, bool HS, int SPLIT>
+__device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int g, int sub, int nnb,
+                                            bool live_item, const int* row, const double4_32a Ca, const double4_32a oi,
+                                            double frac_g, double reach_at2, double sw, bool slow, bool drift,
+                                            const double (&c12r)[NA], const double (&c6r)[NA], const double (&qqr)[NA],
+                                            double& fx, double& fy, double& fz, double& dv, double& e_at, double& e_cg,
+                                            double& vir) {
+  using Q = Prec<P64>;
+  constexpr float kMargin = 1.0001f;
+  constexpr int kBatch = 16;  // neighbours per batch: four hit bits each
+  const float rcf = s.f.rc_at2 * kMargin, rcgf = s.f.rc_cg2 * kMargin, reachf = (float)reach_at2 * kMargin;
+  const int4 Cf = b.com_fx[cur][a];
+  const float waf = __int_as_float(Cf.w);
+  const float* of = (const float*)(b.off32[cur] + 3 * (size_t)a) + (g < NA ? g : 0);
+  const float ox = of[0], oy = of[4], oz = of[8];
+  const int gg = g < NA ? g : 0;
+  double Fx = 0.0, Fy = 0.0, Fz = 0.0;
+  for (int q0 = sub; q0 < nnb; q0 += kBatch * SPLIT) {
+    unsigned long long hits = 0ull;
+    unsigned cgs = 0u;
+    int m_n = row[q0];
+    int4 C_n = b.com_fx[cur][m_n];
+    for (int k = 0; k < kBatch; ++k) {
+      const int q = q0 + k * SPLIT;
+      if (q >= nnb) break;
+      const int m = m_n;
+      const int4 Cb = C_n;
+      if (k + 1 < kBatch && q + SPLIT < nnb) {
+        m_n = row[q + SPLIT];
+        C_n = b.com_fx[cur][m_n];
+      }
+      const float Rx = (float)(int)((unsigned)Cf.x - (unsigned)Cb.x) * B.fx_scale[0];
+      const float Ry = (float)(int)((unsigned)Cf.y - (unsigned)Cb.y) * B.fx_scale[1];
+      const float Rz = (float)(int)((unsigned)Cf.z - (unsigned)Cb.z) * B.fx_scale[2];
+      const float r2 = pair_r2(Rx, Ry, Rz), wbf = __int_as_float(Cb.w);
+      if (g < NA && r2 < reachf && (HS ? waf > 0.f || wbf > 0.f : waf > 0.f && wbf > 0.f)) {
+        const float4* off = b.off32[cur] + 3 * (size_t)m;
+        const float4 X = off[0], Y = off[1], Z = off[2];
+        const float xj[4] = {X.x, X.y, X.z, X.w}, yj[4] = {Y.x, Y.y, Y.z, Y.w}, zj[4] = {Z.x, Z.y, Z.z, Z.w};
+        const float px = Rx + ox, py = Ry + oy, pz = Rz + oz;
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          const float dx = px - xj[j], dy = py - yj[j], dz = pz - zj[j];
+          if (dx * dx + dy * dy + dz * dz < rcf) hits |= 1ull << (4 * k + j);
+        }
+      }
+      if ((k & 3) == g && slow && r2 < rcgf && (waf < 1.f || wbf < 1.f)) cgs |= 1u << k;
+    }
+    while (hits) {
+      const int bit = __ffsll((long long)hits) - 1;
+      hits &= hits - 1;
+      const int m = row[q0 + (bit >> 2) * SPLIT], j = bit & 3;
+      const double4_32a Cb = b.com64[cur][m], oj = b.off64[cur][m * NA + j];
+      const auto R = Q::dR(B, Ca, Cb);
+      const double wab = HS ? 0.5 * (Ca.w + Cb.w) : Ca.w * Cb.w;
+      const double dx = R.x + oi.x - oj.x, dy = R.y + oi.y - oj.y, dz = R.z + oi.z - oj.z;
+      const double d2 = dx * dx + dy * dy + dz * dz;
+      if (d2 < s.rc_at2) {
+        double fr;
+        if (MODEL == 0) {
+          const double ir2 = rcp_nr(d2);
+          const double sr2 = s.sig2 * ir2;
+          const double sr6 = sr2 * sr2 * sr2;
+          fr = 24.0 * s.eps * (2.0 * sr6 * sr6 - sr6) * ir2 * wab;
+          if (ENERGY) e_at += 0.5 * wab * (4.0 * s.eps * (sr6 * sr6 - sr6) + s.eps);
+          if (drift) dv += 4.0 * s.eps * (sr6 * sr6 - sr6) + s.eps;
+        } else {
+          // LJ (c12 r^-12 - c6 r^-6, shifted) + reaction field q_i q_j f (1/r + k_rf r^2 - c_rf);
+          // this atom's coefficients with site j
+          double c12 = c12r[0], c6 = c6r[0], qq = qqr[0];
+#pragma unroll
+          for (int e = 1; e < NA; ++e)
+            if (j == e) {
+              c12 = c12r[e];
+              c6 = c6r[e];
+              qq = qqr[e];
+            }
+          const double ir = rsqrt_nr(d2), ir2 = ir * ir;
+          double flj = 0.0, vlj = 0.0;
+          if ((s.lj_cols >> j) & 1) {
+            const double ir6 = ir2 * ir2 * ir2;
+            flj = (12.0 * c12 * ir6 - 6.0 * c6) * ir6 * ir2;
+            if (ENERGY || drift) vlj = (c12 * ir6 - c6) * ir6;
+          }
+          fr = (flj + qq * (ir2 * ir - 2.0 * s.krf)) * wab;
+          if (ENERGY || drift) {
+            const double v = vlj + s.vsh[gg][j] + qq * (ir + s.krf * d2 - s.crf);
+            if (ENERGY) e_at += 0.5 * wab * v;
+            if (drift) dv += v;
+          }
+        }
+        fx += fr * dx;
+        fy += fr * dy;
+        fz += fr * dz;
+        if (ENERGY) vir += 0.5 * (fr * d2);
+      }
+    }
+    while (cgs) {
+      const int k = __ffs((int)cgs) - 1;
+      cgs &= cgs - 1;
+      const int q = q0 + k * SPLIT;
+      const double4_32a Cb = b.com64[cur][row[q]];
+      const auto R = Q::dR(B, Ca, Cb);
+      const double r2 = pair_r2(R.x, R.y, R.z);
+      const double wab = HS ? 0.5 * (Ca.w + Cb.w) : Ca.w * Cb.w;
+      if (wab < 1.0 && r2 < s.rc_cg2) {
+        const double ir = rsqrt_nr(r2), r = r2 * ir;
+        double V = 0.0;
+        const double F = s.cg_mode ? (double)b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, s.cg_inv_dr, &V);
+        const double fw = (1.0 - wab) * F, c = fw * sw * ir;
+        Fx += c * R.x;
+        Fy += c * R.y;
+        Fz += c * R.z;
+        if (ENERGY) {
+          e_cg += 0.5 * (1.0 - wab) * V;
+          vir += 0.5 * (fw * r);
+        }
+        if (drift) dv -= sw * V;
+      }
+    }
+  }
+  const unsigned gmask = 0xFu << (threadIdx.x & 28);
+#pragma unroll
+  for (int o = 1; o < kGroup; o <<= 1) {
+    Fx += shfl_xor_d(gmask, Fx, o);
+    Fy += shfl_xor_d(gmask, Fy, o);
+    Fz += shfl_xor_d(gmask, Fz, o);
+  }
+  fx += frac_g * Fx;
+  fy += frac_g * Fy;
+  fz += frac_g * Fz;
+}
+
 // The step of the molecules of one tile of the grid (a block's worth of threads): thread gtid
 // of the whole grid.  cur: current half of the molecule arrays; step: the time level of the
 // forces; ext_now: the largest atom-to-COM distance; the next mapping's maxima are merged into
@@ -879,87 +1052,9 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
       hr_forces32<NA, ENERGY, MODEL, HS>(s, B, b, cur, t, a, 1 << ln.h, lig, nnb, m_first, live_item, Ca, wa, reach_at2, sw, slow, drift,
                                              fx, fy, fz, dv, e_at, e_cg, vir);
     } else {
-    // Eq. 1 for atom i against every listed neighbour (of this lane group's share); the next
-    // neighbour's index and centre are fetched while the current one is evaluated
     constexpr int SPLIT = atom_lanes(true, MODEL) / kGroup;
-    const int sub = lig / kGroup;
-    const bool own_pair = live_item && g < NA;  // lanes that evaluate pair forces
-    int m_n = 0;
-    auto C_n = Ca;
-    if (sub < nnb) {
-      m_n = m_first;
-      C_n = Q::com(b, cur, m_n);
-    }
-    for (int q = sub; q < nnb; q += SPLIT) {
-      const int m = m_n;
-      const auto Cb = C_n;
-      if (q + SPLIT < nnb) {
-        m_n = row[q + SPLIT];
-        C_n = Q::com(b, cur, m_n);
-      }
-      const auto R = Q::dR(B, Ca, Cb);
-      const real r2 = pair_r2(R.x, R.y, R.z);
-      const real wab = hs ? (real)0.5 * (wa + Q::w(Cb)) : wa * Q::w(Cb);
-      if (own_pair && wab > (real)0 && r2 < reach_at2) {
-        const real px = R.x + (real)oi.x, py = R.y + (real)oi.y, pz = R.z + (real)oi.z;
-        typename P::off_t oj[NA];
-#pragma unroll
-        for (int j = 0; j < NA; ++j) oj[j] = Q::template off<NA>(b, cur, m, j);
-#pragma unroll
-        for (int j = 0; j < NA; ++j) {
-          const real dx = px - (real)oj[j].x, dy = py - (real)oj[j].y, dz = pz - (real)oj[j].z;
-          const real d2 = dx * dx + dy * dy + dz * dz;
-          if (d2 < rc_at2) {
-            real fr;
-            if (MODEL == 0) {
-              const real ir2 = Q::rcp_(d2);
-              const real sr2 = sig2 * ir2;
-              const real sr6 = sr2 * sr2 * sr2;
-              fr = (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2 * wab;
-              if (ENERGY) e_at += 0.5 * (double)wab * (double)((real)4 * eps * (sr6 * sr6 - sr6) + eps);
-              if (drift) dv += (real)4 * eps * (sr6 * sr6 - sr6) + eps;
-            } else {
-              // LJ (c12 r^-12 - c6 r^-6, shifted) + reaction field q_i q_j f (1/r + k_rf r^2 - c_rf);
-              // the LJ term only for partner sites that have one with some site (water: O)
-              const real ir = Q::rsqrt_(d2);
-              const real ir2 = ir * ir;
-              real flj = 0, vlj = 0;
-              if ((s.lj_cols >> j) & 1) {
-                const real ir6 = ir2 * ir2 * ir2;
-                flj = ((real)12 * c12r[j] * ir6 - (real)6 * c6r[j]) * ir6 * ir2;
-                if (ENERGY || drift) vlj = (c12r[j] * ir6 - c6r[j]) * ir6;
-              }
-              fr = (flj + qqr[j] * (ir2 * ir - krf2)) * wab;
-              if (ENERGY)
-                e_at += 0.5 * (double)wab *
-                        ((double)vlj + s.vsh[gg0][j] + (double)qqr[j] * ((double)ir + s.krf * (double)d2 - s.crf));
-              if (drift)
-                dv += vlj + par<real>(s.vsh[gg0][j], s.f.vsh[gg0][j]) +
-                      qqr[j] * (ir + par<real>(s.krf, s.f.krf) * d2 - par<real>(s.crf, s.f.crf));
-            }
-            fx += fr * dx;
-            fy += fr * dy;
-            fz += fr * dz;
-            if (ENERGY) vir += 0.5 * (double)(fr * d2);
-          }
-        }
-      }
-      if (own_pair && wab < (real)1 && r2 < rc_cg2 && slow) {
-        const real r = Q::sqrt_(r2);
-        real V = 0;
-        const real F = s.cg_mode ? (real)b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, inv_dr, &V);
-        const real fw = ((real)1 - wab) * F;
-        const real c = Q::div_(fw * sw, r);
-        fx += frac_g * c * R.x;
-        fy += frac_g * c * R.y;
-        fz += frac_g * c * R.z;
-        if (ENERGY && g == 0) {
-          e_cg += 0.5 * (double)(((real)1 - wab) * V);
-          vir += 0.5 * (double)(Q::div_(fw, r) * r2);
-        }
-        if (drift && g == 0) dv -= sw * V;
-      }
-    }
+    hr_forces64<NA, ENERGY, MODEL, HS, SPLIT>(s, B, b, cur, t, a, g, lig / kGroup, nnb, live_item, row, Ca, oi, frac_g, reach_at2,
+                                              sw, slow, drift, c12r, c6r, qqr, fx, fy, fz, dv, e_at, e_cg, vir);
     if (SPLIT > 1) {  // the groups' shares of the force (energies are summed per warp)
       const unsigned mk = SPLIT == 2 ? 0xFFu << (lane & 24) : 0xFFFFu << (lane & 16);
 #pragma unroll
@@ -980,29 +1075,51 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
     // coarse-grained item (l_a = 0, so w_ab = 0): neighbour list split over the group
     if (live && g == 0 && wa != (real)0) set_error(b.ctrl, ADRESS_ERR_STATE, a);
     real Fx = 0, Fy = 0, Fz = 0;
-    auto C_n = Ca;
     const int nnb_cg = slow ? nnb : 0;  // no CG force at inner levels of multiple time stepping
-    // centres of the next two neighbours in flight (long lists: the water-like fluid)
-    if (lig < nnb_cg) C_n = Q::com(b, cur, m_first);
-    auto C_n2 = Ca;
-    if (lig + GC < nnb_cg) C_n2 = Q::com(b, cur, row[lig + GC]);
+    auto pair_cg = [&](int q, const typename Q::V3& R, real r2) {
+      // (the FP64 path has 1/r at hand and divides by multiplying)
+      const real ir = P::fp64 ? Q::rsqrt_(r2) : (real)0, r = P::fp64 ? r2 * ir : (real)Prec<P32>::sqrt_((float)r2);
+      real V = 0;
+      const real F = s.cg_mode ? (real)b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, inv_dr, &V);
+      const real c = P::fp64 ? F * ir : Q::div_(F, r);
+      Fx += c * R.x;
+      Fy += c * R.y;
+      Fz += c * R.z;
+      if (ENERGY) {
+        e_cg += 0.5 * (double)V;
+        vir += 0.5 * (double)(c * r2);
+      }
+    };
+    // centres of the next two neighbours in flight (long lists: the water-like fluid); the FP64
+    // path tests the fixed-point ones in FP32 with a margin first (see hr_forces64)
+    const int4* cfx = b.com_fx[cur];
+    const int4 Cf = P::fp64 ? cfx[a] : (const int4&)Ca;
+    const float rcgf = P::fp64 ? s.f.rc_cg2 * 1.0001f : s.f.rc_cg2;
+    int m_n = m_first, m_n2 = 0;
+    int4 C_n = Cf, C_n2 = Cf;
+    if (lig < nnb_cg) C_n = cfx[m_n];
+    if (lig + GC < nnb_cg) {
+      m_n2 = row[lig + GC];
+      C_n2 = cfx[m_n2];
+    }
     for (int q = lig; q < nnb_cg; q += GC) {
-      const auto Cb = C_n;
+      const int m = m_n;
+      const int4 Cb = C_n;
+      m_n = m_n2;
       C_n = C_n2;
-      if (q + 2 * GC < nnb_cg) C_n2 = Q::com(b, cur, row[q + 2 * GC]);
-      const auto R = Q::dR(B, Ca, Cb);
-      const real r2 = pair_r2(R.x, R.y, R.z);
-      if (r2 < rc_cg2) {
-        const real r = Q::sqrt_(r2);
-        real V = 0;
-        const real F = s.cg_mode ? (real)b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, inv_dr, &V);
-        const real c = Q::div_(F, r);
-        Fx += c * R.x;
-        Fy += c * R.y;
-        Fz += c * R.z;
-        if (ENERGY) {
-          e_cg += 0.5 * (double)V;
-          vir += 0.5 * (double)(c * r2);
+      if (q + 2 * GC < nnb_cg) {
+        m_n2 = row[q + 2 * GC];
+        C_n2 = cfx[m_n2];
+      }
+      const auto Rf = Prec<P32>::dR(B, Cf, Cb);
+      const float r2f = pair_r2(Rf.x, Rf.y, Rf.z);
+      if (r2f < rcgf) {
+        if constexpr (P::fp64) {
+          const auto R = Q::dR(B, Ca, Q::com(b, cur, m));
+          const real r2 = pair_r2(R.x, R.y, R.z);
+          if (r2 < rc_cg2) pair_cg(q, R, r2);
+        } else {
+          pair_cg(q, Rf, r2f);
         }
       }
     }
