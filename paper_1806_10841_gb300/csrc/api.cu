@@ -61,9 +61,11 @@ struct adress_ctx {
   long long pcap_alloc = 0, pcap_limit = 0;
   double cg_dr = 0.0;  // node spacing of the CG table
   // radial distribution function scratch
-  double* rdf_com = nullptr;
+  RdfArgs rdf{};
   unsigned long long* rdf_counts = nullptr;
-  size_t rdf_cap = 0;
+  RdfGrid* rdf_grids = nullptr;
+  double* rdf_com = nullptr;
+  size_t rdf_cap = 0, rdf_cell_cap = 0;
   MlpDevArgs mlp_args() const { return MlpDevArgs{mlp_P, mlp_W1p, mlp_W2p, mlp_W2Tp, mlp_norm}; }
 };
 
@@ -1076,15 +1078,59 @@ adress_status adress_rdf(adress_handle h, int32_t nbins, double dr, int64_t* cou
     for (int d = 0; d < 3; ++d)
       if (nbins * dr > B.halfL[d]) return fail(h, ADRESS_ERR_ARG, "nbins * dr exceeds half a box edge");
   const Sys& s = h->sys;
-  if (!h->rdf_com) CUDA_OR_FAIL(h, dalloc(h, &h->rdf_com, (size_t)3 * s.M));
+  RdfArgs& q = h->rdf;
+  if (!h->rdf_com) {
+    CUDA_OR_FAIL(h, dalloc(h, &h->rdf_grids, s.nbox));
+    CUDA_OR_FAIL(h, dalloc(h, &q.cell, s.M));
+    CUDA_OR_FAIL(h, dalloc(h, &q.slot, s.M));
+    CUDA_OR_FAIL(h, dalloc(h, &q.fx, s.M));
+    CUDA_OR_FAIL(h, dalloc(h, &q.sorted, s.M));
+    CUDA_OR_FAIL(h, dalloc(h, &h->rdf_com, (size_t)3 * s.M));
+  }
+  // cells at least the range wide and, on average, at least one molecule each
+  const double range = nbins * dr;
+  std::vector<RdfGrid> grids(s.nbox);
+  long long ncell = 0;
+  double lmax = 0.0;
+  for (int k = 0; k < s.nbox; ++k) {
+    const Box& B = h->boxes[k];
+    // (and the fixed-point centres' rounding wider, so that molecules two cells apart are out of range)
+    const double edge = std::max(range * (1.0 + 1e-9) + 4.0 * std::max(B.L[0], std::max(B.L[1], B.L[2])) / 4294967296.0,
+                                 cbrt(B.L[0] * B.L[1] * B.L[2] / B.nmol));
+    RdfGrid& G = grids[k];
+    for (int d = 0; d < 3; ++d) {
+      G.nc[d] = std::max(1, (int)floor(B.L[d] / edge));
+      lmax = std::max(lmax, B.L[d]);
+    }
+    G.cell0 = (int)ncell;
+    ncell += (long long)G.nc[0] * G.nc[1] * G.nc[2];
+  }
   const size_t n = (size_t)s.nbox * nbins;
   if (h->rdf_cap < n) {
     CUDA_OR_FAIL(h, realloc_owned(h, &h->rdf_counts, n));
     h->rdf_cap = n;
   }
+  if (h->rdf_cell_cap < (size_t)ncell) {
+    CUDA_OR_FAIL(h, realloc_owned(h, &q.count, (size_t)ncell));
+    CUDA_OR_FAIL(h, realloc_owned(h, &q.start, (size_t)ncell + 1));
+    h->rdf_cell_cap = (size_t)ncell;
+  }
+  q.grids = h->rdf_grids;
+  q.com = h->rdf_com;
+  q.counts = h->rdf_counts;
+  q.ncell = (int)ncell;
+  q.nbins = nbins;
+  q.dr = dr;
+  q.inv_dr = (float)(1.0 / dr);
+  // a distance's FP32 error: 2^-32 L per fixed-point coordinate, some 1e-6 of the range in float
+  // arithmetic; twice the sum, in bins
+  const double err = 2.0 * (4.0 * lmax / 4294967296.0 + 1e-6 * range);
+  q.eps = (float)std::min(1.0, err / dr);
+  q.lim2 = (float)((range + err) * (range + err) * (1.0 + 1e-6));
+  CUDA_OR_FAIL(h, cudaMemcpyAsync(h->rdf_grids, grids.data(), sizeof(RdfGrid) * s.nbox, cudaMemcpyHostToDevice, h->stream));
   CUDA_OR_FAIL(h, cudaMemsetAsync(h->rdf_counts, 0, sizeof(unsigned long long) * n, h->stream));
   CUDA_OR_FAIL(h, launch_export_com(s, h->buf, h->precision, h->rdf_com, nullptr, h->stream));
-  CUDA_OR_FAIL(h, launch_rdf(s, h->buf, h->rdf_com, nbins, dr, h->rdf_counts, h->stream));
+  CUDA_OR_FAIL(h, launch_rdf(s, h->buf, q, h->stream));
   CUDA_OR_FAIL(h, cudaMemcpyAsync(counts, h->rdf_counts, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, h->stream));
   CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
   return ADRESS_OK;

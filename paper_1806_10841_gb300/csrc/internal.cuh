@@ -319,9 +319,22 @@ cudaError_t launch_kinetic(const Sys& s, const Bufs& b, cudaStream_t st);
 cudaError_t launch_density(const Sys& s, const Bufs& b, int precision, cudaStream_t st);
 cudaError_t launch_tf_update(const Sys& s, const Bufs& b, double alpha, cudaStream_t st);
 cudaError_t launch_export_com(const Sys& s, const Bufs& b, int precision, double* com, double* w, cudaStream_t st);
-// COM pair-distance histogram of the centres com [3][M] into counts [nbox][nbins] (added).
-cudaError_t launch_rdf(const Sys& s, const Bufs& b, const double* com, int nbins, double dr,
-                       unsigned long long* counts, cudaStream_t st);
+// COM pair-distance histogram (k_rdf): cell grids of the boxes, scratch and parameters.
+struct RdfGrid {
+  int nc[3], cell0;
+};
+struct RdfArgs {
+  const RdfGrid* grids;  // [nbox]
+  const double* com;     // [3][M]
+  int *cell, *slot;      // [M]
+  int4 *fx, *sorted;     // [M] fixed-point centre + molecule, in molecule and in cell order
+  int *count, *start;    // [ncell], [ncell + 1]
+  unsigned long long* counts;  // [nbox][nbins], added to
+  int ncell, nbins;
+  double dr;
+  float inv_dr, lim2, eps;  // 1 / dr, squared range with its margin, error of a distance in bins
+};
+cudaError_t launch_rdf(const Sys& s, const Bufs& b, const RdfArgs& q, cudaStream_t st);
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
