@@ -42,8 +42,6 @@ struct adress_ctx {
   float* smp_target = nullptr;
   int* smp_ids = nullptr;
   long long smp_n = 0, smp_cap = 0;
-  float *bat_feat = nullptr, *bat_target = nullptr;
-  long long bat_cap = 0;
   int* mlp_counts = nullptr;  // [M + 1]
   int* mlp_offs = nullptr;    // [M + 1]
   // boxes (one per replica) and the cell arrays sized for ncell_cap cells
@@ -1588,7 +1586,7 @@ adress_status adress_mlp_loss_grad(adress_handle h, const float* feat, const flo
   if (!h->mlp_ready) return fail(h, ADRESS_ERR_STATE, "no network parameters set");
   adress_status st = mlp_part_for(h, n);
   if (st != ADRESS_OK) return st;
-  CUDA_OR_FAIL(h, mlp_grad(h->mlp_args(), feat, target, n, n, h->mlp_part, h->mlp_grad, nullptr, h->stream));
+  CUDA_OR_FAIL(h, mlp_grad(h->mlp_args(), feat, target, n, h->mlp_part, h->mlp_grad, h->stream));
   CUDA_OR_FAIL(h, cudaMemcpyAsync(grad, h->mlp_grad, sizeof(float) * (kMlpNPar + 1), cudaMemcpyDeviceToHost, h->stream));
   CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
   return ADRESS_OK;
@@ -1614,22 +1612,13 @@ adress_status adress_mlp_train(adress_handle h, int32_t epochs, int32_t batch, f
   if (h->smp_n < batch) return fail(h, ADRESS_ERR_STATE, "fewer samples than one batch");
   adress_status st = mlp_part_for(h, batch);
   if (st != ADRESS_OK) return st;
-  if (h->bat_cap < batch) {
-    CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
-    CUDA_OR_FAIL(h, realloc_owned(h, &h->bat_feat, (size_t)batch * 9));
-    CUDA_OR_FAIL(h, realloc_owned(h, &h->bat_target, (size_t)batch));
-    h->bat_cap = batch;
-  }
   const long long n = h->smp_n, nb = n / batch, stride = coprime_stride(n);
   CUDA_OR_FAIL(h, cudaMemsetAsync(h->mlp_loss, 0, sizeof(float) * epochs, h->stream));
   for (int e = 0; e < epochs; ++e)
     for (long long bi = 0; bi < nb; ++bi) {
-      CUDA_OR_FAIL(h, mlp_gather(h->smp_feat, h->smp_target, n, (e * nb + bi) * batch, batch, stride, h->bat_feat,
-                                 h->bat_target, h->stream));
-      CUDA_OR_FAIL(h, mlp_grad(h->mlp_args(), h->bat_feat, h->bat_target, batch, batch, h->mlp_part, h->mlp_grad,
-                               h->mlp_loss + e, h->stream));
-      CUDA_OR_FAIL(h, mlp_adam(h->mlp_args(), h->mlp_mom, h->mlp_vel, h->mlp_grad, lr, ++h->mlp_step, h->stream));
-      CUDA_OR_FAIL(h, mlp_pack(h->mlp_args(), h->stream));
+      CUDA_OR_FAIL(h, mlp_train_batch(h->mlp_args(), h->smp_feat, h->smp_target, batch,
+                                      SampleOrder{n, (e * nb + bi) * batch, stride}, h->mlp_part, h->mlp_mom, h->mlp_vel,
+                                      h->mlp_loss + e, lr, ++h->mlp_step, h->stream));
     }
   std::vector<float> acc(epochs);
   CUDA_OR_FAIL(h, cudaMemcpyAsync(acc.data(), h->mlp_loss, sizeof(float) * epochs, cudaMemcpyDeviceToHost, h->stream));

@@ -339,10 +339,15 @@ cudaError_t launch_rdf(const Sys& s, const Bufs& b, const RdfArgs& q, cudaStream
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 cudaError_t mlp_forward(const MlpDevArgs& a, const float* feat, long long n, float* y, cudaStream_t st);
-cudaError_t mlp_grad(const MlpDevArgs& a, const float* feat, const float* target, long long n, long long n_total,
-                     float* part, float* grad, float* loss_acc, cudaStream_t st);
-cudaError_t mlp_adam(const MlpDevArgs& a, float* mom, float* vel, const float* grad, float lr, int step,
+// Sample i of a batch: row (start + i) stride mod of.
+struct SampleOrder {
+  long long of, start, stride;
+};
+cudaError_t mlp_grad(const MlpDevArgs& a, const float* feat, const float* target, long long n, float* part, float* grad,
                      cudaStream_t st);
+// Gradient of one batch of n samples and the optimiser step `step` with it.
+cudaError_t mlp_train_batch(const MlpDevArgs& a, const float* feat, const float* target, long long n, SampleOrder order,
+                            float* part, float* mom, float* vel, float* loss_acc, float lr, int step, cudaStream_t st);
 cudaError_t mlp_pack(const MlpDevArgs& a, cudaStream_t st);
 cudaError_t mlp_collect(const Sys& s, const Bufs& b, int pass, const int* offs, long long cap, long long base,
                         float* feat, float* target, int* ids, int* counts, cudaStream_t st);
@@ -353,8 +358,6 @@ cudaError_t mlp_pairs(const Sys& s, const Bufs& b, const MlpDevArgs& a, float* f
 cudaError_t cg_fit(const float* feat, const float* target, long long n, double h, int nb, int n_min, int cg_n,
                    double dr, double rc, unsigned long long* acc, unsigned* cnt, double* F, double* V, int* npop,
                    cudaStream_t st);
-cudaError_t mlp_gather(const float* feat, const float* target, long long n, long long start, long long cnt,
-                       long long stride, float* feat_out, float* target_out, cudaStream_t st);
 
 // Record the message returned by adress_last_error(NULL) and return the status.
 adress_status set_global_error(adress_status s, const std::string& msg);

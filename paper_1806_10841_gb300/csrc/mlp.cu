@@ -338,10 +338,13 @@ __global__ void __launch_bounds__(128) k_mlp_forward(MlpDev m, const float* __re
 
 // ---------------- loss and gradient of one block of 64 samples ---------------------------
 // Writes the block's partial gradient (sum over its samples of dL/dparam with
-// L = (1/n_total) sum (y - t/out_scale)^2) and loss partial to part[blockIdx.x].
+// L = (1/n) sum (y - t/out_scale)^2) and loss partial to part[blockIdx.x].  Sample i of the n is
+// row (order.start + i) order.stride mod order.of of the arrays: a training batch is gathered on
+// the way in.
 __global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float* __restrict__ feat,
-                                                  const float* __restrict__ target, long long n, long long n_total,
+                                                  const float* __restrict__ target, long long n, SampleOrder order,
                                                   float* __restrict__ part) {
+  __shared__ long long srow[4][16];  // the tiles' rows
   __shared__ float ftile[4][16 * kIn];
   __shared__ __nv_bfloat16 sd2[64][kH + 8];  // delta of layer 2 [sample][out]
   __shared__ __nv_bfloat16 sh1[64][kH + 8];  // h1 [sample][in]
@@ -352,9 +355,14 @@ __global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float* __restr
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tg = lane & 3;
   const long long base = ((long long)blockIdx.x * 4 + w) * 16;
   const float inv_scale = 1.0f / m.norm[2 * kIn];
+  if (lane < 16)
+    srow[w][lane] = base + lane < n ? (long long)(((unsigned long long)(order.start + base + lane) * (unsigned long long)order.stride) %
+                                                  (unsigned long long)order.of)
+                                    : -1;
+  __syncwarp();
   for (int e = lane; e < 16 * kIn; e += 32) {
-    const long long s = base + e / kIn;
-    ftile[w][e] = s < n ? feat[s * kIn + e % kIn] : 0.f;
+    const long long s = srow[w][e / kIn];
+    ftile[w][e] = s >= 0 ? feat[s * kIn + e % kIn] : 0.f;
   }
   __syncwarp();
   const MlpView mv = view_of(m);
@@ -364,9 +372,9 @@ __global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float* __restr
   float yg, yg8;
   tile_forward(mv, ax, T, yg, yg8);
   const bool vg = base + g < n, vg8 = base + g + 8 < n;
-  const float rg = vg ? yg - target[base + g] * inv_scale : 0.f;
-  const float rg8 = vg8 ? yg8 - target[base + g + 8] * inv_scale : 0.f;
-  const float dyg = 2.f * rg / (float)n_total, dyg8 = 2.f * rg8 / (float)n_total;
+  const float rg = vg ? yg - target[srow[w][g]] * inv_scale : 0.f;
+  const float rg8 = vg8 ? yg8 - target[srow[w][g + 8]] * inv_scale : 0.f;
+  const float dyg = 2.f * rg / (float)n, dyg8 = 2.f * rg8 / (float)n;
   // layer 2 deltas, bias / w3 partials, and stores for the weight-gradient products
   const float* w3 = m.P + ow3;
   float pb2[8][2], pw3[8][2];
@@ -546,26 +554,58 @@ __global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float* __restr
 }
 
 // Fixed-order sum of the block partials: grad [kNPar + 1] (last entry: sum of squared
-// residuals, also added to *loss_acc when given).
-__global__ void k_mlp_grad_reduce(const float* part, int nblk, float* grad, float* loss_acc) {
+// residuals).
+__global__ void k_mlp_grad_reduce(const float* part, int nblk, float* grad) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p > kNPar) return;
   float acc = 0.f;
   for (int b = 0; b < nblk; ++b) acc += part[(size_t)b * kGradStride + p];
   grad[p] = acc;
-  if (p == kNPar && loss_acc) *loss_acc += acc;
 }
 
-// Adam on the FP32 master parameters.
-__global__ void k_mlp_adam(float* P, float* mom, float* vel, const float* grad, float lr, float b1c, float b2c) {
+// One optimiser step: the fixed-order sum of the block partials (as k_mlp_grad_reduce, sixteen
+// loads in flight), Adam on the FP32 master parameter, and its bfloat16 operand copies.  As four
+// kernels (reduction, Adam, packing, and the gather of the next batch) a batch of 4096 spent most
+// of its 45 us in launches and their gaps.
+__global__ void __launch_bounds__(128) k_mlp_update(const float* __restrict__ part, int nblk, float* __restrict__ P,
+                                                    float* __restrict__ mom, float* __restrict__ vel, float* loss_acc, float lr,
+                                                    float b1c, float b2c, __nv_bfloat16* __restrict__ W1,
+                                                    __nv_bfloat16* __restrict__ W2, __nv_bfloat16* __restrict__ W2T) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kNPar) return;
-  const float gr = grad[p];
-  const float mo = 0.9f * mom[p] + 0.1f * gr;
-  const float ve = 0.999f * vel[p] + 0.001f * gr * gr;
+  if (p > kNPar) return;
+  float mo = 0.f, ve = 0.f, old = 0.f;
+  if (p < kNPar) {
+    mo = mom[p];
+    ve = vel[p];
+    old = P[p];
+  }
+  float gr = 0.f;
+  int b = 0;
+  for (; b + 16 <= nblk; b += 16) {
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = part[(size_t)(b + e) * kGradStride + p];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) gr += v[e];
+  }
+  for (; b < nblk; ++b) gr += part[(size_t)b * kGradStride + p];
+  if (p == kNPar) {
+    *loss_acc += gr;
+    return;
+  }
+  mo = 0.9f * mo + 0.1f * gr;
+  ve = 0.999f * ve + 0.001f * gr * gr;
   mom[p] = mo;
   vel[p] = ve;
-  P[p] -= lr * (mo / b1c) / (sqrtf(ve / b2c) + 1e-8f);
+  const float v = old - lr * (mo / b1c) / (sqrtf(ve / b2c) + 1e-8f);
+  P[p] = v;
+  if (p < ob1) {
+    W1[(p / kIn) * 16 + p % kIn] = __float2bfloat16_rn(v);
+  } else if (p >= oW2 && p < ob2) {
+    const int r = (p - oW2) / kH, k = (p - oW2) % kH;
+    W2[r * kH + k] = __float2bfloat16_rn(v);
+    W2T[k * kH + r] = __float2bfloat16_rn(v);
+  }
 }
 
 // BF16 operand copies of W1 (K padded to 16), W2 and W2 transposed, from the master.
@@ -910,18 +950,6 @@ __global__ void __launch_bounds__(128, 8) k_mlp_eval(MlpDev m, const unsigned* _
   }
 }
 
-// Training batch `cnt` samples starting at `start` of a fixed permutation of the n
-// samples: sample (start + i) * stride mod n (stride coprime with n).
-__global__ void k_mlp_gather(const float* feat, const float* target, long long n, long long start, long long cnt,
-                             long long stride, float* fo, float* to) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= cnt) return;
-  const long long src = (long long)(((unsigned long long)(start + i) * (unsigned long long)stride) % (unsigned long long)n);
-#pragma unroll
-  for (int k = 0; k < kIn; ++k) fo[i * kIn + k] = feat[src * kIn + k];
-  to[i] = target[src];
-}
-
 // ---------------- force-matched CG table ---------------------------------------------------
 // The CG force of Eq. 1 acts between centres of mass (Sec. "Force interpolation").  Its
 // force-matched table is the mean, per distance bin, of the atomistic pair force projected on
@@ -1050,12 +1078,6 @@ cudaError_t cg_fit(const float* feat, const float* target, long long n, double h
 
 // ---------------- launchers ------------------------------------------------------------
 
-cudaError_t mlp_gather(const float* feat, const float* target, long long n, long long start, long long cnt,
-                       long long stride, float* fo, float* to, cudaStream_t st) {
-  k_mlp_gather<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(feat, target, n, start, cnt, stride, fo, to);
-  return cudaGetLastError();
-}
-
 cudaError_t mlp_forward(const MlpDevArgs& a, const float* feat, long long n, float* y, cudaStream_t st) {
   const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
   const long long tiles = (n + 15) / 16;
@@ -1063,19 +1085,23 @@ cudaError_t mlp_forward(const MlpDevArgs& a, const float* feat, long long n, flo
   return cudaGetLastError();
 }
 
-cudaError_t mlp_grad(const MlpDevArgs& a, const float* feat, const float* target, long long n, long long n_total,
-                     float* part, float* grad, float* loss_acc, cudaStream_t st) {
+cudaError_t mlp_grad(const MlpDevArgs& a, const float* feat, const float* target, long long n, float* part, float* grad,
+                     cudaStream_t st) {
   const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
   const int nblk = (int)((n + 63) / 64);
-  k_mlp_grad<<<nblk, 128, 0, st>>>(m, feat, target, n, n_total, part);
-  k_mlp_grad_reduce<<<(kNPar + 1 + 255) / 256, 256, 0, st>>>(part, nblk, grad, loss_acc);
+  k_mlp_grad<<<nblk, 128, 0, st>>>(m, feat, target, n, SampleOrder{n, 0, 1}, part);
+  k_mlp_grad_reduce<<<(kNPar + 1 + 255) / 256, 256, 0, st>>>(part, nblk, grad);
   return cudaGetLastError();
 }
 
-cudaError_t mlp_adam(const MlpDevArgs& a, float* mom, float* vel, const float* grad, float lr, int step,
-                     cudaStream_t st) {
+cudaError_t mlp_train_batch(const MlpDevArgs& a, const float* feat, const float* target, long long n, SampleOrder order,
+                            float* part, float* mom, float* vel, float* loss_acc, float lr, int step, cudaStream_t st) {
+  const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
+  const int nblk = (int)((n + 63) / 64);
+  k_mlp_grad<<<nblk, 128, 0, st>>>(m, feat, target, n, order, part);
   const float b1c = 1.f - powf(0.9f, (float)step), b2c = 1.f - powf(0.999f, (float)step);
-  k_mlp_adam<<<(kNPar + 255) / 256, 256, 0, st>>>((float*)a.P, mom, vel, grad, lr, b1c, b2c);
+  k_mlp_update<<<(kNPar + 1 + 127) / 128, 128, 0, st>>>(part, nblk, (float*)a.P, mom, vel, loss_acc, lr, b1c, b2c,
+                                                        (__nv_bfloat16*)a.W1p, (__nv_bfloat16*)a.W2p, (__nv_bfloat16*)a.W2Tp);
   return cudaGetLastError();
 }
 
