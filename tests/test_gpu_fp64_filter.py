@@ -1,5 +1,6 @@
 """The FP64 path's FP32 pre-test of pairs: centres placed within 1e-11 .. 1e-5 of the cutoffs, on
 either side, in boxes of very different size, must be decided as FP64 decides them."""
+import numpy as np
 import pytest
 
 import oracle
