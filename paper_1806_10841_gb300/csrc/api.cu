@@ -637,10 +637,8 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   Bufs& b = h->buf;
   const int M = s.M, N = s.N;
   {
-    int warps = 0;
-    for (int blk = 32; blk <= kMaxForceBlock; blk *= 2)
-      warps = std::max(warps, ceil_div((long long)M * step_lanes(s), blk) * (blk / 32));
-    h->nparts = std::max(warps, ceil_div(N, 256));
+    // records of the force kernel (smallest blocks) and of the kinetic energy
+    h->nparts = std::max(ceil_div((long long)M * step_lanes(s), 32), ceil_div(N, 256));
   }
   const int ntf = std::max(1, nbox * s.tf_n);
   cudaError_t e = cudaSuccess;
@@ -689,6 +687,9 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
     b.fec64 = f64;
     b.fec32 = f32;
   }
+  float4* log_tab = nullptr;
+  A(log_tab, 128);
+  b.log_tab = log_tab;
   A(b.part, (size_t)h->nparts * 4);
   A(b.result, 8);
   A(b.hist, ntf);
@@ -723,6 +724,12 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
 
   std::vector<float2> fv(s.cg_n + 1);
   for (int k = 0; k <= s.cg_n; ++k) fv[k] = make_float2((float)c->cg_F[k], (float)c->cg_V[k]);
+  // reciprocals of the 128 intervals of [1, 2) rounded to nine bits, and their -log
+  float4 logs[128];
+  for (int k = 0; k < 128; ++k) {
+    const double c = nearbyint(512.0 / (1.0 + (k + 0.5) / 128.0)) / 512.0, l = -log(c);
+    logs[k] = make_float4((float)c, (float)l, (float)(l - (double)(float)l), 0.f);
+  }
   std::vector<double> tf(ntf, 0.0);
   std::vector<float> tff(ntf, 0.f);
   std::vector<float> fecf(c->fec, c->fec + c->fec_n);  // staged until the stream synchronises
@@ -741,6 +748,7 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   } while (0)
   H2D(cgF, c->cg_F, sizeof(double) * (s.cg_n + 1));
   H2D(cgV, c->cg_V, sizeof(double) * (s.cg_n + 1));
+  H2D(log_tab, logs, sizeof(logs));
   H2D(cgFV, fv.data(), sizeof(float2) * (s.cg_n + 1));
   H2D(b.tf64, tf.data(), sizeof(double) * tf.size());
   H2D(b.tf32, tff.data(), sizeof(float) * tff.size());
@@ -818,42 +826,58 @@ static adress_status read_ctrl(adress_handle h, Ctrl* c) {
   return ADRESS_OK;
 }
 
-// Map positions, rebuild lists; grow the capacity and redo while a list overflows.
-static adress_status build_lists_sync(adress_handle h) {
-  for (int attempt = 0; attempt < 4; ++attempt) {
-    CUDA_OR_FAIL(h, launch_map(h->sys, h->buf, h->precision, 0, h->stream));
-    CUDA_OR_FAIL(h, launch_lists(h->sys, h->buf, DecideArgs{1, 0, 1}, h->stream));
-    CUDA_OR_FAIL(h, launch_max_nn(h->sys, h->buf, h->stream));
-    Ctrl c;
-    adress_status st = read_ctrl(h, &c);
-    if (st != ADRESS_OK) return st;
-    if (c.dead) CUDA_OR_FAIL(h, revive(h));
-    if (c.err == ADRESS_ERR_LIST_OVERFLOW || c.max_nn > h->sys.cap) {
-      int cap = ((int)ceil(c.max_nn * 1.5) + 8 + 3) & ~3;
-      cap = std::min(cap, h->sys.M - 1);
-      void* old = h->buf.nbr;
-      int* nbr = nullptr;
-      CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
-      CUDA_OR_FAIL(h, dalloc(h, &nbr, (size_t)cap * h->sys.M));
-      h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), old));
-      cudaFree(old);
-      h->buf.nbr = nbr;
-      h->sys.cap = cap;
-      if (h->buf.fpair) {
-        CUDA_OR_FAIL(h, realloc_owned(h, &h->buf.fpair, (size_t)cap * h->sys.M));
-        CUDA_OR_FAIL(h, alloc_pair_buffers(h));
-      }
-      free_graphs(h);
-      int zero = 0;
-      CUDA_OR_FAIL(h, cudaMemcpyAsync(&h->buf.ctrl->err, &zero, sizeof(int), cudaMemcpyHostToDevice, h->stream));
-      continue;
+// Map positions and build the lists.
+static cudaError_t launch_build(adress_handle h) {
+  const cudaError_t e = launch_map(h->sys, h->buf, h->precision, 0, h->stream);
+  return e == cudaSuccess ? launch_lists(h->sys, h->buf, DecideArgs{1, 0, 1}, h->stream) : e;
+}
+
+// What the control block says of the build (and what was launched after it): *redo when a list
+// overflowed (the capacity is grown), else the status.
+static adress_status judge_build(adress_handle h, const Ctrl& c, bool* redo) {
+  *redo = false;
+  if (c.dead) CUDA_OR_FAIL(h, revive(h));
+  if (c.lists_err == ADRESS_ERR_LIST_OVERFLOW) {
+    // every count was cut at the capacity
+    int cap = ((int)ceil(h->sys.cap * 1.5) + 8 + 3) & ~3;
+    cap = std::min(cap, h->sys.M - 1);
+    void* old = h->buf.nbr;
+    int* nbr = nullptr;
+    CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
+    CUDA_OR_FAIL(h, dalloc(h, &nbr, (size_t)cap * h->sys.M));
+    h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), old));
+    cudaFree(old);
+    h->buf.nbr = nbr;
+    h->sys.cap = cap;
+    if (h->buf.fpair) {
+      CUDA_OR_FAIL(h, realloc_owned(h, &h->buf.fpair, (size_t)cap * h->sys.M));
+      CUDA_OR_FAIL(h, alloc_pair_buffers(h));
     }
-    if (c.err != 0) return fail(h, (adress_status)c.err, std::string("list build: ") +
-                                                          adress_status_string((adress_status)c.err));
-    h->lists_built = true;
+    free_graphs(h);
+    int zero = 0;
+    CUDA_OR_FAIL(h, cudaMemcpyAsync(&h->buf.ctrl->err, &zero, sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    *redo = true;
     return ADRESS_OK;
   }
-  return fail(h, ADRESS_ERR_LIST_OVERFLOW, "neighbour list capacity could not be grown enough");
+  if (c.lists_err != 0)
+    return fail(h, (adress_status)c.lists_err, std::string("list build: ") + adress_status_string((adress_status)c.lists_err));
+  h->lists_built = true;
+  return ADRESS_OK;
+}
+
+static constexpr int kBuildAttempts = 4;
+static const char* kGrowFailed = "neighbour list capacity could not be grown enough";
+
+static adress_status build_lists_sync(adress_handle h) {
+  for (int attempt = 0; attempt < kBuildAttempts; ++attempt) {
+    CUDA_OR_FAIL(h, launch_build(h));
+    Ctrl c;
+    adress_status st = read_ctrl(h, &c);
+    bool redo = false;
+    if (st == ADRESS_OK) st = judge_build(h, c, &redo);
+    if (!redo) return st;
+  }
+  return fail(h, ADRESS_ERR_LIST_OVERFLOW, kGrowFailed);
 }
 
 adress_status adress_build_lists(adress_handle h) {
@@ -862,20 +886,30 @@ adress_status adress_build_lists(adress_handle h) {
   return build_lists_sync(h);
 }
 
+// The forces are launched behind the lists without waiting for their verdict (an overflowing
+// build leaves shorter lists, all in bounds, and everything is done again), so that a call waits
+// for the GPU once.
 adress_status adress_compute_forces(adress_handle h, double* energies) {
   if (!h) return ADRESS_ERR_ARG;
   if (!h->bound) return fail(h, ADRESS_ERR_STATE, "no state bound");
-  adress_status st = build_lists_sync(h);
-  if (st != ADRESS_OK) return st;
-  if (h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
-  CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 0, energies != nullptr, h->stream));
-  if (energies) {
-    CUDA_OR_FAIL(h, launch_energy_reduce(h->sys, h->buf, force_warps(h->sys), 4, h->stream));
-    CUDA_OR_FAIL(h, cudaMemcpyAsync(energies, h->buf.result, 4 * sizeof(double), cudaMemcpyDeviceToHost,
-                                    h->stream));
-    CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
+  for (int attempt = 0; attempt < kBuildAttempts; ++attempt) {
+    CUDA_OR_FAIL(h, launch_build(h));
+    if (h->sys.cg_mode) CUDA_OR_FAIL(h, mlp_pairs(h->sys, h->buf, h->mlp_args(), h->buf.fpair, h->stream));
+    CUDA_OR_FAIL(h, launch_step(h->sys, h->buf, h->precision, 0, energies != nullptr, h->stream));
+    double sums[4];
+    if (energies) {
+      CUDA_OR_FAIL(h, launch_energy_reduce(h->buf, force_blocks(h->sys), h->stream));
+      CUDA_OR_FAIL(h, cudaMemcpyAsync(sums, h->buf.result, sizeof(sums), cudaMemcpyDeviceToHost, h->stream));
+    }
+    Ctrl c;
+    adress_status st = read_ctrl(h, &c);
+    bool redo = false;
+    if (st == ADRESS_OK) st = judge_build(h, c, &redo);
+    if (redo) continue;
+    if (st == ADRESS_OK && energies) memcpy(energies, sums, sizeof(sums));
+    return st;
   }
-  return ADRESS_OK;
+  return fail(h, ADRESS_ERR_LIST_OVERFLOW, kGrowFailed);
 }
 
 // Launch `nsteps` steps:

@@ -33,6 +33,7 @@ constexpr unsigned kBarrierPolls = 1u << 23;
 struct Ctrl {
   int err;                // first device error (adress_status), 0 = none
   int err_info;
+  int lists_err;          // the error word as the last decision or build left it
   int n_hr;               // high-resolution work items (first in `items`)
   int n_cg;
   long long step;         // time level of the state's forces
@@ -212,8 +213,9 @@ struct Bufs {
   float* tf32;
   const double* fec64;  // [fec_n] free-energy correction dDF/dl (energy interpolation)
   const float* fec32;
+  const float4* log_tab;  // [128] reciprocal c of an interval of [1, 2) and -log c as two floats
   // reductions
-  double* part;      // per-warp partials
+  double* part;      // per-block partials [][4]
   double* result;    // reduced results [8]
   unsigned long long* hist;  // density histogram [tf_n]
   long long* nsamples;
@@ -314,7 +316,7 @@ cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, c
 // Whether launch_run is the faster way to advance this system (tabulated CG force only).
 bool run_kernel_pays(const Sys& s);
 
-cudaError_t launch_energy_reduce(const Sys& s, const Bufs& b, int nparts, int nvals, cudaStream_t st);
+cudaError_t launch_energy_reduce(const Bufs& b, int nparts, cudaStream_t st);
 cudaError_t launch_kinetic(const Sys& s, const Bufs& b, cudaStream_t st);
 cudaError_t launch_density(const Sys& s, const Bufs& b, int precision, cudaStream_t st);
 cudaError_t launch_tf_update(const Sys& s, const Bufs& b, double alpha, cudaStream_t st);
@@ -374,9 +376,7 @@ inline int step_lanes(const Sys& s) {
   return !s.fp64 && s.nb_model == 1 ? 1 << s.step_lanes.h : atom_lanes(s.fp64, s.nb_model);
 }
 
-// Warps launched by the force kernel (one energy partial each).
-inline int force_warps(const Sys& s) {
-  return ceil_div((long long)s.M * step_lanes(s), s.force_block) * (s.force_block / 32);
-}
+// Blocks launched by the force kernel (one energy record each).
+inline int force_blocks(const Sys& s) { return ceil_div((long long)s.M * step_lanes(s), s.force_block); }
 
 }  // namespace adress

@@ -26,12 +26,13 @@ __device__ __forceinline__ void finish_mapping(const Bufs& b, const Decision& d,
   if (da.advance) c->step += 1;
   c->parity ^= 1;
   if (b.npair) *b.npair = 0u;
+  c->lists_err = __ldcg(&c->err);
 }
 
 // Decision only (a mapping outside a run: no lists are built for it).
 __global__ void __launch_bounds__(32) k_decide(const __grid_constant__ Sys s, Bufs b, DecideArgs da) {
   const Decision d = decide_rebuild(s, b.ctrl, 0, da.force);
-  finish_mapping(b, d, da);
+  if (!d.dead) finish_mapping(b, d, da);
 }
 
 // Decision and, when needed, the whole list build: 512-thread blocks, four per SM (32
@@ -43,9 +44,9 @@ constexpr int kListThreads = 512, kListBlocksPerSm = 4;
 __global__ void __launch_bounds__(kListThreads, kListBlocksPerSm) k_lists(const __grid_constant__ Sys s, const __grid_constant__ Bufs b,
                                                                         DecideArgs da) {
   Ctrl* c = b.ctrl;
-  if (grid_is_dead(c)) return;
   const int cur = c->parity ^ 1;
   const Decision d = decide_rebuild(s, c, 0, da.force);
+  if (d.dead) return;  // (the barrier left a timeout in lists_err)
   if (d.rebuild) {
     GridBarrier bar(c, &c->bar[0]);
     if (!rebuild_lists<kListThreads / 32>(s, b, cur, bar)) return;

@@ -54,6 +54,7 @@ struct GridBarrier {
         if (n >= kBarrierPolls) {
           dead = 1;
           set_error(c, ADRESS_ERR_TIMEOUT, (int)blockIdx.x);
+          atomicExch(&c->lists_err, ADRESS_ERR_TIMEOUT);
           atomicExch(&c->dead, 1);
           break;
         }
@@ -64,11 +65,6 @@ struct GridBarrier {
     return __syncthreads_or(dead) == 0;
   }
 };
-
-// Whether a barrier gave up earlier (every thread of the block gets the same answer).
-__device__ __forceinline__ bool grid_is_dead(Ctrl* c) {
-  return __syncthreads_or(threadIdx.x == 0 && __ldcg(&c->dead) != 0) != 0;
-}
 
 // True in warp 0 of the last block of the grid to call (each block's warp 0 calls once, after
 // its block's last read of what the caller then writes); nobody waits.
@@ -92,6 +88,7 @@ __device__ __forceinline__ bool last_to_arrive(Ctrl* c) {
 struct Decision {
   int rebuild;
   int too_wide;
+  int dead;  // a grid barrier gave up earlier: the block must leave
   float ext;
 };
 __device__ __forceinline__ Decision decide_rebuild(const Sys& s, Ctrl* c, int set, int force) {
@@ -100,13 +97,14 @@ __device__ __forceinline__ Decision decide_rebuild(const Sys& s, Ctrl* c, int se
   if (threadIdx.x < 32) {
     const unsigned me = __reduce_max_sync(0xffffffffu, __ldcg(&c->ext_slot[set][0][threadIdx.x]));
     const unsigned md2 = __reduce_max_sync(0xffffffffu, __ldcg(&c->ext_slot[set][1][threadIdx.x]));
-    const int host = __ldcg(&c->force_rebuild);
+    const int host = __ldcg(&c->force_rebuild), dead = __ldcg(&c->dead);
     if (threadIdx.x == 0) {
       sd.ext = sqrtf(__uint_as_float(me));
       const float md = sqrtf(__uint_as_float(md2));
       const double cut = fmax(s.rc_cg, s.rc_at + 2.0 * (double)sd.ext);
       sd.rebuild = force || host || (md > 0.5 * s.skin) || (cut + 2.0 * md > s.r_list);
       sd.too_wide = cut > s.r_list;
+      sd.dead = dead;
     }
   }
   __syncthreads();

@@ -32,24 +32,18 @@ __device__ __forceinline__ void block_partials(double (&v)[NV], double* part, in
   }
 }
 
-__global__ void __launch_bounds__(1024) k_reduce_parts(const double* part, int nparts, int nv,
-                                                       double* out) {
-  __shared__ double sm[32][8];
-  double acc[8];
-  for (int j = 0; j < nv; ++j) acc[j] = 0.0;
-  for (int p = threadIdx.x; p < nparts; p += blockDim.x)
-    for (int j = 0; j < nv; ++j) acc[j] += part[(size_t)p * nv + j];
-  for (int j = 0; j < nv; ++j)
-    for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-  if ((threadIdx.x & 31) == 0)
-    for (int j = 0; j < nv; ++j) sm[threadIdx.x >> 5][j] = acc[j];
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int j = 0; j < nv; ++j) {
-      double t = 0.0;
-      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += sm[q][j];
-      out[j] = t;
-    }
+// Sum of the partials [nparts][4], one block.
+__global__ void __launch_bounds__(1024) k_reduce_parts(const double4_32a* part, int nparts, double* out) {
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int p = threadIdx.x; p < nparts; p += blockDim.x) {
+    const double4_32a r = part[p];
+    v[0] += r.x;
+    v[1] += r.y;
+    v[2] += r.z;
+    v[3] += r.w;
+  }
+  block_partials<4>(v, out, 0);
 }
 
 template <int NA>
@@ -350,8 +344,8 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
 // ---- launchers -----------------------------------------------------------------------
 
 
-cudaError_t launch_energy_reduce(const Sys& s, const Bufs& b, int nparts, int nvals, cudaStream_t st) {
-  k_reduce_parts<<<1, 1024, 0, st>>>(b.part, nparts, nvals, b.result);
+cudaError_t launch_energy_reduce(const Bufs& b, int nparts, cudaStream_t st) {
+  k_reduce_parts<<<1, 1024, 0, st>>>((const double4_32a*)b.part, nparts, b.result);
   return cudaGetLastError();
 }
 
@@ -365,7 +359,7 @@ cudaError_t launch_kinetic(const Sys& s, const Bufs& b, cudaStream_t st) {
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_energy_reduce(s, b, blocks, 4, st);
+  return launch_energy_reduce(b, blocks, st);
 }
 
 cudaError_t launch_density(const Sys& s, const Bufs& b, int, cudaStream_t st) {

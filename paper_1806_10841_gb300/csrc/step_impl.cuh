@@ -25,6 +25,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "lists_impl.cuh"
@@ -211,6 +212,72 @@ struct Prec<P32> {
   static __device__ __forceinline__ float acos_(float x) { return acosf(x); }
   static __device__ __forceinline__ float div_(float a, float x) { return __fdividef(a, x); }
 };
+
+// ---------------- energy sums ----------------------------------------------------------------
+// Energies and the virial are sums of FP32 terms in double precision.  Where the terms are FP32
+// (the WCA model's) a lane keeps its sum as two floats (error-free additions, Knuth's TwoSum;
+// products exact through an FMA) and only the block totals are doubles: as doubles from the start,
+// conversions and additions on the FP64 pipe and the double logarithm of every bond made the
+// force kernel with energies 252 us at 800k atoms where it takes 33 without.
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float a) {
+    const float s = __fadd_rn(hi, a), bb = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(a, -bb)));
+    hi = s;
+  }
+  __device__ __forceinline__ void operator+=(double x) {
+    const float h = (float)x;
+    add(h);
+    lo = __fadd_rn(lo, (float)(x - (double)h));
+  }
+  // (an infinite or undefined sum leaves lo undefined)
+  __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+};
+__device__ __forceinline__ void acc(double& s, double x) { s += x; }
+__device__ __forceinline__ void acc(Sum2& s, float x) { s.add(x); }
+// the exact product of two floats
+__device__ __forceinline__ void acc_product(double& s, float a, float b) { s += (double)a * (double)b; }
+__device__ __forceinline__ void acc_product(Sum2& s, float a, float b) {
+  const float p = __fmul_rn(a, b);
+  s.add(p);
+  s.lo = __fadd_rn(s.lo, __fmaf_rn(a, b, -p));
+}
+// log g (normal g > 0 table-driven, after P. T. P. Tang, "Table-driven implementation of
+// the logarithm function", 1990): g = 2^e m, c = tab.x a nine-bit reciprocal of m's interval, so
+// r = m c - 1 is exact in two floats and |r| < 2^-7; log g = e ln 2 - log c + log1p(r), -log c as two
+// floats (tab.y, tab.z) and the series of log1p to r^5 (error below 1e-13).
+__device__ __forceinline__ void acc_log(Sum2& s, float g, const float4* tab) {
+  const unsigned u = __float_as_uint(g);
+  if (u - 0x00800000u >= 0x7f000000u) {  // zero, subnormal, negative, infinite or undefined
+    s.add(logf(g));
+    return;
+  }
+  const float m = __uint_as_float((u & 0x7fffffu) | 0x3f800000u);
+  const float4 T = tab[(u >> 16) & 127u];
+  const float e = (float)((int)(u >> 23) - 127);
+  const float p = __fmul_rn(m, T.x), rl = __fmaf_rn(m, T.x, -p), r = p - 1.f;
+  const float q = r * r * fmaf(r, fmaf(r, fmaf(r, 0.2f, -0.25f), 1.f / 3.f), -0.5f);
+  constexpr float kLn2Hi = 0.693115234375f, kLn2Lo = 3.1946183e-05f;  // ln 2, the first to 13 bits
+  s.add(e * kLn2Hi);
+  s.add(T.y);
+  s.add(r);
+  s.lo = __fadd_rn(s.lo, fmaf(e, kLn2Lo, T.z) + (rl + q - r * rl));
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_sum(Sum2 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, v.hi, o), l = __shfl_xor_sync(0xffffffffu, v.lo, o);
+    v.add(h);
+    v.lo = __fadd_rn(v.lo, l);
+  }
+  return v.value();
+}
 
 // ---------------- mapping of a molecule (group of four lanes) --------------------------
 
@@ -561,11 +628,11 @@ __device__ __forceinline__ float2 wca_fr2(const Sys& s, float2 sr6, float2 ir2, 
 // ~300 in the water-like one), tests each neighbour once instead of once per atom and leaves no
 // lane idle for three-atom molecules.  Water-like fluid, 64,000 molecules: 189 -> 138 us a step;
 // tetrahedral, 1000 molecules in the run kernel: 16.9 -> 9.4 us.
-template <int NA, bool ENERGY, int MODEL, bool HS>
+template <int NA, bool ENERGY, int MODEL, bool HS, class Acc>
 __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int G, int lig, int nnb,
                                             int m_first, bool live_item, const int4 Ca, float wa, float reach_at2, float sw,
-                                            bool slow, bool drift, float& fx, float& fy, float& fz, float& dv, double& e_at,
-                                            double& e_cg, double& vir) {
+                                            bool slow, bool drift, float& fx, float& fy, float& fz, float& dv, Acc& e_at,
+                                            Acc& e_cg, Acc& vir) {
   using Q = Prec<P32>;
   constexpr int NP = (NA + 1) / 2;  // pairs of the molecule's atoms (an odd last one is doubled)
   const int lane = threadIdx.x & 31;
@@ -643,7 +710,10 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
               if (ENERGY || drift) {
                 const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
                 const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
-                if (ENERGY) e_at += 0.5 * (double)wab * ((double)v0 + (double)v1);
+                if (ENERGY) {
+                  acc_product(e_at, 0.5f * wab, v0);
+                  acc_product(e_at, 0.5f * wab, v1);
+                }
                 if (drift) dv += v0 + v1;
               }
             } else {
@@ -685,7 +755,10 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
             ax[p] = __ffma2_rn(fr, dx, ax[p]);
             ay[p] = __ffma2_rn(fr, dy, ay[p]);
             az[p] = __ffma2_rn(fr, dz, az[p]);
-            if (ENERGY) vir += 0.5 * ((double)(fr.x * d2.x) + (double)(fr.y * d2.y));
+            if (ENERGY) {
+              acc(vir, 0.5f * (fr.x * d2.x));
+              acc(vir, 0.5f * (fr.y * d2.y));
+            }
           }
         }
       }
@@ -700,8 +773,8 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
       Fy += c * R.y;
       Fz += c * R.z;
       if (ENERGY) {
-        e_cg += 0.5 * (double)((1.f - wab) * V);
-        vir += 0.5 * (double)(Q::div_(fw, r) * r2);
+        acc(e_cg, 0.5f * ((1.f - wab) * V));
+        acc(vir, 0.5f * (Q::div_(fw, r) * r2));
       }
       if (drift) dv -= sw * V;
     }
@@ -745,11 +818,11 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
 // fetched while the current one is evaluated.  Fewer registers than one lane per neighbour
 // (48 against 90, so twice the warps): the faster way once there are enough molecules to fill
 // the device.
-template <int NA, bool ENERGY, bool HS>
+template <int NA, bool ENERGY, bool HS, class Acc>
 __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int g, int nnb,
                                                  int m_first, const int* row, const int4 Ca, float wa, float3 oi, float frac_g,
                                                  float reach_at2, float sw, bool slow, bool drift, float& fx, float& fy,
-                                                 float& fz, float& dv, double& e_at, double& e_cg, double& vir) {
+                                                 float& fz, float& dv, Acc& e_at, Acc& e_cg, Acc& vir) {
   using Q = Prec<P32>;
   constexpr int NP = (NA + 1) / 2;  // pairs of the neighbour's atoms (an odd last one is doubled)
   const float4* off = b.off32[cur];
@@ -789,7 +862,10 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
           if (ENERGY || drift) {
             const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
             const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
-            if (ENERGY) e_at += 0.5 * (double)wab * ((double)v0 + (double)v1);
+            if (ENERGY) {
+              acc_product(e_at, 0.5f * wab, v0);
+              acc_product(e_at, 0.5f * wab, v1);
+            }
             if (drift) dv += v0 + v1;
           }
           fr.x = h0 ? fr.x : 0.f;
@@ -797,7 +873,10 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
           ax = __ffma2_rn(fr, dx, ax);
           ay = __ffma2_rn(fr, dy, ay);
           az = __ffma2_rn(fr, dz, az);
-          if (ENERGY) vir += 0.5 * ((double)(fr.x * d2.x) + (double)(fr.y * d2.y));
+          if (ENERGY) {
+            acc(vir, 0.5f * (fr.x * d2.x));
+            acc(vir, 0.5f * (fr.y * d2.y));
+          }
         }
       }
     }
@@ -811,8 +890,8 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
       Fy += c * R.y;
       Fz += c * R.z;
       if (ENERGY && g == 0) {
-        e_cg += 0.5 * (double)((1.f - wab) * V);
-        vir += 0.5 * (double)(Q::div_(fw, r) * r2);
+        acc(e_cg, 0.5f * ((1.f - wab) * V));
+        acc(vir, 0.5f * (Q::div_(fw, r) * r2));
       }
       if (drift && g == 0) dv -= sw * V;
     }
@@ -1021,7 +1100,8 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
   }
 
   real fx = 0, fy = 0, fz = 0;
-  double e_at = 0.0, e_cg = 0.0, e_b = 0.0, vir = 0.0;
+  using Acc = std::conditional_t<!P::fp64 && MODEL == 0, Sum2, double>;
+  Acc e_at{}, e_cg{}, e_b{}, vir{}, e_log{};  // e_log: sum of the FENE logarithms
 
   const int a = live_item ? b.items[t] : 0;
   const Box& B = box_t<MULTI>(s, b, a);
@@ -1086,8 +1166,8 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
       Fy += c * R.y;
       Fz += c * R.z;
       if (ENERGY) {
-        e_cg += 0.5 * (double)V;
-        vir += 0.5 * (double)(c * r2);
+        acc(e_cg, (real)0.5 * V);
+        acc(vir, (real)0.5 * (c * r2));
       }
     };
     // centres of the next two neighbours in flight (long lists: the water-like fluid); the FP64
@@ -1181,7 +1261,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
         fz += fr * dz;
         if (ENERGY && (e & 8)) {
           e_b += 0.5 * (double)kb * (double)(dl - r0) * (double)(dl - r0);
-          vir += (double)(fr * d2);
+          acc(vir, fr * d2);
         }
       }
       // harmonic angles (i, vertex j, k): V = k/2 (theta - theta0)^2; the force on i is
@@ -1221,7 +1301,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
           fz -= fiz + fkz;
           if (ENERGY) {
             e_b += 0.5 * (double)ka * (double)(th - th0) * (double)(th - th0);
-            vir += (double)(ux * fix + uy * fiy + uz * fiz + vx * fkx + vy * fky + vz * fkz);
+            acc(vir, ux * fix + uy * fiy + uz * fiz + vx * fkx + vy * fky + vz * fkz);
           }
         }
       }
@@ -1240,22 +1320,22 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
       }
       const real gg = (real)1 - Q::div_(d2, R02);
       real fr = Q::div_(-K, gg);
-      double V = 0.0;
-      if (ENERGY) V = -0.5 * (double)K * (double)R02 * log((double)gg);
+      const bool first = ENERGY && (e & 8);  // accounts the bond's energy
+      if (first) {
+        if constexpr (std::is_same_v<Acc, Sum2>) acc_log(e_log, gg, b.log_tab);
+        else e_log += log((double)gg);
+      }
       if (s.intra_wca && d2 < rc_at2) {
         const real ir2 = Q::rcp_(d2);
         const real sr2 = sig2 * ir2;
         const real sr6 = sr2 * sr2 * sr2;
         fr += (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2;
-        if (ENERGY) V += (double)((real)4 * eps * (sr6 * sr6 - sr6) + eps);
+        if (first) acc(e_b, (real)4 * eps * (sr6 * sr6 - sr6) + eps);
       }
       fx += fr * dx;
       fy += fr * dy;
       fz += fr * dz;
-      if (ENERGY && (e & 8)) {
-        e_b += V;
-        vir += (double)(fr * d2);
-      }
+      if (first) acc(vir, fr * d2);
     }
     }
   }
@@ -1422,20 +1502,18 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
     }
   }
 
-  if (ENERGY) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      e_at += __shfl_xor_sync(0xffffffffu, e_at, o);
-      e_cg += __shfl_xor_sync(0xffffffffu, e_cg, o);
-      e_b += __shfl_xor_sync(0xffffffffu, e_b, o);
-      vir += __shfl_xor_sync(0xffffffffu, vir, o);
-    }
-    if (lane == 0) {
-      const size_t wid = (size_t)gtid >> 5;
-      b.part[wid * 4 + 0] = e_at;
-      b.part[wid * 4 + 1] = e_cg;
-      b.part[wid * 4 + 2] = e_b;
-      b.part[wid * 4 + 3] = vir;
+  if (ENERGY) {  // one record per block
+    __shared__ double part[kMaxForceBlock / 32][4];
+    const double sums[4] = {warp_sum(e_at), warp_sum(e_cg),
+                            warp_sum(e_b) - 0.5 * (double)par<real>(s.fene_k, s.f.fene_k) * (double)par<real>(s.fene_r02, s.f.fene_r02) *
+                                                warp_sum(e_log),
+                            warp_sum(vir)};
+    if (lane < 4) part[threadIdx.x >> 5][lane] = lane == 0 ? sums[0] : lane == 1 ? sums[1] : lane == 2 ? sums[2] : sums[3];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      double v = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += part[w][threadIdx.x];
+      b.part[(size_t)blockIdx.x * 4 + threadIdx.x] = v;
     }
   }
 }
@@ -1468,7 +1546,7 @@ constexpr int run_min_blocks() {
 template <class P, int NA, bool MULTI, int MODEL, bool HS>
 __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, int nsteps) {
   Ctrl* c = b.ctrl;
-  if (grid_is_dead(c)) return;
+  if (__syncthreads_or(threadIdx.x == 0 && __ldcg(&c->dead) != 0)) return;  // a grid barrier gave up earlier
   int cur = c->parity, set = 0, dirty = 0, rebuilt = 0;
   long long step = c->step;
   float ext_now = c->ext_now;
