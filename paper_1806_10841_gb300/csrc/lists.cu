@@ -23,6 +23,7 @@ __device__ __forceinline__ void finish_mapping(const Bufs& b, const Decision& d,
   if (d.too_wide) set_error(c, ADRESS_ERR_EXTENT, (int)(d.ext * 1000));
   c->ext_now = d.ext;
   if (d.rebuild) c->rebuilds += 1;
+  if (d.rebuild && da.build) c->force_rebuild = 0;
   if (da.advance) c->step += 1;
   c->parity ^= 1;
   if (b.npair) *b.npair = 0u;
@@ -35,12 +36,12 @@ __global__ void __launch_bounds__(32) k_decide(const __grid_constant__ Sys s, Bu
   if (!d.dead) finish_mapping(b, d, da);
 }
 
-// Decision and, when needed, the whole list build: 512-thread blocks, four per SM (32
-// registers a thread and 40 KB of staged candidates a block).  Without a build it is two
-// dependent L2 reads and one atomic per block; as a decision kernel and a conditional graph
-// node around nine build kernels the same cost about 12 us a step (800k atoms: 73.8 us a step
-// then, 68.3 us now).
-constexpr int kListThreads = 512, kListBlocksPerSm = 4;
+// Decision and, when needed, the whole list build: one block of 768 threads per SM.  Few blocks
+// keep the steps without a build cheap (two dependent L2 reads and one atomic per block; as a
+// decision kernel and a conditional graph node around nine build kernels the same cost about
+// 12 us a step at 800k atoms), and 80 registers keep the build's cell loop free of spills (800k
+// atoms, us a build: 512 threads x 4 blocks 115, x 3 111, x 2 99, 1024 x 1 94, 768 x 1 90).
+constexpr int kListThreads = 768, kListBlocksPerSm = 1;
 __global__ void __launch_bounds__(kListThreads, kListBlocksPerSm) k_lists(const __grid_constant__ Sys s, const __grid_constant__ Bufs b,
                                                                         DecideArgs da) {
   Ctrl* c = b.ctrl;
@@ -60,9 +61,7 @@ cudaError_t launch_lists(const Sys& s, const Bufs& b, DecideArgs da, cudaStream_
     k_decide<<<1, 32, 0, st>>>(s, b, da);
     return cudaGetLastError();
   }
-  // two and a half cells a warp: more blocks cost the steps that need no build more than they
-  // gain the builds (12k cells: 23.1 us a step with 608 blocks, 22.0 us with 304)
-  // (a block per 256 molecules where the cells are few and dense)
+  // two and a half cells a warp, or a block per 256 molecules where the cells are few and dense
   const long long want = std::max(ceil_div((long long)s.ncell * 32 * 2, kListThreads * 5), ceil_div(s.M, 256));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min<long long>(want, (long long)s.n_sm * kListBlocksPerSm));

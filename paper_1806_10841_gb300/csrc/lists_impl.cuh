@@ -165,22 +165,31 @@ __device__ __forceinline__ void stage_window(const Bufs& b, int lane, int incl, 
   __syncwarp();
 }
 
-// Neighbourhood of cell r: lane c < 27 gets neighbour cell c's slice of the sorted order.
-struct Neighbourhood {
-  int start, incl, pre, total, n_home, home_start, home_pre;
-};
-__device__ __forceinline__ Neighbourhood neighbourhood(const Bufs& b, int r, int lane) {
-  Neighbourhood n;
-  int cnt = 0;
-  n.start = 0;
-  if (lane < 27) {
-    const int rr = b.nbr_cells[(size_t)r * 27 + lane];
-    if (rr >= 0) {
-      n.start = b.cell_start[rr];
-      cnt = b.cell_start[rr + 1] - n.start;
-    }
+// Stage a whole neighbourhood (at most kMaxCand candidates): lane c copies neighbour cell c's
+// members, four at a time in flight.  A quarter of the instructions of stage_window at the
+// tetrahedral fluid's 2.5 molecules a cell; cells of many molecules are for stage_window.
+__device__ __forceinline__ void stage_cells(const Bufs& b, int pre, int start, int cnt, int4* st) {
+  for (int k = 0; __any_sync(0xffffffffu, k < cnt); k += 4) {
+    int4 v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (k + e < cnt) v[e] = b.scom[start + k + e];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (k + e < cnt) st[pre + k + e] = v[e];
   }
-  n.incl = cnt;
+  __syncwarp();
+}
+
+// Neighbourhood of a cell: lane c < 27 brings neighbour cell c's slice of the sorted order
+// (start, cnt; other lanes cnt = 0).
+struct Neighbourhood {
+  int start, cnt, incl, pre, total, n_home, home_start, home_pre;
+};
+__device__ __forceinline__ Neighbourhood neighbourhood(int start, int cnt, int lane) {
+  Neighbourhood n;
+  n.start = start;
+  n.cnt = n.incl = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int t = __shfl_up_sync(0xffffffffu, n.incl, o);
@@ -189,9 +198,52 @@ __device__ __forceinline__ Neighbourhood neighbourhood(const Bufs& b, int r, int
   n.pre = n.incl - cnt;
   n.total = __shfl_sync(0xffffffffu, n.incl, 31);
   n.n_home = __shfl_sync(0xffffffffu, cnt, 13);  // the home cell is neighbour 13
-  n.home_start = __shfl_sync(0xffffffffu, n.start, 13);
+  n.home_start = __shfl_sync(0xffffffffu, start, 13);
   n.home_pre = __shfl_sync(0xffffffffu, n.pre, 13);
   return n;
+}
+__device__ __forceinline__ int neighbour_cell(const Sys& s, const Bufs& b, int r, int lane) {
+  return r < s.ncell && lane < 27 ? b.nbr_cells[(size_t)r * 27 + lane] : -1;
+}
+__device__ __forceinline__ void cell_slice(const Bufs& b, int rr, int& start, int& end) {
+  start = end = 0;
+  if (rr >= 0) {
+    start = b.cell_start[rr];
+    end = b.cell_start[rr + 1];
+  }
+}
+
+// Two molecules H0, H1 of a warp's cell against candidate k's centre D (k < n): their neighbours
+// appended to the two rows in candidate order, by ballot and popcount.  The molecules' own places
+// among the candidates are k0 and k1; `two` is false when there is no second one.
+struct PairRows {
+  int *row0, *row1;
+  int c0, c1;
+};
+__device__ __forceinline__ void test_two(const Sys& s, const Box& B, int4 H0, int4 H1, int k0, int k1, bool two, int4 D, int k,
+                                         bool in, unsigned below, PairRows& P) {
+  const float sx = B.fx_scale[0], sy = B.fx_scale[1], sz = B.fx_scale[2];
+  const float x0 = (float)(int)((unsigned)H0.x - (unsigned)D.x) * sx;
+  const float y0 = (float)(int)((unsigned)H0.y - (unsigned)D.y) * sy;
+  const float z0 = (float)(int)((unsigned)H0.z - (unsigned)D.z) * sz;
+  const float x1 = (float)(int)((unsigned)H1.x - (unsigned)D.x) * sx;
+  const float y1 = (float)(int)((unsigned)H1.y - (unsigned)D.y) * sy;
+  const float z1 = (float)(int)((unsigned)H1.z - (unsigned)D.z) * sz;
+  const float rl2 = s.f.r_list2, rcl2 = s.f.r_cg_list2;
+  const bool hit0 = in && k != k0 && x0 * x0 + y0 * y0 + z0 * z0 < ((H0.w & D.w) < 0 ? rl2 : rcl2);
+  const bool hit1 = in && k != k1 && x1 * x1 + y1 * y1 + z1 * z1 < ((H1.w & D.w) < 0 ? rl2 : rcl2);
+  const unsigned b0 = __ballot_sync(0xffffffffu, hit0), b1 = __ballot_sync(0xffffffffu, hit1);
+  const int p0 = P.c0 + __popc(b0 & below), p1 = P.c1 + __popc(b1 & below);
+  if (hit0 && p0 < s.cap) P.row0[p0] = id_of(D.w);
+  if (hit1 && two && p1 < s.cap) P.row1[p1] = id_of(D.w);
+  P.c0 += __popc(b0);
+  P.c1 += __popc(b1);
+}
+// Record a finished list of c neighbours of molecule H, work item t.
+__device__ __forceinline__ void close_list(const Sys& s, const Bufs& b, int4 H, int t, int c) {
+  b.nn[t] = c < s.cap ? c : s.cap;
+  b.com_ref[id_of(H.w)] = make_int4(H.x, H.y, H.z, 0);
+  if (c > s.cap) set_error(b.ctrl, ADRESS_ERR_LIST_OVERFLOW, c);
 }
 
 // One warp, one cell: the 27 neighbour cells in the fixed (ox, oy, oz) order, their members
@@ -199,63 +251,39 @@ __device__ __forceinline__ Neighbourhood neighbourhood(const Bufs& b, int r, int
 // of the cell then tests all candidates in parallel, two molecules per pass over the
 // candidates, and appends its neighbours in candidate order with ballot/popc compaction.
 // A cell with more than kMaxCand candidates or 32 molecules goes to the dense-cell list.
-__device__ __forceinline__ void list_cell(const Sys& s, const Bufs& b, int r, int lane, int n_hr, int4* st) {
+__device__ __forceinline__ void list_cell(const Sys& s, const Bufs& b, int r, int start, int cnt, int lane, int n_hr, int4* st) {
   const Box& B = s.nbox > 1 ? b.boxes[b.cell_box[r]] : s.bx;
-  const Neighbourhood n = neighbourhood(b, r, lane);
+  const Neighbourhood n = neighbourhood(start, cnt, lane);
   if (n.n_home == 0) return;
   if (n.total > kMaxCand || n.n_home > 32) {
     if (lane == 0) b.dense_cells[atomicAdd(&b.ctrl->n_dense, 1)] = r;
     return;
   }
   __syncwarp();  // the previous cell's candidates are no longer read
-  stage_window(b, lane, n.incl, n.pre, n.start, 0, n.total, st);
+  stage_cells(b, n.pre, n.start, n.cnt, st);
   // work items of the home molecules: high-resolution ones first, then coarse-grained, each
   // in sorted order
   const int hw = lane < n.n_home ? st[n.home_pre + lane].w : 0;
   const unsigned hr_mask = __ballot_sync(0xffffffffu, hw < 0);
-  const int hr_below = __popc(hr_mask & ((1u << lane) - 1u)), h0 = b.cell_hr[r];
+  const unsigned below = (1u << lane) - 1u;
+  const int hr_below = __popc(hr_mask & below), h0 = b.cell_hr[r];
   const int my_item = hw < 0 ? h0 + hr_below : n_hr + (n.home_start - h0) + (lane - hr_below);
   if (lane < n.n_home) {
     const int a = id_of(hw);
     b.items[my_item] = a;
     b.item_of[a] = my_item;
   }
-  const float rl2 = s.f.r_list2, rcl2 = s.f.r_cg_list2;
-  const float sx = B.fx_scale[0], sy = B.fx_scale[1], sz = B.fx_scale[2];
-  const unsigned below = (1u << lane) - 1u;
   for (int h = 0; h < n.n_home; h += 2) {
-    const int hb = h + 1 < n.n_home ? h + 1 : h;
-    const int4 H0 = st[n.home_pre + h], H1 = st[n.home_pre + hb];
-    const int t0 = __shfl_sync(0xffffffffu, my_item, h), t1 = __shfl_sync(0xffffffffu, my_item, hb);
-    int* row0 = b.nbr + (size_t)t0 * s.cap;
-    int* row1 = b.nbr + (size_t)t1 * s.cap;
-    int c0 = 0, c1 = 0;
+    const bool two = h + 1 < n.n_home;
+    const int ka = n.home_pre + h, kb = two ? ka + 1 : ka;
+    const int4 H0 = st[ka], H1 = st[kb];
+    const int t0 = __shfl_sync(0xffffffffu, my_item, h), t1 = __shfl_sync(0xffffffffu, my_item, h + two);
+    PairRows P{b.nbr + (size_t)t0 * s.cap, b.nbr + (size_t)t1 * s.cap, 0, 0};
     for (int k0 = 0; k0 < n.total; k0 += 32) {
       const int k = k0 + lane;
-      const int4 D = st[k < n.total ? k : 0];
-      const float x0 = (float)(int)((unsigned)H0.x - (unsigned)D.x) * sx;
-      const float y0 = (float)(int)((unsigned)H0.y - (unsigned)D.y) * sy;
-      const float z0 = (float)(int)((unsigned)H0.z - (unsigned)D.z) * sz;
-      const float x1 = (float)(int)((unsigned)H1.x - (unsigned)D.x) * sx;
-      const float y1 = (float)(int)((unsigned)H1.y - (unsigned)D.y) * sy;
-      const float z1 = (float)(int)((unsigned)H1.z - (unsigned)D.z) * sz;
-      const bool in = k < n.total;
-      const bool hit0 = in && k != n.home_pre + h && x0 * x0 + y0 * y0 + z0 * z0 < ((H0.w & D.w) < 0 ? rl2 : rcl2);
-      const bool hit1 = in && k != n.home_pre + hb && x1 * x1 + y1 * y1 + z1 * z1 < ((H1.w & D.w) < 0 ? rl2 : rcl2);
-      const unsigned b0 = __ballot_sync(0xffffffffu, hit0), b1 = __ballot_sync(0xffffffffu, hit1);
-      const int p0 = c0 + __popc(b0 & below), p1 = c1 + __popc(b1 & below);
-      if (hit0 && p0 < s.cap) row0[p0] = id_of(D.w);
-      if (hit1 && hb != h && p1 < s.cap) row1[p1] = id_of(D.w);
-      c0 += __popc(b0);
-      c1 += __popc(b1);
+      test_two(s, B, H0, H1, ka, kb, two, st[k < n.total ? k : 0], k, k < n.total, below, P);
     }
-    if (lane < 2 && (lane == 0 || hb != h)) {
-      const int4 H = lane ? H1 : H0;
-      const int c = lane ? c1 : c0, t = lane ? t1 : t0;
-      b.nn[t] = c < s.cap ? c : s.cap;
-      b.com_ref[id_of(H.w)] = make_int4(H.x, H.y, H.z, 0);
-      if (c > s.cap) set_error(b.ctrl, ADRESS_ERR_LIST_OVERFLOW, c);
-    }
+    if (lane < 1 + two) close_list(s, b, lane ? H1 : H0, lane ? t1 : t0, lane ? P.c1 : P.c0);
   }
 }
 
@@ -264,11 +292,15 @@ __device__ __forceinline__ void list_cell(const Sys& s, const Bufs& b, int r, in
 // each lane then walks the staged window for its own molecule and appends its neighbours in
 // candidate order (the order of the ballot compaction in list_cell): the same lists for any
 // density.  Task = (dense cell, part): part j takes the home batches j, j + kHomeParts, ...
+// (Two molecules at a time against 32 candidates, as in list_cell, was slower: a build of 64,000
+// water-like molecules 544 us against 386.)
 constexpr int kHomeParts = 4;
-__device__ __forceinline__ void list_dense_part(const Sys& s, const Bufs& b, int r, int part, int lane, int n_hr,
-                                                int4* st) {
+__device__ __forceinline__ void list_dense_part(const Sys& s, const Bufs& b, int r, int part, int lane, int n_hr, int4* st) {
+  if (part * 32 >= b.cell_start[r + 1] - b.cell_start[r]) return;
   const Box& B = s.nbox > 1 ? b.boxes[b.cell_box[r]] : s.bx;
-  const Neighbourhood n = neighbourhood(b, r, lane);
+  int start, end;
+  cell_slice(b, neighbour_cell(s, b, r, lane), start, end);
+  const Neighbourhood n = neighbourhood(start, end - start, lane);
   const float rl2 = s.f.r_list2, rcl2 = s.f.r_cg_list2;
   int hr_before = 0;  // high-resolution molecules of the cell before the current batch
   for (int hb = 0; hb < n.n_home; hb += 32) {
@@ -306,12 +338,15 @@ __device__ __forceinline__ void list_dense_part(const Sys& s, const Bufs& b, int
         }
       }
     }
-    if (mine) {
-      b.nn[tt] = count < s.cap ? count : s.cap;
-      b.com_ref[a] = make_int4(C.x, C.y, C.z, 0);
-      if (count > s.cap) set_error(b.ctrl, ADRESS_ERR_LIST_OVERFLOW, count);
-    }
+    if (mine) close_list(s, b, C, tt, count);
   }
+}
+
+// High-resolution candidate: decided from the mapping's distance to the region.
+__device__ __forceinline__ int hr_candidate(const Sys& s, const Bufs& b, const Box& B, int cur, int a) {
+  if (s.lam_uniform_on) return s.lam_uniform > 0.0 ? 1 : 0;
+  if (s.fp64) return fabs(b.dxc64[cur][a]) < B.d_hr ? 1 : 0;
+  return fabsf(b.molf[cur][a].x) < B.d_hr_f ? 1 : 0;
 }
 
 // ---- candidate pairs of the network CG force ---------------------------------------------------
@@ -412,11 +447,9 @@ __device__ __forceinline__ void net_candidates_of(const Sys& s, const Bufs& b, i
 
 // ---- the build ---------------------------------------------------------------------------------
 
-// All lists of the mapping `cur`, by every block of a cooperative grid; false when a barrier
-// gave up (the block must leave).  No barrier after the last phase: the caller orders the
-// lists before their readers.  WARPS: warps per block.
+// The lists of any system, through cells (see the head of this file).  WARPS: warps per block.
 template <int WARPS>
-__device__ __forceinline__ bool rebuild_lists(const Sys& s, const Bufs& b, int cur, GridBarrier& bar) {
+__device__ __forceinline__ bool list_cells(const Sys& s, const Bufs& b, int cur, GridBarrier& bar) {
   __shared__ int4 stage[WARPS * kMaxCand];
   Ctrl* c = b.ctrl;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsize = gridDim.x * blockDim.x;
@@ -430,10 +463,7 @@ __device__ __forceinline__ bool rebuild_lists(const Sys& s, const Bufs& b, int c
     const int cx = cell_of((unsigned)C.x, B.nc[0]), cy = cell_of((unsigned)C.y, B.nc[1]),
               cz = cell_of((unsigned)C.z, B.nc[2]);
     const int r = b.cell_rank[B.cell0 + (cx * B.nc[1] + cy) * B.nc[2] + cz];
-    int hr;
-    if (s.lam_uniform_on) hr = s.lam_uniform > 0.0 ? 1 : 0;
-    else if (s.fp64) hr = fabs(b.dxc64[cur][a]) < B.d_hr ? 1 : 0;
-    else hr = fabsf(b.molf[cur][a].x) < B.d_hr_f ? 1 : 0;
+    const int hr = hr_candidate(s, b, B, cur, a);
     const unsigned long long w = atomicAdd(&b.cell_count[r], hr ? 0x100000001ull : 1ull);
     b.mcell[a] = r;
     b.mslot[a] = tag_id((int)(unsigned)w, hr);
@@ -448,11 +478,7 @@ __device__ __forceinline__ bool rebuild_lists(const Sys& s, const Bufs& b, int c
     block_excl_u64(sum, &total);
     if (threadIdx.x == 0) {
       b.scan_tmp[blockIdx.x] = total;
-      if (blockIdx.x == 0) {  // consumed by the previous build
-        c->force_rebuild = 0;
-        c->n_dense = 0;
-        c->n_netc = 0;
-      }
+      if (blockIdx.x == 0) c->n_dense = 0;  // consumed by the previous build
     }
   }
   if (!bar.sync()) return false;
@@ -499,12 +525,35 @@ __device__ __forceinline__ bool rebuild_lists(const Sys& s, const Bufs& b, int c
     b.scom[ps + rank] = make_int4(C.x, C.y, C.z, w);
   }
   if (!bar.sync()) return false;
-  for (int r = gwarp; r < s.ncell; r += nwarps) list_cell(s, b, r, lane, n_hr, st);
+  {
+    // the next cell's slices and the one after's neighbour cells are fetched meanwhile
+    int start, end;
+    cell_slice(b, neighbour_cell(s, b, gwarp, lane), start, end);
+    int rr = neighbour_cell(s, b, gwarp + nwarps, lane);
+    for (int r = gwarp; r < s.ncell; r += nwarps) {
+      const int cs = start, cn = end - start;
+      cell_slice(b, rr, start, end);
+      rr = neighbour_cell(s, b, r + 2 * nwarps, lane);
+      list_cell(s, b, r, cs, cn, lane, n_hr, st);
+    }
+  }
   if (!bar.sync()) return false;
   const int n_dense = __ldcg(&c->n_dense);
   for (int task = gwarp; task < n_dense * kHomeParts; task += nwarps)
     list_dense_part(s, b, b.dense_cells[task / kHomeParts], task % kHomeParts, lane, n_hr, st);
+  return true;
+}
+
+// All lists of the mapping `cur`, by every block of a cooperative grid; false when a barrier
+// gave up (the block must leave).  No barrier after the last phase: the caller orders the
+// lists before their readers, and clears Ctrl::force_rebuild after that.
+template <int WARPS>
+__device__ __forceinline__ bool rebuild_lists(const Sys& s, const Bufs& b, int cur, GridBarrier& bar) {
+  if (!list_cells<WARPS>(s, b, cur, bar)) return false;
   if (s.cg_mode && b.netc) {
+    const int lane = threadIdx.x & 31;
+    const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.ctrl->n_netc = 0;
     if (!bar.sync()) return false;
     for (int w = gwarp; w * 8 < s.M; w += nwarps) {
       if (s.fp64) net_candidates_of<true>(s, b, cur, w * 8 + (lane >> 2), lane & 3);

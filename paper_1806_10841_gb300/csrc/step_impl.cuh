@@ -1579,6 +1579,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
       ++rebuilt;
       if (!rebuild_lists<kMaxForceBlock / 32>(s, b, cur, bar)) return;
       if (!bar.sync()) return;
+      if (blockIdx.x == 0 && threadIdx.x == 0) c->force_rebuild = 0;
     }
   }
   if (threadIdx.x < 32 && last_to_arrive(c)) {
