@@ -762,6 +762,11 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   if (e == cudaSuccess) e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned long long) * ntf, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.nsamples, 0, sizeof(long long), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.com_ref, 0, sizeof(int4) * M, st);
+  // empty lists: forces may be launched behind a build that gave up (adress_compute_forces)
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.items, 0, sizeof(int) * M, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.item_of, 0, sizeof(int) * M, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.nn, 0, sizeof(int) * M, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.nbr, 0, sizeof(int) * (size_t)s.cap * M, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host vectors go out of scope
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -845,6 +850,7 @@ static adress_status judge_build(adress_handle h, const Ctrl& c, bool* redo) {
     int* nbr = nullptr;
     CUDA_OR_FAIL(h, cudaStreamSynchronize(h->stream));
     CUDA_OR_FAIL(h, dalloc(h, &nbr, (size_t)cap * h->sys.M));
+    CUDA_OR_FAIL(h, cudaMemsetAsync(nbr, 0, sizeof(int) * (size_t)cap * h->sys.M, h->stream));
     h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), old));
     cudaFree(old);
     h->buf.nbr = nbr;
