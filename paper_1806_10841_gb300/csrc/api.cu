@@ -190,6 +190,28 @@ static int auto_capacity(const Sys& s, const std::vector<Box>& boxes, const std:
   return std::min(cap, std::max(4, s.M - 1));
 }
 
+// Deal the bonds out to rounds: in a round an atom evaluates at most one bond and receives the
+// force of at most one.  The fewest rounds, by exhaustive search (at most six bonds).
+static bool place_bonds(Sys& s, int q, int rounds) {
+  if (q == s.nb) return true;
+  for (int r = 0; r < rounds; ++r)
+    for (int flip = 0; flip < 2; ++flip) {
+      const int o = s.bonds[2 * q + flip], p = s.bonds[2 * q + 1 - flip], sh = 4 * r;
+      if (((s.bond_send[o] >> sh) & 15) || ((s.bond_recv[p] >> sh) & 15)) continue;
+      s.bond_send[o] |= (unsigned)(p | 8) << sh;
+      s.bond_recv[p] |= (unsigned)(o | 8) << sh;
+      if (place_bonds(s, q + 1, rounds)) return true;
+      s.bond_send[o] &= ~(15u << sh);
+      s.bond_recv[p] &= ~(15u << sh);
+    }
+  return false;
+}
+static void schedule_bonds(Sys& s) {
+  for (int g = 0; g < kMaxNA; ++g) s.bond_send[g] = s.bond_recv[g] = 0;
+  s.bond_rounds = 0;
+  while (!place_bonds(s, 0, s.bond_rounds)) ++s.bond_rounds;  // nb rounds always do
+}
+
 // Validation of one configuration; empty when valid.
 static std::string config_error(const adress_config* c) {
   if (c->n_mols < 2) return "n_mols must be >= 2";
@@ -520,23 +542,10 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   s.rc_at2 = c->rc_at * c->rc_at;
   s.nb = c->n_bonds;
   for (int q = 0; q < 2 * kMaxBonds; ++q) s.bonds[q] = q < 2 * c->n_bonds ? c->bonds[q] : 0;
-  // per-atom bond partners in bond order (bit 3: this atom is the bond's first atom)
-  {
-    int cnt[kMaxNA] = {0, 0, 0, 0};
-    for (int g = 0; g < kMaxNA; ++g) s.bond_word[g] = 0;
-    for (int q = 0; q < c->n_bonds; ++q) {
-      const int p0 = c->bonds[2 * q], p1 = c->bonds[2 * q + 1];
-      s.bond_word[p0] |= (unsigned)(p1 | 8) << (4 * cnt[p0]++);
-      s.bond_word[p1] |= (unsigned)p0 << (4 * cnt[p1]++);
-    }
-    s.bmax = 0;
-    for (int g = 0; g < kMaxNA; ++g) {
-      s.bond_word[g] |= (unsigned)cnt[g] << 28;
-      s.bmax = std::max(s.bmax, cnt[g]);
-    }
-  }
+  schedule_bonds(s);
   s.fene_k = c->fene_k;
   s.fene_r02 = c->fene_r0 * c->fene_r0;
+  s.fene_inv_r02 = 1.0 / s.fene_r02;
   s.intra_wca = c->intra_wca;
   s.cg_n = c->cg_n;
   s.cg_inv_dr = 1.0 / c->cg_dr;

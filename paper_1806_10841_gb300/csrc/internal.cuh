@@ -103,12 +103,12 @@ struct Sys {
   double eps, sig2, rc_at2;
   int nb;
   int bonds[2 * kMaxBonds];
-  // the same bonds per atom, in bond order, one word per atom: entry q in bits 4q..4q+3 =
-  // partner | 8 when the atom is the bond's first atom (which accounts its energy), the
-  // count in bits 28..31; bmax the largest count
-  unsigned bond_word[kMaxNA];
-  int bmax;
-  double fene_k, fene_r02;
+  // who evaluates which bond when (schedule_bonds): in round q atom i evaluates its bond with atom
+  // bond_send[i] nibble q & 3 (bit 3: it has one) and gets the force of the bond that atom
+  // bond_recv[i] nibble q & 3 evaluates (bit 3: there is one)
+  unsigned bond_send[kMaxNA], bond_recv[kMaxNA];
+  int bond_rounds;
+  double fene_k, fene_r02, fene_inv_r02;
   int intra_wca;
   int cg_n;
   double cg_inv_dr, rc_cg2;

@@ -81,6 +81,9 @@ __device__ __forceinline__ double par<double>(double d, float) { return d; }
 template <>
 __device__ __forceinline__ float par<float>(double, float f) { return f; }
 
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
 // floor(x 2^32 / L) for 0 <= x < L from the bits of x: the 53-bit significand times
 // K = floor(2^q / L) (exact 128-bit product, high word kept), shifted by the exponent.
 __device__ __forceinline__ unsigned fixed32(double x, unsigned long long K, int q) {
@@ -205,12 +208,22 @@ struct Prec<P32> {
   static __device__ __forceinline__ float tf(const Bufs& b, int k) { return b.tf32[k]; }
   static __device__ __forceinline__ float fec(const Bufs& b, int k) { return b.fec32[k]; }
   static __device__ __forceinline__ float sin_(float x) { return sinf(x); }
-  // hardware approximations (a few ulp): the FP32 path's error budget is 2e-5 relative
-  static __device__ __forceinline__ float sqrt_(float x) { return x * rsqrtf(x); }
-  static __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
-  static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
+  // hardware approximations (a few ulp): the FP32 path's error budget is 2e-5 relative; in the
+  // forms that take subnormal numbers for zero, which cost two to four instructions less.  A
+  // quotient is a product, so that the compiler can join it with a following sum.
+  static __device__ __forceinline__ float rsqrt_(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+  }
+  static __device__ __forceinline__ float sqrt_(float x) { return x * rsqrt_(x); }
+  static __device__ __forceinline__ float rcp_(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+  }
   static __device__ __forceinline__ float acos_(float x) { return acosf(x); }
-  static __device__ __forceinline__ float div_(float a, float x) { return __fdividef(a, x); }
+  static __device__ __forceinline__ float div_(float a, float x) { return a * rcp_(x); }
 };
 
 // ---------------- energy sums ----------------------------------------------------------------
@@ -461,7 +474,8 @@ __device__ __forceinline__ void map_group32(const Sys& s, const Box& B, const Bu
   }
 }
 
-// P64: the plain double-precision mapping (the FP64 reference path).
+// P64: the mapping in double precision; comparisons and the fixed-point copy run on the integer
+// pipe (the FP64 one runs 2 lanes a clock per SM).
 template <int NA>
 __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bufs& b, int nxt, int a, int g, unsigned gmask,
                                             int base, bool live, const double x[3], const int4 ref, float& ext2,
@@ -471,25 +485,25 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const double x0 = shfl_d(gmask, x[d], base);
-    dl[d] = own ? minimg_cmp(x[d] - x0, B.L[d], B.halfL[d]) : 0.0;
+    dl[d] = own ? minimg_bits(x[d] - x0, B.L[d], B.halfL[d]) : 0.0;
     double cs = own ? s.frac[g] * dl[d] : 0.0;
     cs += shfl_xor_d(gmask, cs, 1);
     cs += shfl_xor_d(gmask, cs, 2);
     c[d] = cs;
-    double r = x0 + cs;
-    if (r < 0.0) r += B.L[d];
-    if (r >= B.L[d]) r -= B.L[d];
-    R[d] = r;
+    R[d] = wrap_bits(x0 + cs, B.L[d], B.Lbits[d]);
   }
   if (own) {
     const double o0 = dl[0] - c[0], o1 = dl[1] - c[1], o2 = dl[2] - c[2];
     b.off64[nxt][a * NA + g] = make_double4_32a(o0, o1, o2, 0.0);
     // as float for the pair tests that decide where FP64 is needed
     float* of = (float*)(b.off32[nxt] + 3 * (size_t)a) + g;
-    of[0] = d2f_bits(o0);
-    of[4] = d2f_bits(o1);
-    of[8] = d2f_bits(o2);
-    ext2 = fmaxf(ext2, (float)(o0 * o0 + o1 * o1 + o2 * o2));
+    const float f0 = d2f_bits(o0), f1 = d2f_bits(o1), f2 = d2f_bits(o2);
+    of[0] = f0;
+    of[4] = f1;
+    of[8] = f2;
+    // (an undefined coordinate is left to the force's check, as fmaxf leaves out a NaN)
+    auto nan = [](double v) { return ((unsigned long long)__double_as_longlong(v) << 1) > 0xFFE0000000000000ull; };
+    if (!(nan(o0) || nan(o1) || nan(o2))) ext2 = fmaxf(ext2, f0 * f0 + f1 * f1 + f2 * f2);
   }
   int kmin = 0;
   const double dxc = s.n_centers > 0 ? nearest_center64(s, B, b, gmask, g, R, kmin)
@@ -509,7 +523,7 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
     if (s.n_centers > 0) b.kcen[nxt][a] = kmin;
     unsigned X[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) X[d] = (unsigned)(unsigned long long)llrint(R[d] * B.fx_inv[d]);
+    for (int d = 0; d < 3; ++d) X[d] = fixed32(R[d], B.fxK[d], B.fxq[d]);
     // the float weight is 0 or 1 only where the double one is
     float wf = (float)w;
     if (w < 1.0 && wf >= 1.f) wf = 0x1.fffffep-1f;
@@ -634,7 +648,7 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
                                             bool slow, bool drift, float& fx, float& fy, float& fz, float& dv, Acc& e_at,
                                             Acc& e_cg, Acc& vir) {
   using Q = Prec<P32>;
-  constexpr int NP = (NA + 1) / 2;  // pairs of the molecule's atoms (an odd last one is doubled)
+  constexpr int NP = (NA + 1) / 2;  // pairs of the molecule's atoms, an odd last one by itself
   const int lane = threadIdx.x & 31;
   const int* row = b.nbr + (size_t)(live_item ? t : 0) * s.cap;
   const float4* off = b.off32[cur];
@@ -690,76 +704,90 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
         Z = off[3 * (size_t)m + 2];
       }
       const float xj[4] = {X.x, X.y, X.z, X.w}, yj[4] = {Y.x, Y.y, Y.z, Y.w}, zj[4] = {Z.x, Z.y, Z.z, Z.w};
+      // two atom pairs (ia, ja), (ib, jb) with the separations dx, dy, dz; `both`: the second one
+      // counts; the forces go to (fx2, fy2, fz2)
+      auto pairs = [&](float2 dx, float2 dy, float2 dz, int ia, int ja, int ib, int jb, bool both, float2& fx2, float2& fy2,
+                       float2& fz2) {
+        const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+        const bool h0 = d2.x < rc_at2, h1 = both && d2.y < rc_at2;
+        if (h0 || h1) {
+          float2 fr;
+          if (MODEL == 0) {
+            const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
+            const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
+            const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
+            fr = wca_fr2(s, sr6, ir2, wab);
+            if (ENERGY || drift) {
+              const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
+              const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
+              if (ENERGY) {
+                acc_product(e_at, 0.5f * wab, v0);
+                acc_product(e_at, 0.5f * wab, v1);
+              }
+              if (drift) dv += v0 + v1;
+            }
+          } else {
+            // LJ (c12 r^-12 - c6 r^-6, shifted) for the site pairs that have one + reaction
+            // field q_i q_j f (1/r + k_rf r^2 - c_rf)
+            const float2 ir = make_float2(Q::rsqrt_(d2.x), Q::rsqrt_(d2.y));
+            const float2 ir2 = __fmul2_rn(ir, ir);
+            const float2 qq = make_float2(s.f.qq[ia][ja], s.f.qq[ib][jb]);
+            float2 flj = make_float2(0.f, 0.f);
+            float vl0 = 0.f, vl1 = 0.f;
+            if ((s.lj_pairs >> (4 * ia + ja)) & 1) {
+              const float ir6 = ir2.x * ir2.x * ir2.x;
+              flj.x = (12.f * s.f.c12[ia][ja] * ir6 - 6.f * s.f.c6[ia][ja]) * ir6 * ir2.x;
+              if (ENERGY || drift) vl0 = (s.f.c12[ia][ja] * ir6 - s.f.c6[ia][ja]) * ir6;
+            }
+            if (both && ((s.lj_pairs >> (4 * ib + jb)) & 1)) {
+              const float ir6 = ir2.y * ir2.y * ir2.y;
+              flj.y = (12.f * s.f.c12[ib][jb] * ir6 - 6.f * s.f.c6[ib][jb]) * ir6 * ir2.y;
+              if (ENERGY || drift) vl1 = (s.f.c12[ib][jb] * ir6 - s.f.c6[ib][jb]) * ir6;
+            }
+            fr = __ffma2_rn(qq, __ffma2_rn(ir2, ir, make_float2(-s.f.krf2, -s.f.krf2)), flj);
+            fr = __fmul2_rn(fr, make_float2(wab, wab));
+            if (ENERGY) {
+              if (h0)
+                acc(e_at, 0.5 * (double)wab *
+                              ((double)vl0 + s.vsh[ia][ja] + (double)qq.x * ((double)ir.x + s.krf * (double)d2.x - s.crf)));
+              if (h1)
+                acc(e_at, 0.5 * (double)wab *
+                              ((double)vl1 + s.vsh[ib][jb] + (double)qq.y * ((double)ir.y + s.krf * (double)d2.y - s.crf)));
+            }
+            if (drift) {
+              if (h0) dv += vl0 + s.f.vsh[ia][ja] + qq.x * (ir.x + s.f.krf * d2.x - s.f.crf);
+              if (h1) dv += vl1 + s.f.vsh[ib][jb] + qq.y * (ir.y + s.f.krf * d2.y - s.f.crf);
+            }
+          }
+          fr.x = h0 ? fr.x : 0.f;
+          fr.y = h1 ? fr.y : 0.f;
+          fx2 = __ffma2_rn(fr, dx, fx2);
+          fy2 = __ffma2_rn(fr, dy, fy2);
+          fz2 = __ffma2_rn(fr, dz, fz2);
+          if (ENERGY) {
+            acc(vir, 0.5f * (fr.x * d2.x));
+            acc(vir, 0.5f * (fr.y * d2.y));
+          }
+        }
+      };
 #pragma unroll
-      for (int p = 0; p < NP; ++p) {
+      for (int p = 0; p < NA / 2; ++p) {
         const float2 px = __fadd2_rn(nx[p], make_float2(R.x, R.x)), py = __fadd2_rn(ny[p], make_float2(R.y, R.y)),
                      pz = __fadd2_rn(nz[p], make_float2(R.z, R.z));
 #pragma unroll
-        for (int j = 0; j < NA; ++j) {
-          const float2 dx = __fadd2_rn(px, make_float2(xj[j], xj[j])), dy = __fadd2_rn(py, make_float2(yj[j], yj[j])),
-                       dz = __fadd2_rn(pz, make_float2(zj[j], zj[j]));
-          const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
-          const bool h0 = d2.x < rc_at2, h1 = 2 * p + 1 < NA && d2.y < rc_at2;
-          if (h0 || h1) {
-            float2 fr;
-            if (MODEL == 0) {
-              const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
-              const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
-              const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
-              fr = wca_fr2(s, sr6, ir2, wab);
-              if (ENERGY || drift) {
-                const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
-                const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
-                if (ENERGY) {
-                  acc_product(e_at, 0.5f * wab, v0);
-                  acc_product(e_at, 0.5f * wab, v1);
-                }
-                if (drift) dv += v0 + v1;
-              }
-            } else {
-              // LJ (c12 r^-12 - c6 r^-6, shifted) for the site pairs that have one + reaction
-              // field q_i q_j f (1/r + k_rf r^2 - c_rf)
-              const float2 ir = make_float2(Q::rsqrt_(d2.x), Q::rsqrt_(d2.y));
-              const float2 ir2 = __fmul2_rn(ir, ir);
-              const int i0 = 2 * p, i1 = 2 * p + 1 < NA ? 2 * p + 1 : 2 * p;
-              const float2 qq = make_float2(s.f.qq[i0][j], s.f.qq[i1][j]);
-              float2 flj = make_float2(0.f, 0.f);
-              float vl0 = 0.f, vl1 = 0.f;
-              if ((s.lj_pairs >> (4 * i0 + j)) & 1) {
-                const float ir6 = ir2.x * ir2.x * ir2.x;
-                flj.x = (12.f * s.f.c12[i0][j] * ir6 - 6.f * s.f.c6[i0][j]) * ir6 * ir2.x;
-                if (ENERGY || drift) vl0 = (s.f.c12[i0][j] * ir6 - s.f.c6[i0][j]) * ir6;
-              }
-              if (i1 != i0 && ((s.lj_pairs >> (4 * i1 + j)) & 1)) {
-                const float ir6 = ir2.y * ir2.y * ir2.y;
-                flj.y = (12.f * s.f.c12[i1][j] * ir6 - 6.f * s.f.c6[i1][j]) * ir6 * ir2.y;
-                if (ENERGY || drift) vl1 = (s.f.c12[i1][j] * ir6 - s.f.c6[i1][j]) * ir6;
-              }
-              fr = __ffma2_rn(qq, __ffma2_rn(ir2, ir, make_float2(-s.f.krf2, -s.f.krf2)), flj);
-              fr = __fmul2_rn(fr, make_float2(wab, wab));
-              if (ENERGY) {
-                if (h0)
-                  e_at += 0.5 * (double)wab *
-                          ((double)vl0 + s.vsh[i0][j] + (double)qq.x * ((double)ir.x + s.krf * (double)d2.x - s.crf));
-                if (h1)
-                  e_at += 0.5 * (double)wab *
-                          ((double)vl1 + s.vsh[i1][j] + (double)qq.y * ((double)ir.y + s.krf * (double)d2.y - s.crf));
-              }
-              if (drift) {
-                if (h0) dv += vl0 + s.f.vsh[i0][j] + qq.x * (ir.x + s.f.krf * d2.x - s.f.crf);
-                if (h1) dv += vl1 + s.f.vsh[i1][j] + qq.y * (ir.y + s.f.krf * d2.y - s.f.crf);
-              }
-            }
-            fr.x = h0 ? fr.x : 0.f;
-            fr.y = h1 ? fr.y : 0.f;
-            ax[p] = __ffma2_rn(fr, dx, ax[p]);
-            ay[p] = __ffma2_rn(fr, dy, ay[p]);
-            az[p] = __ffma2_rn(fr, dz, az[p]);
-            if (ENERGY) {
-              acc(vir, 0.5f * (fr.x * d2.x));
-              acc(vir, 0.5f * (fr.y * d2.y));
-            }
-          }
+        for (int j = 0; j < NA; ++j)
+          pairs(__fadd2_rn(px, make_float2(xj[j], xj[j])), __fadd2_rn(py, make_float2(yj[j], yj[j])),
+                __fadd2_rn(pz, make_float2(zj[j], zj[j])), 2 * p, j, 2 * p + 1, j, true, ax[p], ay[p], az[p]);
+      }
+      if (NA & 1) {  // the odd atom takes the neighbour's atoms two at a time
+        constexpr int p = NA / 2 < NP ? NA / 2 : 0;
+        const float px = nx[p].x + R.x, py = ny[p].x + R.y, pz = nz[p].x + R.z;
+        const float2 p2 = make_float2(px, px), q2 = make_float2(py, py), r2p = make_float2(pz, pz);
+#pragma unroll
+        for (int j = 0; j < NA; j += 2) {
+          const int j1 = j + 1 < NA ? j + 1 : j;
+          pairs(__fadd2_rn(p2, make_float2(xj[j], xj[j1])), __fadd2_rn(q2, make_float2(yj[j], yj[j1])),
+                __fadd2_rn(r2p, make_float2(zj[j], zj[j1])), NA - 1, j, NA - 1, j1, j1 != j, ax[p], ay[p], az[p]);
         }
       }
     }
@@ -784,11 +812,12 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
   float f4[4][3];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const bool hi = i & 1;
     const int p = i / 2 < NP ? i / 2 : 0;
-    f4[i][0] = i < NA ? fmaf(s.f.frac[i], Fx, hi ? ax[p].y : ax[p].x) : 0.f;
-    f4[i][1] = i < NA ? fmaf(s.f.frac[i], Fy, hi ? ay[p].y : ay[p].x) : 0.f;
-    f4[i][2] = i < NA ? fmaf(s.f.frac[i], Fz, hi ? az[p].y : az[p].x) : 0.f;
+    // (an odd last atom's sums lie in both halves)
+    auto of = [&](float2 v) { return (NA & 1) && i == NA - 1 ? v.x + v.y : (i & 1) ? v.y : v.x; };
+    f4[i][0] = i < NA ? fmaf(s.f.frac[i], Fx, of(ax[p])) : 0.f;
+    f4[i][1] = i < NA ? fmaf(s.f.frac[i], Fy, of(ay[p])) : 0.f;
+    f4[i][2] = i < NA ? fmaf(s.f.frac[i], Fz, of(az[p])) : 0.f;
   }
   const unsigned mk = lane_group(G, lane);
   float r[3];
@@ -1237,32 +1266,55 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
     }
   };
   if (live) {
-    // bonded terms of atom g: harmonic bonds and angles, or FENE + WCA, on the listed
-    // intramolecular pairs
-    const real R02 = par<real>(s.fene_r02, s.f.fene_r02), K = par<real>(s.fene_k, s.f.fene_k);
-    // each lane walks its own atom's bonds (bond order), so a warp runs as many bond bodies
-    // as an atom has bonds, not as the molecule has
-    const unsigned bw = own ? s.bond_word[gg0] : 0u;
+    // bonded terms: harmonic bonds and angles, or FENE + WCA, on the listed intramolecular
+    // pairs.  A bond is evaluated once, by one of its atoms, in one of bond_rounds rounds (six
+    // bonds of a tetrahedron: two); the other atom gets the force by a shuffle.  Every lane of the
+    // group takes part in the shuffles.
+    const unsigned send = own ? s.bond_send[gg0] : 0u, recv = own ? s.bond_recv[gg0] : 0u;
+    auto give = [&](int q, real bx, real by, real bz) {
+      const int rv = (recv >> (4 * q)) & 15;
+      real tx, ty, tz;
+      if constexpr (P::fp64) {
+        tx = shfl_d(gmask, bx, base + (rv & 3));
+        ty = shfl_d(gmask, by, base + (rv & 3));
+        tz = shfl_d(gmask, bz, base + (rv & 3));
+      } else {
+        tx = __shfl_sync(gmask, bx, base + (rv & 3));
+        ty = __shfl_sync(gmask, by, base + (rv & 3));
+        tz = __shfl_sync(gmask, bz, base + (rv & 3));
+      }
+      if (rv & 8) {
+        fx -= tx;
+        fy -= ty;
+        fz -= tz;
+      }
+    };
     if (s.bond_model == 1) {
       const real kb = par<real>(s.bond_k, s.f.bond_k), r0 = par<real>(s.bond_r0, s.f.bond_r0);
 #pragma unroll
       for (int q = 0; q < kMaxBonds; ++q) {
-        if (q >= s.bmax) break;
-        const int e = (bw >> (4 * q)) & 15;
+        if (q >= s.bond_rounds) break;
+        const int e = (send >> (4 * q)) & 15;
         const auto oo = atom_off(e & 3);
-        if (q >= (int)(bw >> 28)) continue;
-        const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
-        const real d2 = dx * dx + dy * dy + dz * dz;
-        const real ird = Q::rsqrt_(d2);
-        const real dl = d2 * ird;
-        const real fr = -kb * (dl - r0) * ird;  // V = k/2 (r - r0)^2
-        fx += fr * dx;
-        fy += fr * dy;
-        fz += fr * dz;
-        if (ENERGY && (e & 8)) {
-          e_b += 0.5 * (double)kb * (double)(dl - r0) * (double)(dl - r0);
-          acc(vir, fr * d2);
+        real bx = 0, by = 0, bz = 0;
+        if (e & 8) {
+          const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
+          const real d2 = dx * dx + dy * dy + dz * dz;
+          const real ird = Q::rsqrt_(d2);
+          const real dl = d2 * ird;
+          const real fr = -kb * (dl - r0) * ird;  // V = k/2 (r - r0)^2
+          bx = fr * dx;
+          by = fr * dy;
+          bz = fr * dz;
+          fx = fma_(fr, dx, fx);
+          fy = fma_(fr, dy, fy);
+          fz = fma_(fr, dz, fz);
+          if (ENERGY) {
+            e_b += 0.5 * (double)kb * (double)(dl - r0) * (double)(dl - r0);
+            acc(vir, fr * d2);
+          }
         }
+        give(q, bx, by, bz);
       }
       // harmonic angles (i, vertex j, k): V = k/2 (theta - theta0)^2; the force on i is
       // dV/dtheta (v/(|u||v|) - cos(theta) u/|u|^2) / sin(theta), u = x_i - x_j, v = x_k - x_j,
@@ -1306,37 +1358,43 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
         }
       }
     } else {
+      const real R02 = par<real>(s.fene_r02, s.f.fene_r02), K = par<real>(s.fene_k, s.f.fene_k);
 #pragma unroll
-    for (int q = 0; q < kMaxBonds; ++q) {
-      if (q >= s.bmax) break;
-      const int e = (bw >> (4 * q)) & 15;
-      const auto oo = atom_off(e & 3);
-      if (q >= (int)(bw >> 28)) continue;
-      const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
-      const real d2 = dx * dx + dy * dy + dz * dz;
-      if (d2 >= R02) {
-        set_error(b.ctrl, ADRESS_ERR_BOND_BROKEN, a);
-        continue;
+      for (int q = 0; q < kMaxBonds; ++q) {
+        if (q >= s.bond_rounds) break;
+        const int e = (send >> (4 * q)) & 15;
+        const auto oo = atom_off(e & 3);
+        real bx = 0, by = 0, bz = 0;
+        if (e & 8) {
+          const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
+          const real d2 = dx * dx + dy * dy + dz * dz;
+          if (d2 >= R02) {
+            set_error(b.ctrl, ADRESS_ERR_BOND_BROKEN, a);
+          } else {
+            const real gg = (real)1 - (P::fp64 ? d2 * (real)s.fene_inv_r02 : Q::div_(d2, R02));
+            real fr = Q::div_(-K, gg);
+            if (ENERGY) {
+              if constexpr (std::is_same_v<Acc, Sum2>) acc_log(e_log, gg, b.log_tab);
+              else e_log += log((double)gg);
+            }
+            if (s.intra_wca && d2 < rc_at2) {
+              const real ir2 = Q::rcp_(d2);
+              const real sr2 = sig2 * ir2;
+              const real sr6 = sr2 * sr2 * sr2;
+              fr += (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2;
+              if (ENERGY) acc(e_b, (real)4 * eps * (sr6 * sr6 - sr6) + eps);
+            }
+            bx = fr * dx;
+            by = fr * dy;
+            bz = fr * dz;
+            fx = fma_(fr, dx, fx);
+            fy = fma_(fr, dy, fy);
+            fz = fma_(fr, dz, fz);
+            if (ENERGY) acc(vir, fr * d2);
+          }
+        }
+        give(q, bx, by, bz);
       }
-      const real gg = (real)1 - Q::div_(d2, R02);
-      real fr = Q::div_(-K, gg);
-      const bool first = ENERGY && (e & 8);  // accounts the bond's energy
-      if (first) {
-        if constexpr (std::is_same_v<Acc, Sum2>) acc_log(e_log, gg, b.log_tab);
-        else e_log += log((double)gg);
-      }
-      if (s.intra_wca && d2 < rc_at2) {
-        const real ir2 = Q::rcp_(d2);
-        const real sr2 = sig2 * ir2;
-        const real sr6 = sr2 * sr2 * sr2;
-        fr += (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2;
-        if (first) acc(e_b, (real)4 * eps * (sr6 * sr6 - sr6) + eps);
-      }
-      fx += fr * dx;
-      fy += fr * dy;
-      fz += fr * dz;
-      if (first) acc(vir, fr * d2);
-    }
     }
   }
   if (own) {
@@ -1464,18 +1522,9 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
         const double h2 = s.dt_m[g];
         const double nvx = fma(h2, fdx, vx), nvy = fma(h2, fdy, vy), nvz = fma(h2, fdz, vz);
         double y0 = fma(s.dt, nvx, xo[0]), y1 = fma(s.dt, nvy, xo[1]), y2 = fma(s.dt, nvz, xo[2]);
-        if (P::fp64) {
-          if (y0 < 0.0) y0 += B.L[0];
-          if (y0 >= B.L[0]) y0 -= B.L[0];
-          if (y1 < 0.0) y1 += B.L[1];
-          if (y1 >= B.L[1]) y1 -= B.L[1];
-          if (y2 < 0.0) y2 += B.L[2];
-          if (y2 >= B.L[2]) y2 -= B.L[2];
-        } else {
-          y0 = wrap_bits(y0, B.L[0], B.Lbits[0]);
-          y1 = wrap_bits(y1, B.L[1], B.Lbits[1]);
-          y2 = wrap_bits(y2, B.L[2], B.Lbits[2]);
-        }
+        y0 = wrap_bits(y0, B.L[0], B.Lbits[0]);
+        y1 = wrap_bits(y1, B.L[1], B.Lbits[1]);
+        y2 = wrap_bits(y2, B.L[2], B.Lbits[2]);
         b.v[i] = nvx;
         b.v[N + i] = nvy;
         b.v[2 * N + i] = nvz;
