@@ -282,6 +282,13 @@ __device__ __forceinline__ double minimg_cmp(double d, double L, double halfL) {
   return d;
 }
 
+// Minimum image for |d| < 1.5 L, the comparison on the bits (off the FP64 pipe).
+__device__ __forceinline__ double minimg_bits(double d, double L, double halfL) {
+  const long long b = __double_as_longlong(d), h = __double_as_longlong(halfL);
+  if ((b & 0x7fffffffffffffffll) > h) d -= b < 0 ? -L : L;
+  return d;
+}
+
 // ---- precision policies --------------------------------------------------------------
 struct P64 {
   using real = double;

@@ -10,25 +10,28 @@ namespace adress {
 
 // ---- deterministic FP64 reductions: per-block partials, then one fixed-order block ----
 
-template <int NV>
-__device__ __forceinline__ void block_partials(double (&v)[NV], double* part, int slot) {
-  __shared__ double sm[32][NV];
+// Block sums of four values into part[slot].  A warp's butterfly hands half of the values to
+// each half of its lanes at the first two levels, so that it takes 6 additions a lane instead of
+// 20 (the FP64 pipe is the bound); the additions that reach a sum, and their order, are those of
+// the plain butterfly.
+__device__ __forceinline__ void block_partials(const double (&v)[4], double* part, int slot) {
+  __shared__ double sm[32][4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const bool up = lane & 16, odd = lane & 8;
+  // lanes 0-15 take v[0], v[1], lanes 16-31 v[2], v[3]; then lanes with bit 3 clear the first
+  double a = up ? v[2] : v[0], c = up ? v[3] : v[1];
+  a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+  c += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+  double r = odd ? c : a;
+  r += __shfl_xor_sync(0xffffffffu, odd ? a : c, 8);
 #pragma unroll
-  for (int j = 0; j < NV; ++j)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) sm[w][j] = v[j];
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  if ((lane & 7) == 0) sm[w][lane >> 3] = r;
   __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      double acc = 0.0;
-      for (int q = 0; q < nw; ++q) acc += sm[q][j];
-      part[(size_t)slot * NV + j] = acc;
-    }
+  if (threadIdx.x < 4) {
+    double acc = 0.0;
+    for (int q = 0; q < nw; ++q) acc += sm[q][threadIdx.x];
+    part[(size_t)slot * 4 + threadIdx.x] = acc;
   }
 }
 
@@ -43,7 +46,7 @@ __global__ void __launch_bounds__(1024) k_reduce_parts(const double4_32a* part, 
     v[2] += r.z;
     v[3] += r.w;
   }
-  block_partials<4>(v, out, 0);
+  block_partials(v, out, 0);
 }
 
 template <int NA>
@@ -58,7 +61,7 @@ __global__ void __launch_bounds__(256) k_kinetic(const __grid_constant__ Sys s, 
       v[1 + d] = m * u;
     }
   }
-  block_partials<4>(v, b.part, blockIdx.x);
+  block_partials(v, b.part, blockIdx.x);
 }
 
 // Centre-of-mass x in double exactly as R = sum_k m_k (x_0 + minimg(x_k - x_0)) / M, wrapped.
@@ -185,20 +188,29 @@ __global__ void k_tf_update(const __grid_constant__ Sys s, Bufs b, double alpha)
 // states) and the resolution values the force kernels use.
 __global__ void k_clear_samples(long long* n) { *n = 0; }
 
+// (Wraps and minimum images by comparing bits, and no division where the molecule's mass is a
+// power of two: the same values with a fifth of the FP64 operations.)
 template <int NA>
 __global__ void k_export_com(const __grid_constant__ Sys s, Bufs b, double* com, double* w) {
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= s.M) return;
   const Box& B = box_of(s, b, a);
   const size_t N = (size_t)s.N;
-  double acc[3] = {0.0, 0.0, 0.0};
+  const bool pow2 = (__double_as_longlong(s.Mtot) & 0xFFFFFFFFFFFFFll) == 0 && s.Mtot > 1e-300 && s.Mtot < 1e300;
+  const double inv_m = __longlong_as_double((2046ll << 52) - __double_as_longlong(s.Mtot));  // 1 / Mtot of a power of two
+#pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const double x0 = b.x[d * N + a * NA];
+    const double x0 = b.x[d * N + (size_t)a * NA];
+    double acc = 0.0;
+#pragma unroll
     for (int k = 0; k < NA; ++k)
-      acc[d] += s.mass[k] * (x0 + minimg_cmp(b.x[d * N + a * NA + k] - x0, B.L[d], B.halfL[d]));
-    double r = acc[d] / s.Mtot;
-    r -= B.L[d] * floor(r / B.L[d]);
-    if (r >= B.L[d]) r -= B.L[d];
+      acc += s.mass[k] * (x0 + minimg_bits(b.x[d * N + (size_t)a * NA + k] - x0, B.L[d], B.halfL[d]));
+    double r = pow2 ? acc * inv_m : acc / s.Mtot;
+    const long long bits = __double_as_longlong(r);
+    if (bits < 0 || bits >= B.Lbits[d]) {  // outside [0, L)
+      r -= B.L[d] * floor(r / B.L[d]);
+      if (r >= B.L[d]) r -= B.L[d];
+    }
     com[(size_t)d * s.M + a] = r;
   }
   if (w) {
@@ -309,8 +321,10 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
         // first own molecule (sorted position) this candidate pairs with: all of them for another
         // cell of the half set, else those before it
         const int upto = !in ? hs : (half && cc != 13 ? he : min(he, g));
+        int4 Hn = __ldg(&q.sorted[hs]);
         for (int h = hs; h < he; ++h) {
-          const int4 H = q.sorted[h];
+          const int4 H = Hn;
+          if (h + 1 < he) Hn = __ldg(&q.sorted[h + 1]);
           const float dx = (float)(int)((unsigned)H.x - (unsigned)D.x) * sx;
           const float dy = (float)(int)((unsigned)H.y - (unsigned)D.y) * sy;
           const float dz = (float)(int)((unsigned)H.z - (unsigned)D.z) * sz;

@@ -131,13 +131,6 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   y = fma(fma(-h * y, y, 0.5), y, y);
   return fma(fma(-h * y, y, 0.5), y, y);
 }
-// Minimum image for |d| < 1.5 L, the comparison on the bits (off the FP64 pipe).
-__device__ __forceinline__ double minimg_bits(double d, double L, double halfL) {
-  const long long b = __double_as_longlong(d), h = __double_as_longlong(halfL);
-  if ((b & 0x7fffffffffffffffll) > h) d -= b < 0 ? -L : L;
-  return d;
-}
-
 // ---------------- precision policies for the pair loop --------------------------------
 
 template <class P>
