@@ -215,7 +215,7 @@ adress_status adress_compute_forces(adress_handle h, double* energies);
  * mapping), one fused kernel per further step (forces, thermostat, both half kicks,
  * drift, next mapping), one last kernel (forces, thermostat, second half kick); after each
  * mapping a cooperative list kernel decides on a rebuild and, if needed, does it.  Small
- * systems run all middle steps (between density samples) in one cooperative kernel.
+ * systems run all middle steps, density samples included, in one cooperative kernel.
  * Asynchronous; errors surface at adress_check.  With the environment variable ADRESS_EAGER=1
  * set before adress_init, the same kernels are launched one by one, without a graph. */
 adress_status adress_step(adress_handle h, int32_t nsteps);

@@ -931,31 +931,29 @@ adress_status adress_compute_forces(adress_handle h, double* energies) {
 //   prologue (half kick + drift + mapping) -> decision and lists
 //   { fused step -> decision and lists } x (nsteps - 1)
 //   last step (thermostat + second half kick, v and f stored)
-// with a density sample after every sample_every-th mapping and the thermodynamic-force
-// update at the end.  The middle runs as one kernel per stretch between samples where that is
-// faster (run_kernel_pays), else as a step and a list kernel per step.
+// with a density sample after every sample_every-th mapping and the thermodynamic-force update at
+// the end.  The middle runs as one kernel, which samples as it maps, where that is faster
+// (run_kernel_pays), else as a step and a list kernel per step.
 static cudaError_t launch_steps(adress_handle h, int nsteps, int sample_every, int tf_update, double alpha,
                                 cudaStream_t st) {
   const Sys& s = h->sys;
   const Bufs& b = h->buf;
   const DecideArgs da{0, 1, 1};
   const bool run = run_kernel_pays(s);
+  auto sample = [&](int level) {
+    return sample_every > 0 && level % sample_every == 0 ? launch_density(s, b, h->precision, st) : cudaSuccess;
+  };
   cudaError_t e = launch_map(s, b, h->precision, 1, st);
   if (e == cudaSuccess) e = launch_lists(s, b, da, st);
-  int done = 1;  // mappings so far: positions of time level `done` are current
-  while (e == cudaSuccess) {
-    if (sample_every > 0 && done % sample_every == 0) e = launch_density(s, b, h->precision, st);
-    if (e != cudaSuccess || done >= nsteps) break;
-    if (run) {
-      int m = nsteps - done;
-      if (sample_every > 0) m = std::min(m, sample_every - done % sample_every);
-      e = launch_run(s, b, h->precision, m, st);
-      done += m;
-    } else {
+  if (e == cudaSuccess) e = sample(1);
+  if (run && nsteps > 1) {
+    if (e == cudaSuccess) e = launch_run(s, b, h->precision, 1, nsteps - 1, sample_every, st);
+  } else {
+    for (int level = 2; level <= nsteps && e == cudaSuccess; ++level) {
       if (s.cg_mode) e = mlp_pairs(s, b, h->mlp_args(), b.fpair, st);
       if (e == cudaSuccess) e = launch_step(s, b, h->precision, 2, 0, st);
       if (e == cudaSuccess) e = launch_lists(s, b, da, st);
-      ++done;
+      if (e == cudaSuccess) e = sample(level);
     }
   }
   if (e == cudaSuccess && s.cg_mode) e = mlp_pairs(s, b, h->mlp_args(), b.fpair, st);

@@ -318,8 +318,9 @@ cudaError_t device_exclusive_scan(const int* in, int* out, int n, int* tmp, int*
 // mode: 0 conservative forces, 1 last step of a run (thermostat + second half kick),
 // 2 fused step (thermostat + both half kicks + drift + next mapping)
 cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
-// nsteps fused steps, each with its rebuild decision and lists, in one cooperative launch.
-cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
+// nsteps fused steps after mapping `done`, each with its rebuild decision and lists, in one
+// cooperative launch; every sample_every-th mapping is added to the density profile.
+cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int done, int nsteps, int sample_every, cudaStream_t st);
 // Whether launch_run is the faster way to advance this system (tabulated CG force only).
 bool run_kernel_pays(const Sys& s);
 

@@ -7,7 +7,7 @@ namespace adress {
 
 cudaError_t launch_step_ljrf(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
 cudaError_t launch_step_hadress(const Sys& s, const Bufs& b, int precision, int mode, int energy, cudaStream_t st);
-cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st);
+cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int done, int nsteps, int sample_every, cudaStream_t st);
 
 template <class P, int NA>
 static void launch_prologue_na(const Sys& s, const Bufs& b, int integrate, cudaStream_t st) {
@@ -56,12 +56,12 @@ cudaError_t launch_step(const Sys& s, const Bufs& b, int precision, int mode, in
 }
 
 template <class P>
-static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
+static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int done, int nsteps, int sample_every, cudaStream_t st) {
   switch (s.NA) {
-    case 1: return launch_run_na<P, 1, 0, false>(s, b, nsteps, st);
-    case 2: return launch_run_na<P, 2, 0, false>(s, b, nsteps, st);
-    case 3: return launch_run_na<P, 3, 0, false>(s, b, nsteps, st);
-    default: return launch_run_na<P, 4, 0, false>(s, b, nsteps, st);
+    case 1: return launch_run_na<P, 1, 0, false>(s, b, done, nsteps, sample_every, st);
+    case 2: return launch_run_na<P, 2, 0, false>(s, b, done, nsteps, sample_every, st);
+    case 3: return launch_run_na<P, 3, 0, false>(s, b, done, nsteps, sample_every, st);
+    default: return launch_run_na<P, 4, 0, false>(s, b, done, nsteps, sample_every, st);
   }
 }
 
@@ -74,10 +74,10 @@ bool run_kernel_pays(const Sys& s) {
   return !s.cg_mode && s.nb_model == 0 && s.M <= (s.fp64 ? 32ll : 160ll) * s.n_sm;
 }
 
-cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
-  if (s.scheme == 1) return launch_run_hadress(s, b, precision, nsteps, st);
+cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int done, int nsteps, int sample_every, cudaStream_t st) {
+  if (s.scheme == 1) return launch_run_hadress(s, b, precision, done, nsteps, sample_every, st);
   if (s.nb_model == 1) return cudaErrorInvalidValue;
-  return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, nsteps, st) : launch_run_p<P32>(s, b, nsteps, st);
+  return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, done, nsteps, sample_every, st) : launch_run_p<P32>(s, b, done, nsteps, sample_every, st);
 }
 
 }  // namespace adress

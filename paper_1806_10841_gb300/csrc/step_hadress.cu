@@ -27,17 +27,17 @@ cudaError_t launch_step_hadress(const Sys& s, const Bufs& b, int precision, int 
 }
 
 template <class P>
-static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
+static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int done, int nsteps, int sample_every, cudaStream_t st) {
   switch (s.NA) {
-    case 1: return launch_run_na<P, 1, 0, true>(s, b, nsteps, st);
-    case 2: return launch_run_na<P, 2, 0, true>(s, b, nsteps, st);
-    case 3: return launch_run_na<P, 3, 0, true>(s, b, nsteps, st);
-    default: return launch_run_na<P, 4, 0, true>(s, b, nsteps, st);
+    case 1: return launch_run_na<P, 1, 0, true>(s, b, done, nsteps, sample_every, st);
+    case 2: return launch_run_na<P, 2, 0, true>(s, b, done, nsteps, sample_every, st);
+    case 3: return launch_run_na<P, 3, 0, true>(s, b, done, nsteps, sample_every, st);
+    default: return launch_run_na<P, 4, 0, true>(s, b, done, nsteps, sample_every, st);
   }
 }
 
-cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int nsteps, cudaStream_t st) {
-  return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, nsteps, st) : launch_run_p<P32>(s, b, nsteps, st);
+cudaError_t launch_run_hadress(const Sys& s, const Bufs& b, int precision, int done, int nsteps, int sample_every, cudaStream_t st) {
+  return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, done, nsteps, sample_every, st) : launch_run_p<P32>(s, b, done, nsteps, sample_every, st);
 }
 
 }  // namespace adress

@@ -393,9 +393,9 @@ __device__ __forceinline__ void com_fp64(const Sys& s, const Box& B, unsigned gm
 
 // Map one molecule: fixed-point centre, resolution value, offsets, region flag.
 // P32: integer fixed-point arithmetic (exact, periodic) on the bits of the doubles.
-template <int NA>
+template <int NA, bool SAMPLE>
 __device__ __forceinline__ void map_group32(const Sys& s, const Box& B, const Bufs& b, int nxt, int a, int g, unsigned gmask,
-                                            int base, bool live, const double x[3], const int4 ref, float& ext2,
+                                            int base, bool live, const double x[3], const int4 ref, int sample, float& ext2,
                                             float& disp2) {
   const bool own = live && g < NA;
   unsigned Pk[3], P0[3], R[3];
@@ -431,18 +431,29 @@ __device__ __forceinline__ void map_group32(const Sys& s, const Box& B, const Bu
                                     : (float)(int)(R[0] - B.xc32) * B.fx_scale[0];
   float dd = fabsf(dxc);
   const bool near = fabsf(dd - B.d_at_f) < B.near_at || fabsf(dd - B.d_hyend_f) < B.near_hyend;
-  int region;  // 0 AT, 1 hybrid, 2 CG
-  if (__any_sync(gmask, live && near)) {
-    double dxd;
+  // the distance in FP64 as the definition forms it (all lanes of the group call)
+  auto exact_distance = [&]() -> double {
     if (s.n_centers > 0) {
       double R64[3];
       com_fp64<NA>(s, B, gmask, base, x, R64);
       int k64;
-      dxd = nearest_center64(s, B, b, gmask, g, R64, k64);
-    } else {
-      const double rx = com_x_fp64<NA>(s, B, gmask, base, g, x[0]);
-      dxd = fabs(minimg_cmp(rx - B.xc, B.L[0], B.halfL[0]));
+      return nearest_center64(s, B, b, gmask, g, R64, k64);
     }
+    const double rx = com_x_fp64<NA>(s, B, gmask, base, g, x[0]);
+    return fabs(minimg_cmp(rx - B.xc, B.L[0], B.halfL[0]));
+  };
+  if (SAMPLE && sample) {
+    // density profile: the bin of |dxc|, decided in FP64 within 1e-4 of a bin edge (global
+    // atomics: right for the run kernel's few molecules; 200,000 of them cost 20 us a sample,
+    // k_density's shared-memory counts 8)
+    const float u = dd * s.f.tf_inv_dx, fl = floorf(u), fr = u - fl;
+    int k = (int)fl;
+    if (__any_sync(gmask, live && (fr < 1e-4f || fr > 1.f - 1e-4f))) k = (int)floor(exact_distance() / s.tf_dx);
+    if (live && g == 0 && k < s.tf_n) atomicAdd(&b.hist[B.tf0 + k], 1ull);
+  }
+  int region;  // 0 AT, 1 hybrid, 2 CG
+  if (__any_sync(gmask, live && near)) {
+    const double dxd = exact_distance();
     region = dxd < B.d_at ? 0 : (dxd >= B.d_at + B.d_hy ? 2 : 1);
   } else {
     region = dd < B.d_at_f ? 0 : (dd >= B.d_hyend_f ? 2 : 1);
@@ -469,9 +480,9 @@ __device__ __forceinline__ void map_group32(const Sys& s, const Box& B, const Bu
 
 // P64: the mapping in double precision; comparisons and the fixed-point copy run on the integer
 // pipe (the FP64 one runs 2 lanes a clock per SM).
-template <int NA>
+template <int NA, bool SAMPLE>
 __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bufs& b, int nxt, int a, int g, unsigned gmask,
-                                            int base, bool live, const double x[3], const int4 ref, float& ext2,
+                                            int base, bool live, const double x[3], const int4 ref, int sample, float& ext2,
                                             float& disp2) {
   const bool own = live && g < NA;
   double dl[3], c[3], R[3];
@@ -503,6 +514,10 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
                                      : minimg_cmp(R[0] - B.xc, B.L[0], B.halfL[0]);
   if (live && g == 0) {
     const double dd = fabs(dxc);
+    if (SAMPLE && sample) {
+      const int k = (int)floor(dd / s.tf_dx);
+      if (k < s.tf_n) atomicAdd(&b.hist[B.tf0 + k], 1ull);
+    }
     double w;
     if (dd < B.d_at) w = 1.0;
     else if (dd >= B.d_at + B.d_hy) w = 0.0;
@@ -588,8 +603,8 @@ __global__ void __launch_bounds__(kMaxForceBlock) k_prologue(const __grid_consta
     }
   }
   float ext2 = 0.f, disp2 = 0.f;
-  if (P::fp64) map_group64<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
-  else map_group32<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, disp2);
+  if (P::fp64) map_group64<NA, false>(s, B, b, nxt, a, g, gmask, base, live, x, ref, 0, ext2, disp2);
+  else map_group32<NA, false>(s, B, b, nxt, a, g, gmask, base, live, x, ref, 0, ext2, disp2);
   publish_extent(b, 0, ext2, disp2);
 }
 
@@ -1071,15 +1086,16 @@ __device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bu
 
 // The step of the molecules of one tile of the grid (a block's worth of threads): thread gtid
 // of the whole grid.  cur: current half of the molecule arrays; step: the time level of the
-// forces; ext_now: the largest atom-to-COM distance; the next mapping's maxima are merged into
-// ext2 and disp2 (MODE_FUSED).  Every thread of a block calls.
+// forces; ext_now: the largest atom-to-COM distance; sample (SAMPLE): add the next mapping's
+// molecules to the density profile; its maxima are merged into ext2 and disp2 (MODE_FUSED).  Every thread of a block calls.
 //
 // A high-resolution work item takes 2^ln.h lanes and a coarse-grained one 2^ln.c (32 >= 2^h >=
 // 2^c >= 4, so that no item's lanes straddle a warp); the first four integrate and map the
 // molecule, one lane per atom.  LPN: one lane per neighbour (hr_forces32), else per atom.
-template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, bool LPN>
+template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, bool LPN, bool SAMPLE>
 __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lanes ln, const int gtid, const int cur,
-                                          const long long step, const float ext_now, float& ext2, float& disp2) {
+                                          const long long step, const float ext_now, const int sample, float& ext2,
+                                          float& disp2) {
   using Q = Prec<P>;
   using real = typename Q::real;
   const int lane = threadIdx.x & 31, g = threadIdx.x & 3, base = lane & ~3;
@@ -1538,8 +1554,8 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
       }
       const int nxt = cur ^ 1;
       float d2 = 0.f;
-      if (P::fp64) map_group64<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, d2);
-      else map_group32<NA>(s, B, b, nxt, a, g, gmask, base, live, x, ref, ext2, d2);
+      if (P::fp64) map_group64<NA, SAMPLE>(s, B, b, nxt, a, g, gmask, base, live, x, ref, sample, ext2, d2);
+      else map_group32<NA, SAMPLE>(s, B, b, nxt, a, g, gmask, base, live, x, ref, sample, ext2, d2);
       disp2 = fmaxf(disp2, d2);
     }
   }
@@ -1568,8 +1584,8 @@ __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULT
   const Lanes ln = lanes_of<FORM, P, MODEL>(s.step_lanes);
   // blocks past the last item (the host does not know the number of high-resolution items)
   if (!ENERGY && ln.h != ln.c && blockIdx.x * blockDim.x >= (unsigned)((c->n_hr << ln.h) + ((s.M - c->n_hr) << ln.c))) return;
-  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS, LPN>(s, b, ln, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
-                                                        c->ext_now, ext2, disp2);
+  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS, LPN, false>(s, b, ln, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
+                                                        c->ext_now, 0, ext2, disp2);
   if (MODE == MODE_FUSED) publish_extent(b, 0, ext2, disp2);
 }
 
@@ -1582,11 +1598,13 @@ constexpr int run_min_blocks() {
   return P::fp64 ? 3 : 4;
 }
 
-// nsteps fused steps in one cooperative launch: every block takes its tiles of the step, a
+// nsteps fused steps after mapping `done` in one cooperative launch (a density sample after every
+// sample_every-th mapping): every block takes its tiles of the step, a
 // grid barrier ends the mapping, every block takes the rebuild decision itself and the grid
 // rebuilds the lists when needed.  For small systems (run_kernel_pays).
 template <class P, int NA, bool MULTI, int MODEL, bool HS>
-__global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, int nsteps) {
+__global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, int done, int nsteps,
+                                                                              int sample_every) {
   Ctrl* c = b.ctrl;
   if (__syncthreads_or(threadIdx.x == 0 && __ldcg(&c->dead) != 0)) return;  // a grid barrier gave up earlier
   int cur = c->parity, set = 0, dirty = 0, rebuilt = 0;
@@ -1597,11 +1615,12 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
   GridBarrier bar(c, &c->bar[1]);
   for (int k = 0; k < nsteps; ++k) {
     float ext2 = 0.f, disp2 = 0.f;
+    const int sample = sample_every > 0 && (done + k + 1) % sample_every == 0;
     const int n_hr = c->n_hr;
     const int ntiles = ((n_hr << ln.h) + ((s.M - n_hr) << ln.c) + blockDim.x - 1) / blockDim.x;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, LPN>(s, b, ln, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
-                                                                ext2, disp2);
+      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, LPN, true>(s, b, ln, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
+                                                                sample, ext2, disp2);
     publish_extent(b, set, ext2, disp2);
     if (!bar.sync()) return;
     const Decision d = decide_rebuild(s, c, set, 0);
@@ -1610,6 +1629,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
       // publishes to it
       c->ext_slot[(set + 2) % 3][0][threadIdx.x] = 0u;
       c->ext_slot[(set + 2) % 3][1][threadIdx.x] = 0u;
+      if (threadIdx.x == 0 && sample) *b.nsamples += 1;
       if (threadIdx.x == 0 && d.too_wide) set_error(c, ADRESS_ERR_EXTENT, (int)(d.ext * 1000));
     }
     cur ^= 1;
@@ -1670,7 +1690,7 @@ static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cu
 
 // As many blocks as fit on the device at once, at most one per tile.
 template <class P, int NA, int MODEL, bool HS>
-static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int nsteps, cudaStream_t st) {
+static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int done, int nsteps, int sample_every, cudaStream_t st) {
   const int tiles = ceil_div((long long)s.M << (P::fp64 ? 2 : s.run_lanes.h), s.force_block);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(tiles, s.n_sm * run_min_blocks<P>()));
@@ -1681,8 +1701,8 @@ static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int nsteps, cudaSt
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (s.nbox > 1) return cudaLaunchKernelEx(&cfg, k_run<P, NA, true, MODEL, HS>, s, b, nsteps);
-  return cudaLaunchKernelEx(&cfg, k_run<P, NA, false, MODEL, HS>, s, b, nsteps);
+  if (s.nbox > 1) return cudaLaunchKernelEx(&cfg, k_run<P, NA, true, MODEL, HS>, s, b, done, nsteps, sample_every);
+  return cudaLaunchKernelEx(&cfg, k_run<P, NA, false, MODEL, HS>, s, b, done, nsteps, sample_every);
 }
 
 }  // namespace adress
