@@ -336,6 +336,12 @@ __global__ void __launch_bounds__(128) k_mlp_forward(MlpDev m, const float* __re
   }
 }
 
+// Programmatic dependent launch of the training kernels: the next kernel may be scheduled once
+// every block of this one has called allow_dependent_launch (or left), and loads what the kernels
+// still running do not write before wait_for_primary, which returns when they have completed.
+__device__ __forceinline__ void allow_dependent_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------- loss and gradient of one block of 64 samples ---------------------------
 // Writes the block's partial gradient (sum over its samples of dL/dparam with
 // L = (1/n) sum (y - t/out_scale)^2) and loss partial to part[blockIdx.x].  Sample i of the n is
@@ -365,15 +371,21 @@ __global__ void __launch_bounds__(128) k_mlp_grad(MlpDev m, const float* __restr
     ftile[w][e] = s >= 0 ? feat[s * kIn + e % kIn] : 0.f;
   }
   __syncwarp();
-  const MlpView mv = view_of(m);
+  // (the inputs need the normalisation only; the parameters are read after the wait)
+  const MlpView mv{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, m.norm, m.norm + 2 * kIn + 1};
   unsigned ax[4];
   input_fragment(mv, ftile[w], ax);
+  const bool vg = base + g < n, vg8 = base + g + 8 < n;
+  const float t0 = vg ? target[srow[w][g]] : 0.f, t8 = vg8 ? target[srow[w][g + 8]] : 0.f;
+  // up to here nothing that the previous optimiser step writes was read; the next one may start
+  // loading what this kernel does not write
+  wait_for_primary();
+  allow_dependent_launch();
   Tile T;
   float yg, yg8;
-  tile_forward(mv, ax, T, yg, yg8);
-  const bool vg = base + g < n, vg8 = base + g + 8 < n;
-  const float rg = vg ? yg - target[srow[w][g]] * inv_scale : 0.f;
-  const float rg8 = vg8 ? yg8 - target[srow[w][g + 8]] * inv_scale : 0.f;
+  tile_forward(view_of(m), ax, T, yg, yg8);
+  const float rg = vg ? yg - t0 * inv_scale : 0.f;
+  const float rg8 = vg8 ? yg8 - t8 * inv_scale : 0.f;
   const float dyg = 2.f * rg / (float)n, dyg8 = 2.f * rg8 / (float)n;
   // layer 2 deltas, bias / w3 partials, and stores for the weight-gradient products
   const float* w3 = m.P + ow3;
@@ -567,18 +579,19 @@ __global__ void k_mlp_grad_reduce(const float* part, int nblk, float* grad) {
 // loads in flight), Adam on the FP32 master parameter, and its bfloat16 operand copies.  As four
 // kernels (reduction, Adam, packing, and the gather of the next batch) a batch of 4096 spent most
 // of its 45 us in launches and their gaps.
-__global__ void __launch_bounds__(128) k_mlp_update(const float* __restrict__ part, int nblk, float* __restrict__ P,
-                                                    float* __restrict__ mom, float* __restrict__ vel, float* loss_acc, float lr,
-                                                    float b1c, float b2c, __nv_bfloat16* __restrict__ W1,
-                                                    __nv_bfloat16* __restrict__ W2, __nv_bfloat16* __restrict__ W2T) {
+__global__ void __launch_bounds__(128) k_mlp_update(const float* part, int nblk, float* P, float* mom, float* vel, float* loss_acc, float lr,
+                                                    float b1c, float b2c, __nv_bfloat16* W1, __nv_bfloat16* W2,
+                                                    __nv_bfloat16* W2T) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kNPar) return;
+  allow_dependent_launch();
   float mo = 0.f, ve = 0.f, old = 0.f;
-  if (p < kNPar) {
+  if (p < kNPar) {  // written by the previous optimiser step, complete before the gradient kernel let this one start
     mo = mom[p];
     ve = vel[p];
     old = P[p];
   }
+  wait_for_primary();
+  if (p > kNPar) return;
   float gr = 0.f;
   int b = 0;
   for (; b + 16 <= nblk; b += 16) {
@@ -822,7 +835,8 @@ __device__ __forceinline__ bool needs_network(const Sys& s, const Box& X, const 
 
 // Both orderings of a pair's features, normalised (mean, 1/std in sn) and packed as bf16
 // pairs the way the evaluation kernels read their A operands.
-__device__ __forceinline__ void pack_pair_inputs(const float f[9], const float (*sn)[kIn], unsigned* out) {
+__device__ __forceinline__ void pack_pair_inputs(const float f[9], const float (*sn)[kIn], uint2* out) {
+  unsigned v10[10];
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -834,8 +848,10 @@ __device__ __forceinline__ void pack_pair_inputs(const float f[9], const float (
         const int src = (u == 0 || k == 0) ? k : (k < 5 ? k + 4 : k - 4);
         v[h] = k < kIn ? (f[src < kIn ? src : 0] - sn[0][k < kIn ? k : 0]) * sn[1][k < kIn ? k : 0] : 0.f;
       }
-      out[5 * u + w] = pack_bf16(v[0], v[1]);
+      v10[5 * u + w] = pack_bf16(v[0], v[1]);
     }
+#pragma unroll
+  for (int w = 0; w < 5; ++w) out[w] = make_uint2(v10[2 * w], v10[2 * w + 1]);
 }
 
 // Pairs that need the network this step, from the candidates of the last build: the force
@@ -878,7 +894,7 @@ __global__ void __launch_bounds__(128) k_mlp_feat(const __grid_constant__ Sys s,
       set_error(b.ctrl, ADRESS_ERR_LIST_OVERFLOW, (int)p);
       continue;
     }
-    pack_pair_inputs(f, sn, b.pfrag + p * 10);
+    pack_pair_inputs(f, sn, reinterpret_cast<uint2*>(b.pfrag + p * 10));
     b.pslot[p] = make_int2(rec.x, rec.y);
   }
 }
@@ -1098,11 +1114,21 @@ cudaError_t mlp_train_batch(const MlpDevArgs& a, const float* feat, const float*
                             float* part, float* mom, float* vel, float* loss_acc, float lr, int step, cudaStream_t st) {
   const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
   const int nblk = (int)((n + 63) / 64);
-  k_mlp_grad<<<nblk, 128, 0, st>>>(m, feat, target, n, order, part);
   const float b1c = 1.f - powf(0.9f, (float)step), b2c = 1.f - powf(0.999f, (float)step);
-  k_mlp_update<<<(kNPar + 1 + 127) / 128, 128, 0, st>>>(part, nblk, (float*)a.P, mom, vel, loss_acc, lr, b1c, b2c,
-                                                        (__nv_bfloat16*)a.W1p, (__nv_bfloat16*)a.W2p, (__nv_bfloat16*)a.W2Tp);
-  return cudaGetLastError();
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(nblk);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_mlp_grad, m, feat, target, n, order, part);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3((kNPar + 1 + 127) / 128);
+  return cudaLaunchKernelEx(&cfg, k_mlp_update, (const float*)part, nblk, (float*)a.P, mom, vel, loss_acc, lr, b1c, b2c,
+                            (__nv_bfloat16*)a.W1p, (__nv_bfloat16*)a.W2p, (__nv_bfloat16*)a.W2Tp);
 }
 
 cudaError_t mlp_pack(const MlpDevArgs& a, cudaStream_t st) {
