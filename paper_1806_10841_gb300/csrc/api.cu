@@ -638,6 +638,14 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
     nmol[k] = cfgs[k].n_mols;
     mol0 += cfgs[k].n_mols;
   }
+  {
+    // a separation's error in the FP32 tests: 2^-32 L per component of either centre, some 1e-6 of
+    // the cutoff in float arithmetic; several times both, for the square
+    double lmax = 0.0;
+    for (const Box& B : h->boxes)
+      for (int d = 0; d < 3; ++d) lmax = std::max(lmax, B.L[d]);
+    s.f.pretest = (float)(1.0 + 1e-4 + 32.0 * lmax / 4294967296.0 / std::min(c->rc_at, c->rc_cg));
+  }
   h->skin0 = c->skin;
   s.r_list = std::max(c->rc_cg, c->rc_at + 2.0 * c->r_ext) + c->skin;
   s.cap = c->max_neighbors > 0 ? std::min(c->max_neighbors, s.M - 1) : auto_capacity(s, h->boxes, nmol);

@@ -947,9 +947,9 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
 // Eq. 1 on a high-resolution molecule a of the FP64 path: lane g has atom g, lane group `sub` of
 // SPLIT every SPLIT-th neighbour.  The FP64 pipe is the bound (2 lanes a clock per SM against
 // 128 in FP32), and nine of ten listed atom pairs are beyond the cutoff, so a batch of
-// neighbours is first tested in FP32 with a margin (fixed-point centres and float offsets, errors
-// below 1e-5 of the cutoff against a margin of 1e-4) and only what passes is evaluated, and
-// tested again, in FP64; the coarse-grained force of a pair is evaluated by one lane of the
+// neighbours is first tested in FP32 with a margin (fixed-point centres and float offsets; the
+// margin, Sys::f.pretest, covers both and grows with the box) and only what passes is evaluated,
+// and tested again, in FP64; the coarse-grained force of a pair is evaluated by one lane of the
 // group.  800k atoms: 930 -> 516 us a step, 80k atoms all-atomistic 216 -> 80 us.
 template <int NA, bool ENERGY, int MODEL, bool HS, int SPLIT>
 __device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int g, int sub, int nnb,
@@ -959,9 +959,8 @@ __device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bu
                                             double& fx, double& fy, double& fz, double& dv, double& e_at, double& e_cg,
                                             double& vir) {
   using Q = Prec<P64>;
-  constexpr float kMargin = 1.0001f;
   constexpr int kBatch = 16;  // neighbours per batch: four hit bits each
-  const float rcf = s.f.rc_at2 * kMargin, rcgf = s.f.rc_cg2 * kMargin, reachf = (float)reach_at2 * kMargin;
+  const float rcf = s.f.rc_at2 * s.f.pretest, rcgf = s.f.rc_cg2 * s.f.pretest, reachf = (float)reach_at2 * s.f.pretest;
   const int4 Cf = b.com_fx[cur][a];
   const float waf = __int_as_float(Cf.w);
   const float* of = (const float*)(b.off32[cur] + 3 * (size_t)a) + (g < NA ? g : 0);
@@ -1212,7 +1211,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
     // path tests the fixed-point ones in FP32 with a margin first (see hr_forces64)
     const int4* cfx = b.com_fx[cur];
     const int4 Cf = P::fp64 ? cfx[a] : (const int4&)Ca;
-    const float rcgf = P::fp64 ? s.f.rc_cg2 * 1.0001f : s.f.rc_cg2;
+    const float rcgf = P::fp64 ? s.f.rc_cg2 * s.f.pretest : s.f.rc_cg2;
     int m_n = m_first, m_n2 = 0;
     int4 C_n = Cf, C_n2 = Cf;
     if (lig < nnb_cg) C_n = cfx[m_n];

@@ -9,13 +9,13 @@ from paper_1806_10841_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("na", [1, 4])
-@pytest.mark.parametrize("L", [24.0, 800.0])
+# (in the longest box the fixed-point centres are good to 2e-5, the coordinates to 1e-11)
+@pytest.mark.parametrize("na,L,nearest", [(1, 24.0, -11), (4, 24.0, -11), (1, 800.0, -11), (4, 800.0, -11), (1, 1.0e5, -9)])
 @pytest.mark.parametrize("scheme", [0, 1])
-def test_pairs_at_the_cutoffs(na, L, scheme):
+def test_pairs_at_the_cutoffs(na, L, nearest, scheme):
     from paper_1806_10841_gb300 import adress
 
-    n = 40  # molecule pairs, centres a cutoff apart to within 1e-11 .. 1e-5 of it
+    n = 40  # molecule pairs, centres a cutoff apart to within 10^nearest .. 1e-5 of it
     box = (L, 24.0, 24.0)
     s = inputs.tetra_system(2 * n, box, 8.0, 4.0, seed=2, scheme=scheme)
     s.na, s.mass = na, np.ones(na)
@@ -32,7 +32,7 @@ def test_pairs_at_the_cutoffs(na, L, scheme):
         u = rng.normal(size=3)
         u /= np.linalg.norm(u)
         rc = s.rc_cg if k % 2 else s.rc_at
-        d = rc * (1 + rng.choice([-1, 1]) * 10.0 ** rng.uniform(-11, -5))
+        d = rc * (1 + rng.choice([-1, 1]) * 10.0 ** rng.uniform(nearest, -5))
         x[2 * k] = c + body
         x[2 * k + 1] = c + d * u + (body if na == 1 or k % 2 else -body)
     x = np.mod(x.reshape(-1, 3), np.array(box))
