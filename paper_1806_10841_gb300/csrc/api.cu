@@ -210,6 +210,18 @@ static void schedule_bonds(Sys& s) {
   for (int g = 0; g < kMaxNA; ++g) s.bond_send[g] = s.bond_recv[g] = 0;
   s.bond_rounds = 0;
   while (!place_bonds(s, 0, s.bond_rounds)) ++s.bond_rounds;  // nb rounds always do
+  int cnt[kMaxNA] = {};
+  for (int g = 0; g < kMaxNA; ++g) s.bond_word[g] = 0;
+  for (int q = 0; q < s.nb; ++q) {
+    const int p0 = s.bonds[2 * q], p1 = s.bonds[2 * q + 1];
+    s.bond_word[p0] |= (unsigned)(p1 | 8) << (4 * cnt[p0]++);
+    s.bond_word[p1] |= (unsigned)p0 << (4 * cnt[p1]++);
+  }
+  s.bond_max = 0;
+  for (int g = 0; g < kMaxNA; ++g) {
+    s.bond_word[g] |= (unsigned)cnt[g] << 28;
+    s.bond_max = std::max(s.bond_max, cnt[g]);
+  }
 }
 
 // Validation of one configuration; empty when valid.

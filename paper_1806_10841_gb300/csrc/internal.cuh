@@ -108,6 +108,10 @@ struct Sys {
   // bond_recv[i] nibble q & 3 evaluates (bit 3: there is one)
   unsigned bond_send[kMaxNA], bond_recv[kMaxNA];
   int bond_rounds;
+  // per-atom bond partners in bond order, a nibble each (bit 3: this atom is the bond's first),
+  // and their number in the top nibble; the largest of these numbers
+  unsigned bond_word[kMaxNA];
+  int bond_max;
   double fene_k, fene_r02, fene_inv_r02;
   int intra_wca;
   int cg_n;

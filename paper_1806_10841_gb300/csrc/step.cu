@@ -66,10 +66,11 @@ static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int done, int nstep
 }
 
 // The run kernel where the device is far from full: there a step is latency, and a grid barrier
-// costs less than two launches (us a step, run kernel against launches, FP32: 1000 molecules 9.4
-// and 17.6; 12,000: 13.8 and 19.5; 25,000: 19.9 and 20.7; 40,000: 25 and 23).  Not for the
-// water-like fluid: its long lists make the step itself longer than the launches (2000
-// molecules: 33 both ways), nor in FP64 beyond one tile per SM (two blocks an SM reside).
+// costs less than two launches (us a step, run kernel against launches, FP32: 1000 molecules 8.8
+// and 17.1; 12,000: 12.8 and 18.5; 24,000: 18.9 and 19.4; 30,000: 19.5 and 20.3; 40,000: 24.5 and
+// 21.8).  Not for the water-like fluid: its long lists make the step itself longer than the
+// launches (2000 molecules: 33 both ways), nor in FP64 beyond one tile per SM (two blocks an SM
+// reside; 2000 molecules 26.7 and 29.8, 4800: 27.5 and 30.7).
 bool run_kernel_pays(const Sys& s) {
   return !s.cg_mode && s.nb_model == 0 && s.M <= (s.fp64 ? 32ll : 160ll) * s.n_sm;
 }

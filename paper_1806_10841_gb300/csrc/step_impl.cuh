@@ -548,7 +548,7 @@ __device__ __forceinline__ void map_group64(const Sys& s, const Box& B, const Bu
 // build, merged into the control block with one fire-and-forget atomic per block (no
 // fence, no returned value, so blocks retire at once) into slot blockIdx mod kExtSlots:
 // spread over 32 slots the blocks' atomics rarely meet at one address (one address for
-// all blocks cost ~2 us of the fused step at 800k atoms); the decide kernel folds them.
+// all blocks cost ~2 us of the fused step at 800k atoms); whoever takes the rebuild decision folds them.
 __device__ __forceinline__ void publish_extent(const Bufs& b, int set, float ext2, float disp2) {
   __shared__ unsigned red[2][kMaxForceBlock / 32];
   const unsigned e = __reduce_max_sync(0xffffffffu, __float_as_uint(ext2));
@@ -622,8 +622,13 @@ constexpr int step_min_blocks() {
 
 // How a step kernel deals out a work item's neighbours (its template parameter FORM): one lane
 // per atom (four lanes an item; FP64 water-like items two such groups); one lane per neighbour
-// with the lanes per item chosen by the host; the same fixed to eight and four lanes.
-constexpr int FORM_ATOM = 0, FORM_NEIGHBOUR = 1, FORM_NEIGHBOUR_8_4 = 2;
+// with the lanes per item chosen by the host; the same fixed to eight and four lanes; one lane per
+// atom with every force added to the atom's sum one by one, in list and bond order.  The last is
+// for the learned force: its inputs are rounded to bfloat16, which turns a last-bit difference of
+// a position into 2^-9 of an input, so a trajectory should not depend on how sums are grouped
+// (outliers of 1e-3 of the force RMS after 50 steps with grouped sums, none with ordered ones;
+// 50 steps of 200,000 molecules 6136 us grouped, 6014 ordered).
+constexpr int FORM_ATOM = 0, FORM_NEIGHBOUR = 1, FORM_NEIGHBOUR_8_4 = 2, FORM_ORDERED = 3;
 template <int FORM, class P, int MODEL>
 __device__ __forceinline__ Lanes lanes_of(Lanes chosen) {
   if (FORM == FORM_NEIGHBOUR) return chosen;
@@ -648,8 +653,9 @@ __device__ __forceinline__ float2 wca_fr2(const Sys& s, float2 sr6, float2 ir2, 
 // neighbour keeps several neighbours' loads in flight per molecule, where one lane per atom
 // walked the whole list as one dependent chain (13 neighbours deep in the tetrahedral fluid,
 // ~300 in the water-like one), tests each neighbour once instead of once per atom and leaves no
-// lane idle for three-atom molecules.  Water-like fluid, 64,000 molecules: 189 -> 138 us a step;
-// tetrahedral, 1000 molecules in the run kernel: 16.9 -> 9.4 us.
+// lane idle for three-atom molecules.  Water-like fluid, 64,000 molecules: 189 -> 138 us a step
+// (126 with later changes); tetrahedral, 1000 molecules in the run kernel: 16.9 -> 9.4
+// us (8.9).
 template <int NA, bool ENERGY, int MODEL, bool HS, class Acc>
 __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int G, int lig, int nnb,
                                             int m_first, bool live_item, const int4 Ca, float wa, float reach_at2, float sw,
@@ -855,7 +861,8 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
 // fetched while the current one is evaluated.  Fewer registers than one lane per neighbour
 // (48 against 90, so twice the warps): the faster way once there are enough molecules to fill
 // the device.
-template <int NA, bool ENERGY, bool HS, class Acc>
+// ORDERED: one sum per component, every term added to it by itself.
+template <int NA, bool ENERGY, bool HS, bool ORDERED, class Acc>
 __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int g, int nnb,
                                                  int m_first, const int* row, const int4 Ca, float wa, float3 oi, float frac_g,
                                                  float reach_at2, float sw, bool slow, bool drift, float& fx, float& fy,
@@ -892,7 +899,7 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
         const float2 d2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
         const bool h0 = d2.x < rc_at2, h1 = j1 != j0 && d2.y < rc_at2;
         if (h0 || h1) {
-              const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
+          const float2 ir2 = make_float2(Q::rcp_(d2.x), Q::rcp_(d2.y));
           const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
           const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
           float2 fr = wca_fr2(s, sr6, ir2, wab);
@@ -907,9 +914,15 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
           }
           fr.x = h0 ? fr.x : 0.f;
           fr.y = h1 ? fr.y : 0.f;
-          ax = __ffma2_rn(fr, dx, ax);
-          ay = __ffma2_rn(fr, dy, ay);
-          az = __ffma2_rn(fr, dz, az);
+          if (ORDERED) {
+            ax.x = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, ax.x));
+            ay.x = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, ay.x));
+            az.x = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, az.x));
+          } else {
+            ax = __ffma2_rn(fr, dx, ax);
+            ay = __ffma2_rn(fr, dy, ay);
+            az = __ffma2_rn(fr, dz, az);
+          }
           if (ENERGY) {
             acc(vir, 0.5f * (fr.x * d2.x));
             acc(vir, 0.5f * (fr.y * d2.y));
@@ -923,9 +936,16 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
       const float F = s.cg_mode ? b.fpair[(size_t)t * s.cap + q] : Q::cg(b, s.cg_n, r, s.f.cg_inv_dr, &V);
       const float fw = (1.f - wab) * F;
       const float c = Q::div_(fw * sw, r);
-      Fx += c * R.x;
-      Fy += c * R.y;
-      Fz += c * R.z;
+      if (ORDERED) {
+        const float cf = frac_g * c;
+        ax.x = fmaf(cf, R.x, ax.x);
+        ay.x = fmaf(cf, R.y, ay.x);
+        az.x = fmaf(cf, R.z, az.x);
+      } else {
+        Fx += c * R.x;
+        Fy += c * R.y;
+        Fz += c * R.z;
+      }
       if (ENERGY && g == 0) {
         acc(e_cg, 0.5f * ((1.f - wab) * V));
         acc(vir, 0.5f * (Q::div_(fw, r) * r2));
@@ -933,9 +953,9 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
       if (drift && g == 0) dv -= sw * V;
     }
   }
-  fx = -fmaf(frac_g, Fx, ax.x + ax.y);
-  fy = -fmaf(frac_g, Fy, ay.x + ay.y);
-  fz = -fmaf(frac_g, Fz, az.x + az.y);
+  fx = ORDERED ? -ax.x : -fmaf(frac_g, Fx, ax.x + ax.y);
+  fy = ORDERED ? -ay.x : -fmaf(frac_g, Fy, ay.x + ay.y);
+  fz = ORDERED ? -az.x : -fmaf(frac_g, Fz, az.x + az.y);
   if (HS) {  // V_AT_a - V_CG_a = half the group's sum (every pair is listed from both sides)
     const unsigned gmask = 0xFu << (threadIdx.x & 28);
     dv += __shfl_xor_sync(gmask, dv, 1);
@@ -950,7 +970,8 @@ __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, con
 // neighbours is first tested in FP32 with a margin (fixed-point centres and float offsets; the
 // margin, Sys::f.pretest, covers both and grows with the box) and only what passes is evaluated,
 // and tested again, in FP64; the coarse-grained force of a pair is evaluated by one lane of the
-// group.  800k atoms: 930 -> 516 us a step, 80k atoms all-atomistic 216 -> 80 us.
+// group.  800k atoms: 930 -> 516 us a step, 80k atoms all-atomistic 216 -> 80 us (400 and
+// 64 us with the bonds evaluated once and positions wrapped in integers).
 template <int NA, bool ENERGY, int MODEL, bool HS, int SPLIT>
 __device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int a, int g, int sub, int nnb,
                                             bool live_item, const int* row, const double4_32a Ca, const double4_32a oi,
@@ -1090,8 +1111,9 @@ __device__ __forceinline__ void hr_forces64(const Sys& s, const Box& B, const Bu
 //
 // A high-resolution work item takes 2^ln.h lanes and a coarse-grained one 2^ln.c (32 >= 2^h >=
 // 2^c >= 4, so that no item's lanes straddle a warp); the first four integrate and map the
-// molecule, one lane per atom.  LPN: one lane per neighbour (hr_forces32), else per atom.
-template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, bool LPN, bool SAMPLE>
+// molecule, one lane per atom.  LPN: one lane per neighbour (hr_forces32), else per atom (ORDERED:
+// FORM_ORDERED).
+template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS, bool LPN, bool SAMPLE, bool ORDERED>
 __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lanes ln, const int gtid, const int cur,
                                           const long long step, const float ext_now, const int sample, float& ext2,
                                           float& disp2) {
@@ -1163,7 +1185,7 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
   if (hr_item) {
     if constexpr (!P::fp64 && !LPN) {
       static_assert(MODEL == 0, "one lane per atom");
-      hr_forces32_atom<NA, ENERGY, HS>(s, B, b, cur, t, g, nnb, m_first, row, Ca, wa, make_float3(oi.x, oi.y, oi.z), frac_g,
+      hr_forces32_atom<NA, ENERGY, HS, ORDERED>(s, B, b, cur, t, g, nnb, m_first, row, Ca, wa, make_float3(oi.x, oi.y, oi.z), frac_g,
                                        reach_at2, sw, slow, drift, fx, fy, fz, dv, e_at, e_cg, vir);
     } else if constexpr (!P::fp64) {
       hr_forces32<NA, ENERGY, MODEL, HS>(s, B, b, cur, t, a, 1 << ln.h, lig, nnb, m_first, live_item, Ca, wa, reach_at2, sw, slow, drift,
@@ -1367,41 +1389,56 @@ __device__ __forceinline__ void step_tile(const Sys& s, const Bufs& b, const Lan
       }
     } else {
       const real R02 = par<real>(s.fene_r02, s.f.fene_r02), K = par<real>(s.fene_k, s.f.fene_k);
-#pragma unroll
-      for (int q = 0; q < kMaxBonds; ++q) {
-        if (q >= s.bond_rounds) break;
-        const int e = (send >> (4 * q)) & 15;
-        const auto oo = atom_off(e & 3);
-        real bx = 0, by = 0, bz = 0;
-        if (e & 8) {
-          const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
-          const real d2 = dx * dx + dy * dy + dz * dz;
-          if (d2 >= R02) {
-            set_error(b.ctrl, ADRESS_ERR_BOND_BROKEN, a);
-          } else {
-            const real gg = (real)1 - (P::fp64 ? d2 * (real)s.fene_inv_r02 : Q::div_(d2, R02));
-            real fr = Q::div_(-K, gg);
-            if (ENERGY) {
-              if constexpr (std::is_same_v<Acc, Sum2>) acc_log(e_log, gg, b.log_tab);
-              else e_log += log((double)gg);
-            }
-            if (s.intra_wca && d2 < rc_at2) {
-              const real ir2 = Q::rcp_(d2);
-              const real sr2 = sig2 * ir2;
-              const real sr6 = sr2 * sr2 * sr2;
-              fr += (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2;
-              if (ENERGY) acc(e_b, (real)4 * eps * (sr6 * sr6 - sr6) + eps);
-            }
-            bx = fr * dx;
-            by = fr * dy;
-            bz = fr * dz;
-            fx = fma_(fr, dx, fx);
-            fy = fma_(fr, dy, fy);
-            fz = fma_(fr, dz, fz);
-            if (ENERGY) acc(vir, fr * d2);
+      // FENE + WCA with the atom at oo, added to this atom's force; its energy if it counts; the
+      // force itself, for the other atom
+      auto fene = [&](auto oo, bool counts, real& bx, real& by, real& bz) {
+        const real dx = (real)oi.x - (real)oo.x, dy = (real)oi.y - (real)oo.y, dz = (real)oi.z - (real)oo.z;
+        const real d2 = dx * dx + dy * dy + dz * dz;
+        if (d2 >= R02) {
+          set_error(b.ctrl, ADRESS_ERR_BOND_BROKEN, a);
+        } else {
+          const real gg = (real)1 - (P::fp64 ? d2 * (real)s.fene_inv_r02 : Q::div_(d2, R02));
+          real fr = Q::div_(-K, gg);
+          if (ENERGY && counts) {
+            if constexpr (std::is_same_v<Acc, Sum2>) acc_log(e_log, gg, b.log_tab);
+            else e_log += log((double)gg);
           }
+          if (s.intra_wca && d2 < rc_at2) {
+            const real ir2 = Q::rcp_(d2);
+            const real sr2 = sig2 * ir2;
+            const real sr6 = sr2 * sr2 * sr2;
+            fr += (real)24 * eps * ((real)2 * sr6 * sr6 - sr6) * ir2;
+            if (ENERGY && counts) acc(e_b, (real)4 * eps * (sr6 * sr6 - sr6) + eps);
+          }
+          bx = fr * dx;
+          by = fr * dy;
+          bz = fr * dz;
+          fx = fma_(fr, dx, fx);
+          fy = fma_(fr, dy, fy);
+          fz = fma_(fr, dz, fz);
+          if (ENERGY && counts) acc(vir, fr * d2);
         }
-        give(q, bx, by, bz);
+      };
+      if constexpr (ORDERED) {  // every atom its own bonds, in bond order
+        const unsigned bw = own ? s.bond_word[gg0] : 0u;
+#pragma unroll
+        for (int q = 0; q < kMaxBonds; ++q) {
+          if (q >= s.bond_max) break;
+          const int e = (bw >> (4 * q)) & 15;
+          const auto oo = atom_off(e & 3);
+          real bx, by, bz;
+          if (q < (int)(bw >> 28)) fene(oo, e & 8, bx, by, bz);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < kMaxBonds; ++q) {
+          if (q >= s.bond_rounds) break;
+          const int e = (send >> (4 * q)) & 15;
+          const auto oo = atom_off(e & 3);
+          real bx = 0, by = 0, bz = 0;
+          if (e & 8) fene(oo, true, bx, by, bz);
+          give(q, bx, by, bz);
+        }
       }
     }
   }
@@ -1579,11 +1616,11 @@ template <class P, int NA, int MODE, bool ENERGY, bool MULTI, int MODEL, bool HS
 __global__ void __launch_bounds__(kMaxForceBlock, step_min_blocks<P, MODEL, MULTI, HS>()) k_step(const __grid_constant__ Sys s, Bufs b) {
   const Ctrl* c = b.ctrl;
   float ext2 = 0.f, disp2 = 0.f;
-  constexpr bool LPN = FORM != FORM_ATOM;
+  constexpr bool LPN = FORM == FORM_NEIGHBOUR || FORM == FORM_NEIGHBOUR_8_4;
   const Lanes ln = lanes_of<FORM, P, MODEL>(s.step_lanes);
   // blocks past the last item (the host does not know the number of high-resolution items)
   if (!ENERGY && ln.h != ln.c && blockIdx.x * blockDim.x >= (unsigned)((c->n_hr << ln.h) + ((s.M - c->n_hr) << ln.c))) return;
-  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS, LPN, false>(s, b, ln, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
+  step_tile<P, NA, MODE, ENERGY, MULTI, MODEL, HS, LPN, false, FORM == FORM_ORDERED>(s, b, ln, blockIdx.x * blockDim.x + threadIdx.x, c->parity, c->step,
                                                         c->ext_now, 0, ext2, disp2);
   if (MODE == MODE_FUSED) publish_extent(b, 0, ext2, disp2);
 }
@@ -1618,7 +1655,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
     const int n_hr = c->n_hr;
     const int ntiles = ((n_hr << ln.h) + ((s.M - n_hr) << ln.c) + blockDim.x - 1) / blockDim.x;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, LPN, true>(s, b, ln, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
+      step_tile<P, NA, MODE_FUSED, false, MULTI, MODEL, HS, LPN, true, false>(s, b, ln, tile * blockDim.x + threadIdx.x, cur, step, ext_now,
                                                                 sample, ext2, disp2);
     publish_extent(b, set, ext2, disp2);
     if (!bar.sync()) return;
@@ -1683,6 +1720,9 @@ static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cu
     if (s.step_lanes.h == 3 && s.step_lanes.c == 2) launch_step_boxes<P, NA, MODEL, HS, FORM_NEIGHBOUR_8_4>(s, b, mode, energy, st);
     else launch_step_boxes<P, NA, MODEL, HS, FORM_NEIGHBOUR>(s, b, mode, energy, st);
   } else {
+    if constexpr (!P::fp64 && !HS) {  // (energy interpolation has no learned force)
+      if (s.cg_mode) return launch_step_boxes<P, NA, MODEL, HS, FORM_ORDERED>(s, b, mode, energy, st);
+    }
     launch_step_boxes<P, NA, MODEL, HS, FORM_ATOM>(s, b, mode, energy, st);
   }
 }
