@@ -51,6 +51,9 @@ __global__ void __launch_bounds__(kListThreads, kListBlocksPerSm) k_lists(const 
   if (d.rebuild) {
     GridBarrier bar(c, &c->bar[0]);
     if (!rebuild_lists<kListThreads / 32>(s, b, cur, bar)) return;
+    // the last phase ends without a barrier: a block arrives below only with the errors of all its
+    // warps set, for the host takes lists_err for the outcome of the build
+    __syncthreads();
   }
   // the last block to get here (no block waits) closes the mapping
   if (threadIdx.x < 32 && last_to_arrive(c)) finish_mapping(b, d, da);
