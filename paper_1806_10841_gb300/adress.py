@@ -389,12 +389,13 @@ class AdResS:
         self._call("adress_autotune", C.c_int32(int(nsteps)), _dptr(rows), 32, C.byref(n))
         return [(int(r[0]), float(r[1]), float(r[2]), float(r[3]), float(r[4])) for r in rows[:n.value]]
 
-    LIMIT_PAIR_CAPACITY, LIMIT_MMA_WAIT_POLLS = 0, 1
+    LIMIT_PAIR_CAPACITY, LIMIT_MMA_WAIT_POLLS, LIMIT_BARRIER_POLLS = 0, 1, 2
 
     def set_limit(self, which: int, value: int):
         """Run-time limit of the handle (adress_set_limit): LIMIT_PAIR_CAPACITY (pairs the
-        learned force's buffers may hold, <= 0: the allocation) or LIMIT_MMA_WAIT_POLLS (polls
-        of the tcgen05 evaluation's bounded waits, < 0: the default)."""
+        learned force's buffers may hold, <= 0: the allocation), LIMIT_MMA_WAIT_POLLS (polls
+        of the tcgen05 evaluation's bounded waits, < 0: the default) or LIMIT_BARRIER_POLLS
+        (polls of the grid-wide barriers, < 0: the default)."""
         self._call("adress_set_limit", C.c_int32(int(which)), C.c_int64(int(value)))
 
     def list_stats(self):

@@ -736,6 +736,7 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   b.boxes = h->d_boxes;
   b.mol_box = h->mol_box;
   b.wait_polls = kMmaWaitPolls;
+  b.barrier_polls = kBarrierPolls;
   b.cen64 = h->cen64;
   b.cen32 = h->cen32;
   if (e != cudaSuccess) {
@@ -1474,6 +1475,10 @@ adress_status adress_set_limit(adress_handle h, int32_t which, int64_t value) {
     case ADRESS_LIMIT_MMA_WAIT_POLLS:
       if (value > 0xFFFFFFFFll) return fail(h, ADRESS_ERR_ARG, "wait poll limit must be below 2^32");
       h->buf.wait_polls = value < 0 ? kMmaWaitPolls : (unsigned)value;
+      break;
+    case ADRESS_LIMIT_BARRIER_POLLS:
+      if (value > 0xFFFFFFFFll) return fail(h, ADRESS_ERR_ARG, "wait poll limit must be below 2^32");
+      h->buf.barrier_polls = value < 0 ? kBarrierPolls : (unsigned)value;
       break;
     default:
       return fail(h, ADRESS_ERR_ARG, "unknown limit");

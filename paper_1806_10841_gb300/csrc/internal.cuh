@@ -25,7 +25,7 @@ constexpr int kExtSlots = 32;
 // Candidates a warp of the list build stages at once.
 constexpr int kMaxCand = 160;
 
-// Poll limit of a grid-wide barrier (each poll is one L2 read): seconds, far beyond the
+// Default poll limit of a grid-wide barrier (each poll is one L2 read): seconds, far beyond the
 // longest phase between two barriers.
 constexpr unsigned kBarrierPolls = 1u << 23;
 
@@ -235,6 +235,7 @@ struct Bufs {
   long long pcap;   // pairs the buffers may hold (the allocation, or a smaller limit the host set)
   long long ncap;   // candidate records netc may hold (the allocation)
   unsigned wait_polls;  // poll limit of the tcgen05 evaluation's product waits (kMmaWaitPolls)
+  unsigned barrier_polls;  // poll limit of the grid-wide barriers (kBarrierPolls)
   // batched replicas (nbox > 1)
   const Box* boxes;    // [nbox]
   const int* mol_box;  // [M] box of each molecule

@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kListThreads, kListBlocksPerSm) k_lists(const 
   const Decision d = decide_rebuild(s, c, 0, da.force);
   if (d.dead) return;  // (the barrier left a timeout in lists_err)
   if (d.rebuild) {
-    GridBarrier bar(c, &c->bar[0]);
+    GridBarrier bar(b, &c->bar[0]);
     if (!rebuild_lists<kListThreads / 32>(s, b, cur, bar)) return;
     // the last phase ends without a barrier: a block arrives below only with the errors of all its
     // warps set, for the host takes lists_err for the outcome of the build

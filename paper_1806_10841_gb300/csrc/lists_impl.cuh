@@ -28,17 +28,20 @@ __device__ __forceinline__ int cell_of(unsigned int X, int nc) {
 
 // ---- grid-wide barrier -----------------------------------------------------------------
 // All blocks of a cooperative launch; one 64-bit arrival counter that only grows (a launch
-// finds it at a multiple of its grid).  The wait is bounded: when it gives up, the error word
-// gets a timeout, Ctrl::dead is set and the block leaves the kernel; every later kernel with
-// barriers leaves at once (the counters are out of step, the lists half built but in bounds)
-// until the host has reported the error and reset both.
+// finds it at a multiple of its grid).  The wait is bounded (Bufs::barrier_polls): when it gives
+// up, the error word gets a timeout, Ctrl::dead is set and the block leaves the kernel; every
+// later kernel with barriers leaves at once (the counters are out of step, the lists half built
+// but in bounds) until the host has reported the error and reset both.  A block that passes the
+// barrier all the same goes no further than the next one, where the blocks that left are missing:
+// so a phase starts only when the phase before it is complete.
 struct GridBarrier {
   Ctrl* c;
   unsigned long long* count;
   unsigned long long target;
+  const unsigned polls;
   bool first;
-  __device__ __forceinline__ GridBarrier(Ctrl* ctrl, unsigned long long* ctr)
-      : c(ctrl), count(ctr), target(0), first(true) {}
+  __device__ __forceinline__ GridBarrier(const Bufs& b, unsigned long long* ctr)
+      : c(b.ctrl), count(ctr), target(0), polls(b.barrier_polls), first(true) {}
   __device__ __forceinline__ bool sync() {
     int dead = 0;
     __syncthreads();
@@ -50,16 +53,16 @@ struct GridBarrier {
       if (first) target = old - old % gridDim.x;
       target += gridDim.x;
       for (unsigned n = 0;; ++n) {
-        unsigned long long v;
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
-        if ((long long)(v - target) >= 0) break;
-        if (n >= kBarrierPolls) {
+        if (n >= polls) {
           dead = 1;
           set_error(c, ADRESS_ERR_TIMEOUT, (int)blockIdx.x);
           atomicExch(&c->lists_err, ADRESS_ERR_TIMEOUT);
           atomicExch(&c->dead, 1);
           break;
         }
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+        if ((long long)(v - target) >= 0) break;
       }
     }
     first = false;

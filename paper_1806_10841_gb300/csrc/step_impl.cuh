@@ -1648,7 +1648,7 @@ __global__ void __launch_bounds__(kMaxForceBlock, run_min_blocks<P>()) k_run(con
   float ext_now = c->ext_now;
   constexpr bool LPN = !P::fp64;
   const Lanes ln = lanes_of<LPN ? FORM_NEIGHBOUR : FORM_ATOM, P, MODEL>(s.run_lanes);
-  GridBarrier bar(c, &c->bar[1]);
+  GridBarrier bar(b, &c->bar[1]);
   for (int k = 0; k < nsteps; ++k) {
     float ext2 = 0.f, disp2 = 0.f;
     const int sample = sample_every > 0 && (done + k + 1) % sample_every == 0;

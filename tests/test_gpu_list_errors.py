@@ -42,3 +42,68 @@ def test_one_overflowing_molecule_in_a_dense_cell_grows_the_capacity(seed, preci
         assert np.array_equal(f, f_ref)
         sim.check()
         sim.close()
+
+
+TIMEOUT = 6
+
+
+def reported(call):
+    from paper_1806_10841_gb300 import adress
+
+    with pytest.raises(adress.AdressError) as ei:
+        call()
+    assert ei.value.status == TIMEOUT
+
+
+def per_sm(n):
+    import torch
+
+    return n * torch.cuda.get_device_properties(0).multi_processor_count
+
+
+# one block, the run kernel, a step and a list kernel per step; dense cells
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("make,M", [(inputs.scaled_c2, 216), (inputs.scaled_c2, 4001), (inputs.scaled_c2, (161, 3)),
+                                    (inputs.scaled_c3, 4001)])
+def test_a_grid_barrier_that_gives_up_is_reported_and_the_next_call_is_clean(make, M, precision):
+    """Barriers limited to zero polls give up at once: a build returns the timeout, a run reports it
+    at the check.  With the default limit again forces and trajectory are those of a fresh handle."""
+    from paper_1806_10841_gb300 import adress
+
+    M = per_sm(M[0]) + M[1] if isinstance(M, tuple) else M
+    s = make(M, seed=5)
+    x, v = inputs.tetra_state(s) if s.na == 4 else inputs.water_state(s)
+
+    def run(sim):
+        sim.set_state(x, v)
+        sim.set_step(0)
+        f, e = sim.forces()
+        sim.run(60, sample_every=9)
+        sim.check()
+        return (f, *sim.get_state()), e
+
+    ref = adress.AdResS(s, precision=precision)
+    want, e_ref = run(ref)
+    ref.close()
+    sim = adress.AdResS(s, precision=precision)
+    run(sim)
+    calls = (sim.build_lists, lambda: sim.compute_forces(True), lambda: sim.compute_forces(False))
+    for call in calls:
+        sim.set_state(x, v)
+        sim.set_limit(sim.LIMIT_BARRIER_POLLS, 0)
+        reported(call)
+        reported(sim.check)
+        sim.check()  # reported once
+        with pytest.raises(adress.AdressError):
+            sim.step(1)  # no lists
+        sim.set_limit(sim.LIMIT_BARRIER_POLLS, -1)
+        got, e = run(sim)
+        assert e == e_ref and all(np.array_equal(a, b) for a, b in zip(got, want))
+    # lists due in the middle of a run, the run kernel's own barriers
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, 0)
+    sim.run(100, sample_every=9)
+    reported(sim.check)
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, -1)
+    got, e = run(sim)
+    assert e == e_ref and all(np.array_equal(a, b) for a, b in zip(got, want))
+    sim.close()
