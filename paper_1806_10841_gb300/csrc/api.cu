@@ -797,6 +797,19 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
   if (e == cudaSuccess) e = cudaMemsetAsync(b.item_of, 0, sizeof(int) * M, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.nn, 0, sizeof(int) * M, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(b.nbr, 0, sizeof(int) * (size_t)s.cap * M, st);
+  // and molecules at rest at the origin: such a build does not make its mapping current, so that
+  // the forces behind a first one read the other half of the double-buffered arrays (an index of a
+  // nearest centre and a table position among them)
+  auto clear = [&](auto* p, size_t n) {
+    if (e == cudaSuccess && p) e = cudaMemsetAsync(p, 0, sizeof(*p) * n, st);
+  };
+  clear(b.com_fx[0], M);
+  clear(b.com64[0], M);
+  clear(b.dxc64[0], M);
+  clear(b.off64[0], N);
+  clear(b.molf[0], M);
+  clear(b.off32[0], (size_t)3 * M);
+  clear(b.kcen[0], M);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host vectors go out of scope
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {

@@ -107,3 +107,41 @@ def test_a_grid_barrier_that_gives_up_is_reported_and_the_next_call_is_clean(mak
     got, e = run(sim)
     assert e == e_ref and all(np.array_equal(a, b) for a, b in zip(got, want))
     sim.close()
+
+
+def spheres(scheme):
+    s = inputs.scaled_c2(3000, seed=7, scheme=scheme)
+    L = np.array(s.box)
+    s.d_at, s.d_hy = 4.0, 3.0
+    s.centers = np.array([[0.2, 0.5, 0.5], [0.7, 0.3, 0.8]]) * L
+    s.tf = 0.3 * np.cos(np.arange(int((s.d_at + s.d_hy) / s.tf_dx) + 2))
+    return s
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("make", [lambda: spheres(0), lambda: spheres(1), lambda: inputs.scaled_c2(3000, scheme=1),
+                                  lambda: inputs.scaled_c3(3000)])
+def test_forces_behind_a_first_build_that_gave_up(make, precision):
+    """Nothing was ever mapped when the first build of a handle gives up and the forces run behind
+    it: they read the arrays as the handle was created, and the next call is that of a fresh handle."""
+    from paper_1806_10841_gb300 import adress
+
+    s = make()
+    x, _ = inputs.tetra_state(s) if s.na == 4 else inputs.water_state(s)
+    ref = adress.AdResS(s, precision=precision)
+    ref.set_state(x)
+    f_ref, e_ref = ref.forces()
+    ref.check()
+    ref.close()
+    sim = adress.AdResS(s, precision=precision)
+    sim.set_state(x)
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, 0)
+    reported(lambda: sim.compute_forces(True))
+    reported(sim.check)
+    reported(lambda: sim.compute_forces(False))
+    reported(sim.check)
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, -1)
+    f, e = sim.forces()
+    sim.check()
+    assert e == e_ref and np.array_equal(f, f_ref)
+    sim.close()
