@@ -110,6 +110,13 @@ static cudaError_t realloc_owned(adress_ctx* h, T** p, size_t n) {
   return dalloc(h, p, n);
 }
 
+// No candidates of the network force and no pairs: what new buffers hold.
+static cudaError_t clear_pairs(adress_ctx* h) {
+  cudaError_t e = cudaMemsetAsync(&h->buf.ctrl->n_netc, 0, sizeof(Ctrl::n_netc), h->stream);
+  if (e == cudaSuccess && h->buf.npair) e = cudaMemsetAsync(h->buf.npair, 0, sizeof(unsigned), h->stream);
+  return e;
+}
+
 // Pair buffers of the network CG force: every unordered listed pair at most once
 // (sum of list lengths / 2 <= M cap / 2), plus 16 bytes of slack each for the evaluation's
 // bulk copies, which round a ragged last tile up to 16 bytes.
@@ -124,6 +131,7 @@ static cudaError_t alloc_pair_buffers(adress_ctx* h) {
     h->pcap_alloc = pcap;
     b.pcap = h->pcap_limit > 0 ? std::min(h->pcap_limit, pcap) : pcap;
     b.ncap = pcap;
+    e = clear_pairs(h);
   }
   return e;
 }
@@ -136,13 +144,14 @@ static cudaError_t reset_barriers(adress_ctx* h) {
   return e;
 }
 
-// After a barrier gave up: the barriers, the maxima and the cell counters (a build may have
-// stopped anywhere) as a fresh handle has them; the lists must be built again.
+// After a barrier gave up: the barriers, the maxima, the cell counters (a build may have stopped
+// anywhere) and the network's pairs as a fresh handle has them; the lists must be built again.
 static cudaError_t revive(adress_ctx* h) {
   cudaError_t e = reset_barriers(h);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->buf.ctrl->ext_slot, 0, sizeof(Ctrl::ext_slot), h->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(h->buf.cell_count, 0, sizeof(unsigned long long) * (size_t)h->sys.ncell, h->stream);
+  if (e == cudaSuccess) e = clear_pairs(h);
   if (e == cudaSuccess) e = cudaMemsetAsync(&h->buf.ctrl->dead, 0, sizeof(Ctrl::dead), h->stream);
   h->lists_built = false;
   return e;

@@ -863,6 +863,9 @@ __global__ void __launch_bounds__(128) k_mlp_feat(const __grid_constant__ Sys s,
   // multiple time stepping: the network gives a slow (CG) force, needed only at outer time
   // levels; elsewhere no pair is written and the evaluation kernel finds nothing to do
   if (s.respa_n > 1 && b.ctrl->step % s.respa_n != 0) return;
+  // a build gave up: the candidates may be another build's, or nobody's in new buffers, and the
+  // pair count was not cleared
+  if (b.ctrl->dead) return;
   __shared__ float sn[2][kIn];
   if (threadIdx.x < kIn) {
     sn[0][threadIdx.x] = norm[threadIdx.x];
@@ -1154,7 +1157,8 @@ cudaError_t mlp_collect(const Sys& s, const Bufs& b, int pass, const int* offs, 
 
 cudaError_t mlp_pairs(const Sys& s, const Bufs& b, const MlpDevArgs& a, float* fpair, cudaStream_t st) {
   const MlpDev m{a.P, a.W1p, a.W2p, a.W2Tp, a.norm};
-  // the pair count is zero here: cleared with the mapping (k_lists)
+  // the pair count is zero here: cleared with the mapping (k_lists), unless a build gave up, and
+  // then no pairs are added
   cudaError_t e;
   // persistent grid for the candidates (their count is on the device): 22 blocks per SM,
   // about two waves of the 10 that the kernel's 48 registers let reside (11, 16, 20, 33 and

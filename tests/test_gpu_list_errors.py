@@ -145,3 +145,51 @@ def test_forces_behind_a_first_build_that_gave_up(make, precision):
     sim.check()
     assert e == e_ref and np.array_equal(f, f_ref)
     sim.close()
+
+
+@pytest.mark.parametrize("max_neighbors", [0, 4])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_learned_force_behind_a_build_that_gave_up(precision, max_neighbors):
+    """The network's candidate pairs belong to the last complete build: none are evaluated behind
+    one that gave up, the first of a handle or a later one, with buffers that grew (four neighbours)
+    or not, nor in the steps that follow."""
+    from paper_1806_10841_gb300 import adress
+
+    s = inputs.scaled_c2(3000, seed=8)
+    x, v = inputs.tetra_state(s)
+    rng = np.random.default_rng(5)
+    params = dict(W1=rng.normal(0, 0.2, (64, 9)), b1=rng.normal(0, 0.1, 64), W2=rng.normal(0, 0.1, (64, 64)),
+                  b2=rng.normal(0, 0.1, 64), w3=rng.normal(0, 0.1, 64), b3=0.1)
+
+    def fresh(cap):
+        sim = adress.AdResS(s, precision=precision, max_neighbors=cap)
+        sim.mlp_set(params, np.full(9, 0.1), np.full(9, 0.8), 3.0)
+        sim.set_cg_mode(1)
+        return sim
+
+    def run(sim):
+        sim.set_state(x, v)
+        sim.set_step(0)
+        sim.compute_forces(energies=False)
+        f = sim.get_state()[2]
+        sim.run(20)
+        sim.check()
+        return (f, *sim.get_state())
+
+    ref = fresh(0)
+    want = run(ref)
+    ref.close()
+    sim = fresh(max_neighbors)
+    for _ in range(2):
+        sim.set_state(x, v)
+        sim.set_limit(sim.LIMIT_BARRIER_POLLS, 0)
+        reported(lambda: sim.compute_forces(False))
+        reported(sim.check)
+        sim.set_limit(sim.LIMIT_BARRIER_POLLS, -1)
+        assert all(np.array_equal(a, b) for a, b in zip(run(sim), want))
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, 0)
+    sim.run(100)
+    reported(sim.check)
+    sim.set_limit(sim.LIMIT_BARRIER_POLLS, -1)
+    assert all(np.array_equal(a, b) for a, b in zip(run(sim), want))
+    sim.close()
