@@ -347,6 +347,7 @@ struct RdfArgs {
   int *count, *start;    // [ncell], [ncell + 1]
   unsigned long long* counts;  // [nbox][nbins], added to
   int ncell, nbins;
+  int batch, parts;  // a cell's molecules are dealt out to `parts` warps, `batch` at a time
   double dr;
   float inv_dr, lim2, eps;  // 1 / dr, squared range with its margin, error of a distance in bins
 };

@@ -252,37 +252,44 @@ __global__ void k_rdf_fill(int M, const RdfArgs q) {
   if (a < M) q.sorted[q.start[q.cell[a]] + q.slot[a]] = q.fx[a];
 }
 
-// Each block takes a run of cells, box by box (a box's counts in shared memory, added to the
-// global ones when the run leaves the box); a warp takes a cell: its lanes hold 32 candidates of
-// the neighbour cells at a time and go through the cell's own molecules.  Where a box has at
-// least three cells each way only half the neighbour cells are visited (each pair of cells once),
-// else all distinct ones, counting the pairs whose candidate comes later in the sorted order.
+// Each block takes a run of tasks, box by box (a box's counts in shared memory, added to the
+// global ones when the run leaves the box).  A warp's task is a part of a cell: batches of its
+// molecules, against which the lanes hold 32 candidates of the neighbour cells at a time.  Where a
+// box has at least three cells each way only half the neighbour cells are visited (each pair of
+// cells once), else all distinct ones, counting the pairs whose candidate comes later in the
+// sorted order.  The parts are many where the cells are few (a range near half the box leaves one
+// cell to some sixteen; the cell's first molecules then have the most candidates after them, so
+// early and late parts alternate).  ms a call, all pairs in double / a warp per cell / now: 200,000
+// molecules r < 5 32 / 0.19 / 0.18, a quarter of the shortest edge 1061 / 543 / 21, just below half
+// 1610 / 16,624 / 123; 20,000: 5.6 / 0.10 / 0.08, 36 / 5.6 / 0.40, 53 / 114 / 1.1; 1000 at half the
+// edge 2.5 / 1.6 / 0.10.
 constexpr int kRdfThreads = 256;
 __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, const RdfArgs q) {
   extern __shared__ unsigned rh[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int chunk = (q.ncell + gridDim.x - 1) / gridDim.x;
-  int c0 = blockIdx.x * chunk;
-  const int c_end = min(q.ncell, c0 + chunk);
-  while (c0 < c_end) {
-    // the box of cell c0 (boxes in cell order)
+  const int ntask = q.ncell * q.parts, chunk = (ntask + gridDim.x - 1) / gridDim.x;
+  int t0 = blockIdx.x * chunk;
+  const int t_end = min(ntask, t0 + chunk);
+  while (t0 < t_end) {
+    // the box of the run's first cell (boxes in cell order)
     int lo = 0, hi = s.nbox - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (q.grids[mid].cell0 <= c0) lo = mid;
+      if (q.grids[mid].cell0 <= t0 / q.parts) lo = mid;
       else hi = mid - 1;
     }
     const RdfGrid G = q.grids[lo];
     const Box& B = s.nbox > 1 ? b.boxes[lo] : s.bx;
     const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
-    const int c1 = min(c_end, G.cell0 + nx * ny * nz);
+    const int t1 = min(t_end, (G.cell0 + nx * ny * nz) * q.parts);
     const bool half = nx >= 3 && ny >= 3 && nz >= 3;
     const float sx = B.fx_scale[0], sy = B.fx_scale[1], sz = B.fx_scale[2];
     for (int k = threadIdx.x; k < q.nbins; k += blockDim.x) rh[k] = 0u;
     __syncthreads();
-    for (int r = c0 + warp; r < c1; r += kRdfThreads / 32) {
-      const int hs = q.start[r], he = q.start[r + 1];
-      if (hs == he) continue;
+    for (int t = t0 + warp; t < t1; t += kRdfThreads / 32) {
+      const int r = t / q.parts, e = t - r * q.parts, part = e & 1 ? q.parts - 1 - (e >> 1) : e >> 1;
+      const int hs = q.start[r], he = q.start[r + 1], first = hs + part * q.batch;
+      if (first >= he) continue;
       const int l = r - G.cell0, cx = l / (ny * nz), cy = (l / nz) % ny, cz = l % nz;
       // lane j < 27: neighbour cell (ox, oy, oz) = (j / 9 - 1, (j / 3) % 3 - 1, j % 3 - 1)
       int cnt = 0, start = 0;
@@ -304,45 +311,49 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
         if (lane >= o) incl += v;
       }
       const int pre = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
-      for (int k0 = 0; k0 < total; k0 += 32) {
-        // this lane's candidate: the cells whose inclusive prefix is <= k come before its own
-        const int k = k0 + lane;
-        int j = 0;
+      for (int hb = first; hb < he; hb += q.parts * q.batch) {
+        const int ht = min(he, hb + q.batch);
+        for (int k0 = 0; k0 < total; k0 += 32) {
+          // this lane's candidate: the cells whose inclusive prefix is <= k come before its own
+          const int k = k0 + lane;
+          int j = 0;
 #pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-          const int probe = j + step - 1;
-          const int v = __shfl_sync(0xffffffffu, incl, probe < 27 ? probe : 26);
-          if (probe < 27 && v <= k) j += step;
-        }
-        const int cc = j < 27 ? j : 26;
-        const int g = __shfl_sync(0xffffffffu, start, cc) + (k - __shfl_sync(0xffffffffu, pre, cc));
-        const bool in = k < total;
-        const int4 D = q.sorted[in ? g : hs];
-        // first own molecule (sorted position) this candidate pairs with: all of them for another
-        // cell of the half set, else those before it
-        const int upto = !in ? hs : (half && cc != 13 ? he : min(he, g));
-        int4 Hn = __ldg(&q.sorted[hs]);
-        for (int h = hs; h < he; ++h) {
-          const int4 H = Hn;
-          if (h + 1 < he) Hn = __ldg(&q.sorted[h + 1]);
-          const float dx = (float)(int)((unsigned)H.x - (unsigned)D.x) * sx;
-          const float dy = (float)(int)((unsigned)H.y - (unsigned)D.y) * sy;
-          const float dz = (float)(int)((unsigned)H.z - (unsigned)D.z) * sz;
-          const float r2 = dx * dx + dy * dy + dz * dz;
-          if (h < upto && r2 < q.lim2) {
-            float rr;
-            asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rr) : "f"(r2));
-            const float u = rr * q.inv_dr, fl = floorf(u), fr = u - fl;
-            int bin = (int)fl;
-            if (fr < q.eps || fr > 1.f - q.eps) {
-              const size_t M = (size_t)s.M;
-              const double ex = minimg_cmp(q.com[H.w] - q.com[D.w], B.L[0], B.halfL[0]);
-              const double ey = minimg_cmp(q.com[M + H.w] - q.com[M + D.w], B.L[1], B.halfL[1]);
-              const double ez = minimg_cmp(q.com[2 * M + H.w] - q.com[2 * M + D.w], B.L[2], B.halfL[2]);
-              const double e2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-              bin = (int)floor(sqrt(e2) / q.dr);
+          for (int step = 16; step >= 1; step >>= 1) {
+            const int probe = j + step - 1;
+            const int v = __shfl_sync(0xffffffffu, incl, probe < 27 ? probe : 26);
+            if (probe < 27 && v <= k) j += step;
+          }
+          const int cc = j < 27 ? j : 26;
+          const int g = __shfl_sync(0xffffffffu, start, cc) + (k - __shfl_sync(0xffffffffu, pre, cc));
+          const bool in = k < total;
+          const int4 D = q.sorted[in ? g : hb];
+          // the batch's molecules (sorted positions) this candidate pairs with: all of them for
+          // another cell of the half set, else those before it
+          const int upto = !in ? hb : (half && cc != 13 ? ht : min(ht, g));
+          const int most = __reduce_max_sync(0xffffffffu, upto);
+          int4 Hn = __ldg(&q.sorted[hb]);
+          for (int h = hb; h < most; ++h) {
+            const int4 H = Hn;
+            if (h + 1 < most) Hn = __ldg(&q.sorted[h + 1]);
+            const float dx = (float)(int)((unsigned)H.x - (unsigned)D.x) * sx;
+            const float dy = (float)(int)((unsigned)H.y - (unsigned)D.y) * sy;
+            const float dz = (float)(int)((unsigned)H.z - (unsigned)D.z) * sz;
+            const float r2 = dx * dx + dy * dy + dz * dz;
+            if (h < upto && r2 < q.lim2) {
+              float rr;
+              asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rr) : "f"(r2));
+              const float u = rr * q.inv_dr, fl = floorf(u), fr = u - fl;
+              int bin = (int)fl;
+              if (fr < q.eps || fr > 1.f - q.eps) {
+                const size_t M = (size_t)s.M;
+                const double ex = minimg_cmp(q.com[H.w] - q.com[D.w], B.L[0], B.halfL[0]);
+                const double ey = minimg_cmp(q.com[M + H.w] - q.com[M + D.w], B.L[1], B.halfL[1]);
+                const double ez = minimg_cmp(q.com[2 * M + H.w] - q.com[2 * M + D.w], B.L[2], B.halfL[2]);
+                const double e2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
+                bin = (int)floor(sqrt(e2) / q.dr);
+              }
+              if (bin < q.nbins) atomicAdd(&rh[bin], 1u);
             }
-            if (bin < q.nbins) atomicAdd(&rh[bin], 1u);
           }
         }
       }
@@ -351,7 +362,7 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
     for (int k = threadIdx.x; k < q.nbins; k += blockDim.x)
       if (rh[k]) atomicAdd(&q.counts[(size_t)lo * q.nbins + k], (unsigned long long)rh[k]);
     __syncthreads();
-    c0 = c1;
+    t0 = t1;
   }
 }
 
@@ -404,7 +415,7 @@ cudaError_t launch_rdf(const Sys& s, const Bufs& b, const RdfArgs& q, cudaStream
   e = device_exclusive_scan(q.count, q.start, q.ncell, (int*)b.scan_tmp, q.start + q.ncell, st);
   if (e != cudaSuccess) return e;
   k_rdf_fill<<<ceil_div(s.M, 256), 256, 0, st>>>(s.M, q);
-  const int blocks = std::max(1, std::min(ceil_div(q.ncell, 2), 8 * s.n_sm));
+  const int blocks = std::max(1, std::min(ceil_div((long long)q.ncell * q.parts, 2), 8 * s.n_sm));
   k_rdf<<<blocks, kRdfThreads, sizeof(unsigned) * q.nbins, st>>>(s, b, q);
   return cudaGetLastError();
 }
