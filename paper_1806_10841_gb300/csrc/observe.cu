@@ -264,6 +264,18 @@ __global__ void k_rdf_fill(int M, const RdfArgs q) {
 // 1610 / 16,624 / 123; 20,000: 5.6 / 0.10 / 0.08, 36 / 5.6 / 0.40, 53 / 114 / 1.1; 1000 at half the
 // edge 2.5 / 1.6 / 0.10.
 constexpr int kRdfThreads = 256;
+
+// A block counts in 32 bits: a warp hands the counts on whenever it has tested this many pairs, so
+// that the eight warps of a block never hold more than eight times as many.  (Of 2^20 pairs each
+// costs a fraction of a percent.)
+constexpr unsigned kRdfHandOn = 1u << 20;
+__device__ __noinline__ void hand_on_counts(unsigned* rh, unsigned long long* counts, int nbins) {
+  for (int k = threadIdx.x & 31; k < nbins; k += 32) {
+    const unsigned c = atomicExch(&rh[k], 0u);
+    if (c) atomicAdd(&counts[k], (unsigned long long)c);
+  }
+}
+
 __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, const RdfArgs q) {
   extern __shared__ unsigned rh[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -284,6 +296,7 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
     const int t1 = min(t_end, (G.cell0 + nx * ny * nz) * q.parts);
     const bool half = nx >= 3 && ny >= 3 && nz >= 3;
     const float sx = B.fx_scale[0], sy = B.fx_scale[1], sz = B.fx_scale[2];
+    unsigned tested = 0;
     for (int k = threadIdx.x; k < q.nbins; k += blockDim.x) rh[k] = 0u;
     __syncthreads();
     for (int t = t0 + warp; t < t1; t += kRdfThreads / 32) {
@@ -354,6 +367,11 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
               }
               if (bin < q.nbins) atomicAdd(&rh[bin], 1u);
             }
+          }
+          tested += 32u * (unsigned)max(0, most - hb);
+          if (tested >= kRdfHandOn) {
+            hand_on_counts(rh, q.counts + (size_t)lo * q.nbins, q.nbins);
+            tested = 0;
           }
         }
       }

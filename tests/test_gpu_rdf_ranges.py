@@ -84,3 +84,18 @@ def test_boxes_of_unequal_fill():
     sim.close()
     for r in range(3):
         assert np.array_equal(got[r], all_pairs(xs[r], boxes[r], 128, 0.0625)), r
+
+
+def test_more_pairs_in_a_cell_than_32_bits_count():
+    """All molecules in one cell of many, so one warp counts every pair, all in one bin."""
+    from paper_1806_10841_gb300 import adress
+
+    M, box = 92_700, (200.0, 100.0, 100.0)
+    assert M * (M - 1) // 2 > 2 ** 32
+    s = beads(M, box)
+    rng = np.random.default_rng(2)
+    sim = adress.AdResS(s, precision="fp32", max_neighbors=8)
+    sim.set_state(rng.uniform(1.0, 3.0, (M, 3)))  # farthest apart 3.5
+    got = sim.rdf_counts(2, 2.5 * 1.5)[0]
+    sim.close()
+    assert got.tolist() == [M * (M - 1) // 2, 0]
