@@ -584,11 +584,15 @@ __global__ void __launch_bounds__(128) k_mlp_update(const float* part, int nblk,
                                                     __nv_bfloat16* W2T) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   allow_dependent_launch();
+  // What the optimiser step before wrote is read here before the wait: that step is complete (the
+  // gradient kernel in between waited for it before it let this one start), its writes performed
+  // for the whole device, and the loads go to L2, where they are, past an L1 that need not know of
+  // them.  After the wait the loads cost 0.4 us a batch (74 batches 1660 us -> 1689).
   float mo = 0.f, ve = 0.f, old = 0.f;
-  if (p < kNPar) {  // written by the previous optimiser step, complete before the gradient kernel let this one start
-    mo = mom[p];
-    ve = vel[p];
-    old = P[p];
+  if (p < kNPar) {
+    mo = __ldcg(mom + p);
+    ve = __ldcg(vel + p);
+    old = __ldcg(P + p);
   }
   wait_for_primary();
   if (p > kNPar) return;
