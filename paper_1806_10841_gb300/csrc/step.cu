@@ -77,7 +77,6 @@ bool run_kernel_pays(const Sys& s) {
 
 cudaError_t launch_run(const Sys& s, const Bufs& b, int precision, int done, int nsteps, int sample_every, cudaStream_t st) {
   if (s.scheme == 1) return launch_run_hadress(s, b, precision, done, nsteps, sample_every, st);
-  if (s.nb_model == 1) return cudaErrorInvalidValue;
   return precision == ADRESS_FP64 ? launch_run_p<P64>(s, b, done, nsteps, sample_every, st) : launch_run_p<P32>(s, b, done, nsteps, sample_every, st);
 }
 

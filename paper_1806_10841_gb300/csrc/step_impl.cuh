@@ -243,7 +243,6 @@ struct Sum2 {
 __device__ __forceinline__ void acc(double& s, double x) { s += x; }
 __device__ __forceinline__ void acc(Sum2& s, float x) { s.add(x); }
 // the exact product of two floats
-__device__ __forceinline__ void acc_product(double& s, float a, float b) { s += (double)a * (double)b; }
 __device__ __forceinline__ void acc_product(Sum2& s, float a, float b) {
   const float p = __fmul_rn(a, b);
   s.add(p);
@@ -662,6 +661,7 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
                                             bool slow, bool drift, float& fx, float& fy, float& fz, float& dv, Acc& e_at,
                                             Acc& e_cg, Acc& vir) {
   using Q = Prec<P32>;
+  static_assert(MODEL == 1 || !ENERGY, "the tetrahedral model's energies: one lane per atom");
   constexpr int NP = (NA + 1) / 2;  // pairs of the molecule's atoms, an odd last one by itself
   const int lane = threadIdx.x & 31;
   const int* row = b.nbr + (size_t)(live_item ? t : 0) * s.cap;
@@ -731,14 +731,10 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
             const float2 sr2 = __fmul2_rn(make_float2(s.f.sig2, s.f.sig2), ir2);
             const float2 sr6 = __fmul2_rn(__fmul2_rn(sr2, sr2), sr2);
             fr = wca_fr2(s, sr6, ir2, wab);
-            if (ENERGY || drift) {
+            if (drift) {
               const float v0 = h0 ? 4.f * s.f.eps * (sr6.x * sr6.x - sr6.x) + s.f.eps : 0.f;
               const float v1 = h1 ? 4.f * s.f.eps * (sr6.y * sr6.y - sr6.y) + s.f.eps : 0.f;
-              if (ENERGY) {
-                acc_product(e_at, 0.5f * wab, v0);
-                acc_product(e_at, 0.5f * wab, v1);
-              }
-              if (drift) dv += v0 + v1;
+              dv += v0 + v1;
             }
           } else {
             // LJ (c12 r^-12 - c6 r^-6, shifted) for the site pairs that have one + reaction
