@@ -763,12 +763,8 @@ static adress_status init_impl(const adress_config* cfgs, int nbox, void* stream
 
   std::vector<float2> fv(s.cg_n + 1);
   for (int k = 0; k <= s.cg_n; ++k) fv[k] = make_float2((float)c->cg_F[k], (float)c->cg_V[k]);
-  // reciprocals of the 128 intervals of [1, 2) rounded to nine bits, and their -log
   float4 logs[128];
-  for (int k = 0; k < 128; ++k) {
-    const double c = nearbyint(512.0 / (1.0 + (k + 0.5) / 128.0)) / 512.0, l = -log(c);
-    logs[k] = make_float4((float)c, (float)l, (float)(l - (double)(float)l), 0.f);
-  }
+  fill_log_table(logs);
   std::vector<double> tf(ntf, 0.0);
   std::vector<float> tff(ntf, 0.f);
   std::vector<float> fecf(c->fec, c->fec + c->fec_n);  // staged until the stream synchronises

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <string>
@@ -245,6 +246,14 @@ struct Bufs {
   const int4* cen32;         // the same in 32-bit fixed point
   const int* nbr_cells; // [ncell][27] Morton ranks of each cell's neighbour cells (-1: none)
 };
+
+// Bufs::log_tab: reciprocals of the 128 intervals of [1, 2) rounded to nine bits, and their -log.
+inline void fill_log_table(float4 (&tab)[128]) {
+  for (int k = 0; k < 128; ++k) {
+    const double c = nearbyint(512.0 / (1.0 + (k + 0.5) / 128.0)) / 512.0, l = -log(c);
+    tab[k] = make_float4((float)c, (float)l, (float)(l - (double)(float)l), 0.f);
+  }
+}
 
 // Box of molecule a (the single box unless the system holds batched replicas).
 __device__ __forceinline__ const Box& box_of(const Sys& s, const Bufs& b, int a) {
