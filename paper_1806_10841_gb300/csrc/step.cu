@@ -66,11 +66,14 @@ static cudaError_t launch_run_p(const Sys& s, const Bufs& b, int done, int nstep
 }
 
 // The run kernel where the device is far from full: there a step is latency, and a grid barrier
-// costs less than two launches (us a step, run kernel against launches, FP32: 1000 molecules 8.8
-// and 17.1; 12,000: 12.8 and 18.5; 24,000: 18.9 and 19.4; 30,000: 19.5 and 20.3; 40,000: 24.5 and
-// 21.8).  Not for the water-like fluid: its long lists make the step itself longer than the
-// launches (2000 molecules: 33 both ways), nor in FP64 beyond one tile per SM (two blocks an SM
-// reside; 2000 molecules 26.7 and 29.8, 4800: 27.5 and 30.7).
+// costs less than two launches (us a step, run kernel against launches, FP32: 1000 molecules 8.6
+// and 16.6; 12,000: 12.2 and 18.0; 24,000: 18.6 and 19.3; 30,000: 19.0 and 19.9; 35,000: 19.4 and
+// 20.5; 40,000: 23.8 and 21.1, its blocks' third round of tiles).  The line lies short of the crossing,
+// where the gain has fallen to a twentieth, and leaves that to the launches up to some 38,000.
+// Not for the water-like fluid: its long lists make the step itself longer than the launches (2000
+// molecules: 33 both ways), nor in FP64 beyond one tile per SM, on which three blocks reside (2000
+// molecules 26.3 and 29.4; 4800: 26.7 and 29.9; 7000: 32.8 and 34.3; 10,000: 46.1 and 41.4; 20,000:
+// 71.7 and 62.6).
 bool run_kernel_pays(const Sys& s) {
   return !s.cg_mode && s.nb_model == 0 && s.M <= (s.fp64 ? 32ll : 160ll) * s.n_sm;
 }

@@ -629,10 +629,11 @@ constexpr int step_min_blocks() {
 // per atom (four lanes an item; FP64 water-like items two such groups); one lane per neighbour
 // with the lanes per item chosen by the host; the same fixed to eight and four lanes; one lane per
 // atom with every force added to the atom's sum one by one, in list and bond order.  The last is
-// for the learned force: its inputs are rounded to bfloat16, which turns a last-bit difference of
-// a position into 2^-9 of an input, so a trajectory should not depend on how sums are grouped
-// (outliers of 1e-3 of the force RMS after 50 steps with grouped sums, none with ordered ones;
-// 50 steps of 200,000 molecules 6136 us grouped, 6014 ordered).
+// for the learned force of the tetrahedral model: its inputs are rounded to bfloat16, which turns a
+// last-bit difference of a position into 2^-9 of an input, so a trajectory should not depend on how
+// sums are grouped (outliers of 1e-3 of the force RMS after 50 steps with grouped sums, none with
+// ordered ones; 50 steps of 200,000 molecules 6136 us grouped, 6014 ordered).  The water-like
+// model has no lane per atom in FP32: with a learned force too its sums are grouped by lanes.
 constexpr int FORM_ATOM = 0, FORM_NEIGHBOUR = 1, FORM_NEIGHBOUR_8_4 = 2, FORM_ORDERED = 3;
 template <int FORM, class P, int MODEL>
 __device__ __forceinline__ Lanes lanes_of(Lanes chosen) {
@@ -860,9 +861,9 @@ __device__ __forceinline__ void hr_forces32(const Sys& s, const Box& B, const Bu
 
 // The same with one lane per atom: lane g evaluates its atom against every listed neighbour
 // (two of the neighbour's atoms per packed instruction), the next neighbour's index and centre
-// fetched while the current one is evaluated.  Fewer registers than one lane per neighbour
-// (48 against 90, so twice the warps): the faster way once there are enough molecules to fill
-// the device.
+// fetched while the current one is evaluated.  Fewer registers than one lane per neighbour (56
+// against the 128 it has in the run kernel, so twice the warps): the faster way once there are
+// enough molecules to fill the device.
 // ORDERED: one sum per component, every term added to it by itself.
 template <int NA, bool ENERGY, bool HS, bool ORDERED, class Acc>
 __device__ __forceinline__ void hr_forces32_atom(const Sys& s, const Box& B, const Bufs& b, int cur, int t, int g, int nnb,
