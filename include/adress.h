@@ -366,11 +366,11 @@ adress_status adress_get_tf(adress_handle h, double* tf_host, int32_t n); /* syn
  *    products it has in flight before it frees its tensor memory; the next evaluation runs
  *    normally.  0 makes every such wait give up at once (for testing the error path).
  *  ADRESS_LIMIT_BARRIER_POLLS: polls of the bounded grid-wide barriers of the list build and of
- *    the kernel that runs all steps of a small system (default 2^23, seconds); value < 0 restores
- *    the default.  A barrier that gives up records ADRESS_ERR_TIMEOUT: adress_build_lists and
+ *    the kernel that runs all steps of a small system (default 2^23, seconds), in steps of 1024;
+ *    value < 0 restores the default.  A barrier that gives up records ADRESS_ERR_TIMEOUT: adress_build_lists and
  *    adress_compute_forces return it, adress_check reports it after adress_step and adress_run,
  *    whose state is then undefined.  No list is built until adress_check has reported the error;
- *    then build the lists again.  0 makes every barrier give up at once (for testing).
+ *    then build the lists again.  With 0 every barrier gives up (for testing).
  * Discards captured graphs.  The paper has no counterpart (resource handling of this
  * implementation). */
 typedef enum {
