@@ -398,7 +398,7 @@ adress_status adress_list_stats(adress_handle h, int64_t* out);
 adress_status adress_time_kernels(adress_handle h, int32_t reps, float* ms_out);
 
 /* Launch configuration: threads per block of the mapping and force kernels (32, 64 or
- * 128; 4 threads per molecule) and the list skin (cells have edge >= max(rc_cg, rc_at +
+ * 128; the kernel that runs all steps of a small system keeps 128) and the list skin (cells have edge >= max(rc_cg, rc_at +
  * 2 r_ext) + skin, so the skin sets the cell size and how often lists are rebuilt).  The
  * results do not depend on either beyond the order of floating-point sums.  Setting them
  * discards captured graphs and the lists (build them again before stepping). */

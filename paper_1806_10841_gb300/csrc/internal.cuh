@@ -129,7 +129,7 @@ struct Sys {
   double rc_at, rc_cg;
   int ncell;  // cells of all boxes
   int cap;  // neighbour-list capacity per molecule
-  int force_block;  // threads per block of the mapping and force kernels
+  int force_block;  // threads per block of the mapping and force kernels (the run kernel: kMaxForceBlock)
   int n_sm;         // multiprocessors of the handle's device
   Lanes step_lanes, run_lanes;  // lanes per work item of the step and run kernels (FP32 path)
   int cg_mode;  // 0: tabulated F^CG, 1: learned network (pair forces in Bufs::fpair)

@@ -1730,13 +1730,15 @@ static void launch_step_na(const Sys& s, const Bufs& b, int mode, int energy, cu
   }
 }
 
-// As many blocks as fit on the device at once, at most one per tile.
+// As many blocks as fit on the device at once, at most one per tile.  Their size is fixed: at a force
+// kernel's 32 threads the four blocks an SM are four warps (us a step with 32 / 64 / 128 threads: 4000
+// molecules 17.4 / 13.6 / 10.3, 20,000 32.8 / 21.6 / 18.0, where launches at 32 took 28.1).
 template <class P, int NA, int MODEL, bool HS>
 static cudaError_t launch_run_na(const Sys& s, const Bufs& b, int done, int nsteps, int sample_every, cudaStream_t st) {
-  const int tiles = ceil_div((long long)s.M << (P::fp64 ? 2 : s.run_lanes.h), s.force_block);
+  const int tiles = ceil_div((long long)s.M << (P::fp64 ? 2 : s.run_lanes.h), kMaxForceBlock);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(tiles, s.n_sm * run_min_blocks<P>()));
-  cfg.blockDim = dim3(s.force_block);
+  cfg.blockDim = dim3(kMaxForceBlock);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
