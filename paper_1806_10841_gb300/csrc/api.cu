@@ -1175,7 +1175,7 @@ adress_status adress_rdf(adress_handle h, int32_t nbins, double dr, int64_t* cou
   const double range = nbins * dr;
   std::vector<RdfGrid> grids(s.nbox);
   long long ncell = 0;
-  double lmax = 0.0, fill = 0.0;  // fill: molecules a cell, in the box where they are most
+  double lmax = 0.0;
   for (int k = 0; k < s.nbox; ++k) {
     const Box& B = h->boxes[k];
     // (and the fixed-point centres' rounding wider, so that molecules two cells apart are out of range)
@@ -1187,17 +1187,24 @@ adress_status adress_rdf(adress_handle h, int32_t nbins, double dr, int64_t* cou
       lmax = std::max(lmax, B.L[d]);
     }
     G.cell0 = (int)ncell;
-    const long long nc = (long long)G.nc[0] * G.nc[1] * G.nc[2];
-    fill = std::max(fill, (double)B.nmol / nc);
-    ncell += nc;
+    ncell += (long long)G.nc[0] * G.nc[1] * G.nc[2];
   }
   // a warp per cell where there are cells for all warps (eight blocks of eight an SM) and they hold
   // at most a batch; else the cells are dealt out, in smaller batches while there are too few parts
   // (a batch of four costs as much for fetching its candidates as for testing them)
-  auto parts_of = [&](int batch) { return std::max(1, (int)ceil(fill / batch)); };
-  q.batch = 32;
-  while (q.batch > 4 && ncell * parts_of(q.batch) < 64ll * s.n_sm) q.batch /= 2;
-  q.parts = parts_of(q.batch);
+  long long ntask = 0;
+  for (q.batch = 32;; q.batch /= 2) {
+    ntask = 0;
+    for (int k = 0; k < s.nbox; ++k) {
+      RdfGrid& G = grids[k];
+      const int nc = G.nc[0] * G.nc[1] * G.nc[2];
+      G.parts = std::max(1, ceil_div(h->boxes[k].nmol, (long long)nc * q.batch));
+      G.task0 = (int)ntask;
+      ntask += (long long)nc * G.parts;
+    }
+    if (q.batch == 4 || ntask >= 64ll * s.n_sm) break;
+  }
+  q.ntask = (int)ntask;
   const size_t n = (size_t)s.nbox * nbins;
   if (h->rdf_cap < n) {
     CUDA_OR_FAIL(h, realloc_owned(h, &h->rdf_counts, n));

@@ -328,7 +328,8 @@ cudaError_t launch_max_nn(const Sys& s, const Bufs& b, cudaStream_t st);
 // (Bufs::netc, counted in Ctrl::n_netc, which the caller zeroes); a list build adds them
 // itself in CG mode 1.
 cudaError_t launch_net_candidates(const Sys& s, const Bufs& b, cudaStream_t st);
-// out[i] = sum_{j<i} in[j] for i < n, *total = sum of all (n <= 8M)
+// out[i] = sum_{j<i} in[j] for i < n, *total = sum of all (n <= kMaxScan)
+constexpr long long kMaxScan = 8388608;
 cudaError_t device_exclusive_scan(const int* in, int* out, int n, int* tmp, int* total, cudaStream_t st);
 // mode: 0 conservative forces, 1 last step of a run (thermostat + second half kick),
 // 2 fused step (thermostat + both half kicks + drift + next mapping)
@@ -347,6 +348,7 @@ cudaError_t launch_export_com(const Sys& s, const Bufs& b, int precision, double
 // COM pair-distance histogram (k_rdf): cell grids of the boxes, scratch and parameters.
 struct RdfGrid {
   int nc[3], cell0;
+  int parts, task0;  // warps a cell is dealt out to, first task (part of a cell) of the box
 };
 struct RdfArgs {
   const RdfGrid* grids;  // [nbox]
@@ -356,7 +358,7 @@ struct RdfArgs {
   int *count, *start;    // [ncell], [ncell + 1]
   unsigned long long* counts;  // [nbox][nbins], added to
   int ncell, nbins;
-  int batch, parts;  // a cell's molecules are dealt out to `parts` warps, `batch` at a time
+  int batch, ntask;  // molecules of a cell a warp takes at a time; tasks of all boxes
   double dr;
   float inv_dr, lim2, eps;  // 1 / dr, squared range with its margin, error of a distance in bins
 };

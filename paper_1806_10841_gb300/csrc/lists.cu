@@ -105,6 +105,7 @@ cudaError_t launch_net_candidates(const Sys& s, const Bufs& b, cudaStream_t st) 
 // tiles before its own (at most kScanMaxTiles of them) and scans its tile ----
 
 constexpr int kScanMaxTiles = 4096;
+static_assert((long long)kScanMaxTiles * kScanTile == kMaxScan, "largest scan");
 
 // Block-wide sum of v (every thread gets it).
 __device__ __forceinline__ int block_sum(int v) {

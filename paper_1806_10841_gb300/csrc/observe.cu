@@ -265,10 +265,12 @@ __global__ void k_rdf_fill(int M, const RdfArgs q) {
 // edge 2.5 / 1.6 / 0.10.
 constexpr int kRdfThreads = 256;
 
-// A block counts in 32 bits: a warp hands the counts on whenever it has tested this many pairs, so
-// that the eight warps of a block never hold more than eight times as many.  (Of 2^20 pairs each
-// costs a fraction of a percent.)
+// A block counts in 32 bits: after a batch a warp hands the counts on when it has tested this many
+// pairs since it last did.  A batch of 32 molecules has at most 2^28 (adress_init takes fewer than
+// 2^23 molecules), so the eight warps of a block never hold 2^32.  (Once in 2^20 pairs costs a
+// fraction of a percent.)
 constexpr unsigned kRdfHandOn = 1u << 20;
+static_assert(8ll * (32 * kMaxScan + kRdfHandOn) < 1ll << 32, "counts of a block");
 __device__ __noinline__ void hand_on_counts(unsigned* rh, unsigned long long* counts, int nbins) {
   for (int k = threadIdx.x & 31; k < nbins; k += 32) {
     const unsigned c = atomicExch(&rh[k], 0u);
@@ -279,31 +281,36 @@ __device__ __noinline__ void hand_on_counts(unsigned* rh, unsigned long long* co
 __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys s, const __grid_constant__ Bufs b, const RdfArgs q) {
   extern __shared__ unsigned rh[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ntask = q.ncell * q.parts, chunk = (ntask + gridDim.x - 1) / gridDim.x;
+  const int chunk = (q.ntask + gridDim.x - 1) / gridDim.x;
   int t0 = blockIdx.x * chunk;
-  const int t_end = min(ntask, t0 + chunk);
+  const int t_end = min(q.ntask, t0 + chunk);
   while (t0 < t_end) {
-    // the box of the run's first cell (boxes in cell order)
+    // the box of the run's first task (boxes in task order)
     int lo = 0, hi = s.nbox - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (q.grids[mid].cell0 <= t0 / q.parts) lo = mid;
+      if (q.grids[mid].task0 <= t0) lo = mid;
       else hi = mid - 1;
     }
     const RdfGrid G = q.grids[lo];
     const Box& B = s.nbox > 1 ? b.boxes[lo] : s.bx;
     const int nx = G.nc[0], ny = G.nc[1], nz = G.nc[2];
-    const int t1 = min(t_end, (G.cell0 + nx * ny * nz) * q.parts);
+    const int t1 = min(t_end, G.task0 + nx * ny * nz * G.parts);
     const bool half = nx >= 3 && ny >= 3 && nz >= 3;
     const float sx = B.fx_scale[0], sy = B.fx_scale[1], sz = B.fx_scale[2];
     unsigned tested = 0;
     for (int k = threadIdx.x; k < q.nbins; k += blockDim.x) rh[k] = 0u;
     __syncthreads();
     for (int t = t0 + warp; t < t1; t += kRdfThreads / 32) {
-      const int r = t / q.parts, e = t - r * q.parts, part = e & 1 ? q.parts - 1 - (e >> 1) : e >> 1;
-      const int hs = q.start[r], he = q.start[r + 1], first = hs + part * q.batch;
+      int l = t - G.task0, part = 0;
+      if (G.parts > 1) {
+        const int e = l % G.parts;
+        l /= G.parts;
+        part = e & 1 ? G.parts - 1 - (e >> 1) : e >> 1;
+      }
+      const int r = G.cell0 + l, hs = q.start[r], he = q.start[r + 1], first = hs + part * q.batch;
       if (first >= he) continue;
-      const int l = r - G.cell0, cx = l / (ny * nz), cy = (l / nz) % ny, cz = l % nz;
+      const int cx = l / (ny * nz), cy = (l / nz) % ny, cz = l % nz;
       // lane j < 27: neighbour cell (ox, oy, oz) = (j / 9 - 1, (j / 3) % 3 - 1, j % 3 - 1)
       int cnt = 0, start = 0;
       if (lane < 27 && (!half || lane >= 13)) {
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
         if (lane >= o) incl += v;
       }
       const int pre = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
-      for (int hb = first; hb < he; hb += q.parts * q.batch) {
+      for (int hb = first; hb < he; hb += G.parts * q.batch) {
         const int ht = min(he, hb + q.batch);
         for (int k0 = 0; k0 < total; k0 += 32) {
           // this lane's candidate: the cells whose inclusive prefix is <= k come before its own
@@ -368,11 +375,11 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const __grid_constant__ Sys
               if (bin < q.nbins) atomicAdd(&rh[bin], 1u);
             }
           }
-          tested += 32u * (unsigned)max(0, most - hb);
-          if (tested >= kRdfHandOn) {
-            hand_on_counts(rh, q.counts + (size_t)lo * q.nbins, q.nbins);
-            tested = 0;
-          }
+        }
+        tested += (unsigned)(ht - hb) * (unsigned)total;
+        if (tested >= kRdfHandOn) {
+          hand_on_counts(rh, q.counts + (size_t)lo * q.nbins, q.nbins);
+          tested = 0;
         }
       }
     }
@@ -433,7 +440,7 @@ cudaError_t launch_rdf(const Sys& s, const Bufs& b, const RdfArgs& q, cudaStream
   e = device_exclusive_scan(q.count, q.start, q.ncell, (int*)b.scan_tmp, q.start + q.ncell, st);
   if (e != cudaSuccess) return e;
   k_rdf_fill<<<ceil_div(s.M, 256), 256, 0, st>>>(s.M, q);
-  const int blocks = std::max(1, std::min(ceil_div((long long)q.ncell * q.parts, 2), 8 * s.n_sm));
+  const int blocks = std::max(1, std::min(ceil_div(q.ntask, 2), 8 * s.n_sm));
   k_rdf<<<blocks, kRdfThreads, sizeof(unsigned) * q.nbins, st>>>(s, b, q);
   return cudaGetLastError();
 }
